@@ -27,8 +27,7 @@ struct evp_handle {
     char *ws;
     size_t ws_bytes;
     // fields
-    void *sig, *sigk, *epse, *epst, *epsp, *deps, *rho, *tauc, *eta, *eta2, *spec, *Stab, *Mtab, *fac, *Sal, *lam, *pal;
-    float *Stabf, *Mtabf;
+    void *sig, *sigk, *epse, *epst, *epsp, *deps, *rho, *tauc, *eta, *eta2, *spec, *Stab, *Mtab, *Rtab, *fac, *Sal, *lam, *pal;
     double *k, *kappa, *partials, *scal;
     int32_t *g0, *g, *gprev, *draws, *ids, *ids2, *flags, *blk_counts, *blk_off, *count, *wlist;
     int nsm;
@@ -203,13 +202,12 @@ size_t layout(const evp_config *c, evp_handle *h, char *base) {
     char *epsp = take(6 * N3 * T), *deps = take(6 * N3 * T), *rho = take(12 * N3 * T), *tauc = take(N3 * T);
     char *eta = take(K * M3 * T), *eta2 = take(K * M3 * T), *spec = take(6 * H * 2 * T);
     char *Stab = take(36 * (size_t)G * T), *Mtab = take(72 * (size_t)G * T);
+    char *Rtab = take(T == 8 ? kFrameWords * (size_t)G * T : 0);
     // stored tangent factors: 21 words per voxel, in planes of 16-byte vectors and one scalar plane
     char *fac = take(c->newton_mode == EVP_NEWTON_REUSE ? 21 * N3 * T : 0);
     char *wlist = take(c->newton_mode == EVP_NEWTON_REUSE ? 4 * N3 : 0);      // voxels left for the second pass
     const bool al = c->scheme == EVP_SCHEME_AL;
-    char *Sal = take(al ? 36 * (size_t)G * T : 0), *lam = take(al ? 6 * N3 * T : 0), *pal = take(al ? 6 * N3 * T : 0);
-    const bool f32t = c->newton_mode == EVP_NEWTON_F32_TANGENT;
-    char *Stabf = take(f32t ? 36 * (size_t)G * 4 : 0), *Mtabf = take(f32t ? 72 * (size_t)G * 4 : 0);
+    char *Sal = take(al && T == 4 ? 36 * (size_t)G * T : 0), *lam = take(al ? 6 * N3 * T : 0), *pal = take(al ? 6 * N3 * T : 0);
     char *k = take(N3 * 8), *kappa = take(N3 * 8);
     char *g0 = take(N3 * 4), *g = take(N3 * 4), *gprev = take(N3 * 4), *draws = take(N3 * 4);
     char *ids = take(K * M3 * 4), *ids2 = take(K * M3 * 4);
@@ -233,11 +231,9 @@ size_t layout(const evp_config *c, evp_handle *h, char *base) {
         h->mr = mr ? 1 : 0;
         h->gs = gs; h->ge = ge; h->gnd = gnd; h->tpi = tpi; h->gdm = gdm; h->aux = aux; h->vec = vec;
         h->sig = sig; h->sigk = sigk; h->epse = epse; h->epst = epst; h->epsp = epsp; h->deps = deps;
-        h->rho = rho; h->tauc = tauc; h->eta = eta; h->eta2 = eta2; h->spec = spec; h->Stab = Stab; h->Mtab = Mtab;
+        h->rho = rho; h->tauc = tauc; h->eta = eta; h->eta2 = eta2; h->spec = spec; h->Stab = Stab; h->Mtab = Mtab; h->Rtab = Rtab;
         h->fac = fac;
         h->wlist = (int32_t *)wlist;
-        h->Stabf = (float *)Stabf;
-        h->Mtabf = (float *)Mtabf;
         h->Sal = Sal;
         h->lam = lam;
         h->pal = pal;
@@ -298,6 +294,23 @@ void mandel_rotation(const double R[3][3], double Q[6][6]) {
     }
 }
 
+// Rotation crystal -> sample of a quaternion (w, x, y, z).
+void rotation_of(const double *q, double R[3][3]) {
+    const double qn = std::sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+    const double w = q[0] / qn, x = q[1] / qn, y = q[2] / qn, z = q[3] / qn;
+    const double r[3][3] = {{1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)},
+                            {2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)},
+                            {2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)}};
+    for (int i = 0; i < 3; ++i)
+        for (int j = 0; j < 3; ++j) R[i][j] = r[i][j];
+}
+
+// Compliance of the crystal in its own axes.
+Cubic<double> cubic_of(const evp_params *p) {
+    const double den = (p->C11 - p->C12) * (p->C11 + 2.0 * p->C12);
+    return Cubic<double>{(p->C11 + 2.0 * p->C12) / den, -p->C12 / den, 1.0 / (2.0 * p->C44)};
+}
+
 template <typename T> void build_tables(const evp_params *p, int G, const double *quat, T *S, T *M) {
     const double den = (p->C11 - p->C12) * (p->C11 + 2.0 * p->C12);
     double Sc[6][6] = {};
@@ -317,12 +330,8 @@ template <typename T> void build_tables(const evp_params *p, int G, const double
             tensor_to_mandel(Tm, mc[3 * pl + d]);
         }
     for (int g = 0; g < G; ++g) {
-        const double *q = quat + 4 * g;
-        const double qn = std::sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-        const double w = q[0] / qn, x = q[1] / qn, y = q[2] / qn, z = q[3] / qn;
-        const double R[3][3] = {{1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)},
-                                {2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)},
-                                {2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)}};
+        double R[3][3];
+        rotation_of(quat + 4 * g, R);
         double Q[6][6];
         mandel_rotation(R, Q);
         double QS[6][6];
@@ -428,12 +437,8 @@ template <typename T> void mr_setup(evp_handle *h, const evp_params *p, const do
     // prefactor A = 2 k_B T nu_D sqrt(rho_P) exp(-Q_slip/k_B T) / (c1 c3 mu b^2) per unit tau_pass = tp_c sqrt(rho_P)
     h->mc.mr_ga = 2.0 * kT * p->nu_D * std::exp(-p->Q_slip / kT) / (p->c1 * p->c3 * muPa * b * b) / d.tp_c;
     for (int g = 0; g < h->G; ++g) {
-        const double *q = quat + 4 * g;
-        const double qn = std::sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-        const double w = q[0] / qn, x = q[1] / qn, y = q[2] / qn, z = q[3] / qn;
-        const double R[3][3] = {{1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y)},
-                                {2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x)},
-                                {2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)}};
+        double R[3][3];
+        rotation_of(quat + 4 * g, R);
         for (int a = 0; a < 12; ++a)
             for (int i = 0; i < 3; ++i) {
                 vec[72 * (size_t)g + 3 * a + i] = (T)(R[i][0] * dd[a][0] + R[i][1] * dd[a][1] + R[i][2] * dd[a][2]);
@@ -460,6 +465,20 @@ cudaError_t mr_soften_sel(evp_handle *h, int mode, int lo) {
                                  (double *)h->ge, (double *)h->gnd, h->k, h->mrc, h->st);
     return mr_soften<float>(h->N3, mode, h->gprev, h->g, lo, (const float *)h->rho, (float *)h->gs, (float *)h->ge,
                             (float *)h->gnd, h->k, h->mrc, h->st);
+}
+// Crystal data of the local problems; al_step: with the compliance S + S0 of the augmented-Lagrangian step, S0 that of
+// the isotropic medium (lam0, mu0).
+template <typename TA> LocalTab<TA> local_tab(const evp_handle *h, bool al_step = false, double lam0 = 0.0, double mu0 = 1.0) {
+    if constexpr (sizeof(TA) == 4) {
+        return LocalTab<float>{(const float *)(al_step ? h->Sal : h->Stab), (const float *)h->Mtab};
+    } else {
+        Cubic<double> c = cubic_of(&h->p);
+        if (al_step) {
+            const double sa = 1.0 / (2.0 * mu0), sb = lam0 / (2.0 * mu0 * (3.0 * lam0 + 2.0 * mu0));
+            c = Cubic<double>{c.d + sa, c.s12 - sb, c.s44 + sa};
+        }
+        return LocalTab<double>{c, (const double *)h->Rtab};
+    }
 }
 template <typename TA> MRPtr<TA> mr_ptr(const evp_handle *h) {
     return h->mr ? MRPtr<TA>{(const TA *)h->tpi} : MRPtr<TA>{nullptr};
@@ -533,7 +552,7 @@ int al_loop(evp_handle *h, MatConst mc, double *dE, int *it_out, int *conv_out, 
     auto local = [&](int init, int refresh) -> int {
         { PROF(0, 1);
           CK(al_local<TA>(N3, (const TA *)h->epst, (const TA *)h->epse, (const TA *)h->tauc, h->g0, (TA *)h->sigk,
-                          (TA *)h->lam, (TA *)h->pal, (const TA *)h->Stab, (const TA *)h->Sal, (const TA *)h->Mtab, mc,
+                          (TA *)h->lam, (TA *)h->pal, local_tab<TA>(h, !init, lam0, mu0), mc,
                           lam0, mu0, tol_loc, h->cfg.newton_max, solve64, init, h->flags, h->partials, fac,
                           refresh, h->st, h->nsm, mr_ptr<TA>(h))); }
         { PROF(6, 1); CK(reduce_partials(h->partials, nb, 14, h->scal + 24, h->st)); }
@@ -686,7 +705,7 @@ int evp_init(evp_handle **out, const evp_config *cfg, const evp_params *p, const
         if (!hS || !hM) { std::free(hS); std::free(hM); return fail(h, EVP_ERR_OOM, "host allocation"); }
         if (h->dbl) build_tables<double>(p, h->G, quat, (double *)hS, (double *)hM);
         else build_tables<float>(p, h->G, quat, (float *)hS, (float *)hM);
-        if (cfg->scheme == EVP_SCHEME_AL) {
+        if (cfg->scheme == EVP_SCHEME_AL && !h->dbl) {
             // S + S0 with S0 the compliance of the AL reference medium (Voigt bulk, shear mu/al_scale)
             void *hA = std::malloc(36 * G * h->tsz);
             if (!hA) { std::free(hS); std::free(hM); return fail(h, EVP_ERR_OOM, "host allocation"); }
@@ -696,8 +715,7 @@ int evp_init(evp_handle **out, const evp_config *cfg, const evp_params *p, const
                 for (int i = 0; i < 6; ++i)
                     for (int j = 0; j < 6; ++j) {
                         const double s0 = (i == j ? sa : 0.0) - (i < 3 && j < 3 ? sb : 0.0);
-                        if (h->dbl) ((double *)hA)[36 * gg + 6 * i + j] = ((double *)hS)[36 * gg + 6 * i + j] + s0;
-                        else ((float *)hA)[36 * gg + 6 * i + j] = (float)((double)((float *)hS)[36 * gg + 6 * i + j] + s0);
+                        ((float *)hA)[36 * gg + 6 * i + j] = (float)((double)((float *)hS)[36 * gg + 6 * i + j] + s0);
                     }
             cudaError_t ea = cudaMemcpyAsync(h->Sal, hA, 36 * G * h->tsz, cudaMemcpyHostToDevice, h->st);
             cudaError_t eb = cudaStreamSynchronize(h->st);
@@ -705,19 +723,20 @@ int evp_init(evp_handle **out, const evp_config *cfg, const evp_params *p, const
             CK(ea);
             CK(eb);
         }
-        if (cfg->newton_mode == EVP_NEWTON_F32_TANGENT) {
-            float *fS = (float *)std::malloc(36 * G * 4), *fM = (float *)std::malloc(72 * G * 4);
-            if (!fS || !fM) { std::free(fS); std::free(fM); std::free(hS); std::free(hM); return fail(h, EVP_ERR_OOM, "host allocation"); }
-            for (size_t i = 0; i < 36 * G; ++i) fS[i] = (float)((double *)hS)[i];
-            for (size_t i = 0; i < 72 * G; ++i) fM[i] = (float)((double *)hM)[i];
-            cudaError_t ea = cudaMemcpyAsync(h->Stabf, fS, 36 * G * 4, cudaMemcpyHostToDevice, h->st);
-            cudaError_t eb = cudaMemcpyAsync(h->Mtabf, fM, 72 * G * 4, cudaMemcpyHostToDevice, h->st);
-            cudaError_t ec = cudaStreamSynchronize(h->st);
-            std::free(fS);
-            std::free(fM);
+        if (h->dbl) {   // the FP64 local problems' crystal axes
+            double *hR = (double *)std::malloc(kFrameWords * G * sizeof(double));
+            if (!hR) { std::free(hS); std::free(hM); return fail(h, EVP_ERR_OOM, "host allocation"); }
+            for (size_t gg = 0; gg < G; ++gg) {
+                double R[3][3];
+                rotation_of(quat + 4 * gg, R);
+                for (int i = 0; i < kFrameWords; ++i) hR[kFrameWords * gg + i] = i < 9 ? R[i / 3][i % 3] : 0.0;
+            }
+            cudaError_t ea = cudaMemcpyAsync(h->Rtab, hR, kFrameWords * G * sizeof(double), cudaMemcpyHostToDevice, h->st);
+            cudaError_t eb = cudaStreamSynchronize(h->st);
+            std::free(hR);
+            if (ea != cudaSuccess || eb != cudaSuccess) { std::free(hS); std::free(hM); }
             CK(ea);
             CK(eb);
-            CK(ec);
         }
         cudaError_t e1 = cudaMemcpyAsync(h->Stab, hS, 36 * G * h->tsz, cudaMemcpyHostToDevice, h->st);
         cudaError_t e2 = cudaMemcpyAsync(h->Mtab, hM, 72 * G * h->tsz, cudaMemcpyHostToDevice, h->st);
@@ -902,16 +921,16 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
                   { PROF(0, 1);
                     if (h->cfg.newton_mode == EVP_NEWTON_F32_TANGENT)
                         CK(newton_field_df(N3, (double *)h->epst, (double *)h->tauc, h->g0, (double *)h->sigk,
-                                           (double *)h->Stab, (double *)h->Mtab, h->Stabf, h->Mtabf, mc, ntol,
+                                           local_tab<double>(h), mc, ntol,
                                            h->cfg.newton_max, h->flags, h->st, skip, tl64));
                     else if (reuse)
                         CK(newton_chord_field<double>(N3, (double *)h->epst, (double *)h->tauc, h->g0, (double *)h->sigk,
-                                                      (double *)h->Stab, (double *)h->Mtab, h->fac, mc, ntol,
+                                                      local_tab<double>(h), h->fac, mc, ntol,
                                                       h->cfg.newton_max, 1, first, h->flags, h->wlist, h->nsm, h->st,
                                                       skip, tl64, mr_ptr<double>(h), two));
                     else
                         CK(newton_field<double>(N3, (double *)h->epst, (double *)h->tauc, h->g0, (double *)h->sigk,
-                                                (double *)h->Stab, (double *)h->Mtab, mc, ntol, h->cfg.newton_max, 1,
+                                                local_tab<double>(h), mc, ntol, h->cfg.newton_max, 1,
                                                 h->flags, h->st, skip, tl64, mr_ptr<double>(h))); }
                   CK(fwd_xy<double>(h, (const double *)h->sigk, skip));
                   { PROF(3, 1);
@@ -921,12 +940,12 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
                   { PROF(0, 1);
                     if (reuse)
                         CK(newton_chord_field<float>(N3, (float *)h->epst, (float *)h->tauc, h->g0, (float *)h->sigk,
-                                                     (float *)h->Stab, (float *)h->Mtab, h->fac, mc, ntol,
+                                                     local_tab<float>(h), h->fac, mc, ntol,
                                                      h->cfg.newton_max, solve64, first, h->flags, h->wlist, h->nsm,
                                                      h->st, skip, tl32, mr_ptr<float>(h), two));
                     else
                         CK(newton_field<float>(N3, (float *)h->epst, (float *)h->tauc, h->g0, (float *)h->sigk,
-                                               (float *)h->Stab, (float *)h->Mtab, mc, ntol, h->cfg.newton_max, solve64,
+                                               local_tab<float>(h), mc, ntol, h->cfg.newton_max, solve64,
                                                h->flags, h->st, skip, tl32, mr_ptr<float>(h))); }
                   CK(fwd_xy<float>(h, (const float *)h->sigk, skip));
                   { PROF(3, 1);

@@ -6,6 +6,19 @@
 namespace evp {
 
 // ---- material / solver constants passed by value to the kernels ----
+// Compliance of a cubic crystal in its own axes, on a Mandel vector x: d x_i + s12 (x_0 + x_1 + x_2) for the normal
+// components, s44 x_i for the shears (d = S11 - S12, s44 the Mandel shear compliance 1 / (2 C44)).
+template <typename T> struct Cubic {
+    T d, s12, s44;
+    template <typename U> __host__ __device__ Cubic<U> as() const { return Cubic<U>{(U)d, (U)s12, (U)s44}; }
+};
+// Crystal data of the local problems (Sec. 2.1; frames in local.cuh). FP32: per-grain compliance (36 words) and
+// Schmid vectors (12 x 6 words) in the sample frame. FP64: the crystal's compliance and the per-grain rotations crystal ->
+// sample (kFrameWords words: 9, row-major, and padding).
+constexpr int kFrameWords = 10;
+template <typename TA> struct LocalTab;
+template <> struct LocalTab<float> { const float *S, *M; };
+template <> struct LocalTab<double> { Cubic<double> cub; const double *R; };
 struct MatConst {
     double gdot0, n, dt, tau0, alpha_mu_b, k1, k2;
     double lam0, mu0;       // reference medium (Voigt isotropic average)
@@ -70,8 +83,8 @@ cudaError_t fft_xy_c2r(const void *spec, T *out, int n, int nfields, T scale, co
 // solve_fp64: 1 -> the 6x6 Newton system is solved in FP64 even when TA = float.
 // mrp (optional): the Ma-Roters flow data; tauc then holds the stopping scale tau_ref = min_a tau_pass^a.
 template <typename TA>
-cudaError_t newton_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, const TA *Stab,
-                         const TA *Mtab, MatConst mc, double tol, int maxit, int solve_fp64, int *flags,
+cudaError_t newton_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, LocalTab<TA> tab,
+                         MatConst mc, double tol, int maxit, int solve_fp64, int *flags,
                          cudaStream_t s,
                          const int *skip = nullptr, const TA *tol_dev = nullptr, MRPtr<TA> mrp = MRPtr<TA>{});
 // Jacobian-reuse variant: fac holds 21 factor words per voxel in TA (factorised in FP64 if solve_fp64).
@@ -79,24 +92,23 @@ cudaError_t newton_field(long N3, const TA *epst, const TA *tauc, const int32_t 
 // nsm = multiprocessors, for the grid of the second pass. two_step: the first pass also takes the chord
 // iteration's next two moves where they stay on its common path (same results, fewer listed voxels).
 template <typename TA>
-cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, const TA *Stab,
-                               const TA *Mtab, void *fac, MatConst mc, double tol, int maxit, int solve_fp64,
+cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, LocalTab<TA> tab,
+                               void *fac, MatConst mc, double tol, int maxit, int solve_fp64,
                                int force_refresh, int *flags, int32_t *wl, int nsm, cudaStream_t s,
                                const int *skip = nullptr,
                                const TA *tol_dev = nullptr, MRPtr<TA> mrp = MRPtr<TA>{}, int two_step = 1);
-// FP64 residual / FP32 tangent Newton (FP64 path); Stabf / Mtabf are FP32 copies of the tables.
+// FP64 residual / FP32 tangent Newton (FP64 path).
 cudaError_t newton_field_df(long N3, const double *epst, const double *tauc, const int32_t *g0, double *sig,
-                            const double *Stab, const double *Mtab, const float *Stabf, const float *Mtabf,
-                            MatConst mc, double tol, int maxit, int *flags, cudaStream_t s,
+                            LocalTab<double> tab, MatConst mc, double tol, int maxit, int *flags, cudaStream_t s,
                             const int *skip = nullptr,
                             const double *tol_dev = nullptr);
-// Augmented-Lagrangian local step, grid-stride over al_grid(N3, nsm, sizeof(TA)) blocks; part: 14 doubles per
+// Augmented-Lagrangian local step (tab: the compliance S of the crystal with init, S + S0 without), grid-stride over al_grid(N3, nsm, sizeof(TA)) blocks; part: 14 doubles per
 // block. al_blocks(N3) bounds the block count (for sizing).
 int al_blocks(long N3);
 int al_grid(long N3, int nsm, int tsize);
 template <typename TA>
 cudaError_t al_local(long N3, const TA *epst, const TA *epse, const TA *tauc, const int32_t *g0, TA *sig, TA *lam, TA *p,
-                     const TA *Stab, const TA *Sal, const TA *Mtab, MatConst mc, double lam0, double mu0, double tol,
+                     LocalTab<TA> tab, MatConst mc, double lam0, double mu0, double tol,
                      int maxit, int solve_fp64, int init, int *flags, double *part, void *fac, int refresh,
                      cudaStream_t s, int nsm, MRPtr<TA> mrp = MRPtr<TA>{});
 template <typename TA>

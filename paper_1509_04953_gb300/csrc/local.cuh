@@ -91,6 +91,94 @@ template <typename TA> __device__ __forceinline__ void load_slip_pair(const TA *
     }
 }
 
+// ---- the crystal frame ----
+// The FP64 local problems are solved in the axes of their crystal: the FP64 pipe (2 multiply-adds per clock and SM)
+// bounds them, and there an evaluation takes about half the FP64 operations. The cubic compliance has three
+// constants (Cubic) and a Schmid vector of the {111}<110> systems has four entries, +-1/sqrt6 on two normal
+// components and +-1/sqrt12 on two shears (Mandel), so the 12 resolved stresses take 21 additions, the plastic strain
+// another 28 and the tangent 24 before its scaling, where the sample-frame Schmid vectors take 72, 72 and 252
+// multiply-adds. A solve adds three rotations of a symmetric tensor (51 operations each): trial strain and stress in,
+// stress out. k_newton_df at 64^3: 328 us per fixed-point iteration, 501 with the sample-frame vectors.
+// The FP32 problems stay in the sample frame: rotating the stress in FP32 adds a rounding of the stress itself, and
+// the equilibrium residual of the converged FP32 field rose from 5.0e-7 to 7.5e-7 of its tolerance's 1e-6.
+// The grain table holds kFrameWords words per grain: R (crystal -> sample, row-major) and 3 words of padding.
+template <typename T> __device__ __forceinline__ void load_frame(const T *__restrict__ R, T r[9]) {
+    if constexpr (sizeof(T) == 4) {
+        const float4 *R4 = reinterpret_cast<const float4 *>(R);
+        const float4 a = __ldg(R4), b = __ldg(R4 + 1);
+        r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
+        r[8] = __ldg(R + 8);
+    } else {
+        const double2 *R2 = reinterpret_cast<const double2 *>(R);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double2 t = __ldg(R2 + k);
+            r[2 * k] = t.x; r[2 * k + 1] = t.y;
+        }
+        r[8] = __ldg(R + 8);
+    }
+}
+// out = Mandel(A^T X A) with X the symmetric tensor of Mandel vector x and A given by its entries a(i, j).
+template <typename T, typename F> __device__ __forceinline__ void rotate_mandel(const T x[6], F a, T out[6]) {
+    const T h = (T)0.70710678118654752440, q2 = (T)1.41421356237309504880;
+    const T x23 = h * x[3], x13 = h * x[4], x12 = h * x[5];
+    T b[3][3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        b[0][j] = x[0] * a(0, j) + x12 * a(1, j) + x13 * a(2, j);
+        b[1][j] = x12 * a(0, j) + x[1] * a(1, j) + x23 * a(2, j);
+        b[2][j] = x13 * a(0, j) + x23 * a(1, j) + x[2] * a(2, j);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) out[i] = a(0, i) * b[0][i] + a(1, i) * b[1][i] + a(2, i) * b[2][i];
+    out[3] = q2 * (a(0, 1) * b[0][2] + a(1, 1) * b[1][2] + a(2, 1) * b[2][2]);
+    out[4] = q2 * (a(0, 0) * b[0][2] + a(1, 0) * b[1][2] + a(2, 0) * b[2][2]);
+    out[5] = q2 * (a(0, 0) * b[0][1] + a(1, 0) * b[1][1] + a(2, 0) * b[2][1]);
+}
+template <typename T> __device__ __forceinline__ void to_crystal(const T r[9], const T x[6], T out[6]) {
+    rotate_mandel(x, [&](int i, int j) { return r[3 * i + j]; }, out);
+}
+template <typename T> __device__ __forceinline__ void to_sample(const T r[9], const T x[6], T out[6]) {
+    rotate_mandel(x, [&](int i, int j) { return r[3 * j + i]; }, out);
+}
+
+// One voxel's local problem: what evaluate needs of the crystal besides the flow rule. enter() takes the trial strain
+// and the stress from the sample frame into the frame the problem is solved in, leave() takes the stress back.
+template <typename TA> struct Problem;
+template <> struct Problem<float> {   // sample frame: compliance (packed lower) and the grain's Schmid vectors
+    float Sp[21];
+    const float *M;
+    __device__ __forceinline__ void init(const LocalTab<float> &t, int g) {
+        load_compliance(t.S + 36 * (long)g, Sp);
+        M = t.M + 72 * (long)g;
+    }
+    __device__ __forceinline__ void enter(float *, float *) const {}
+    __device__ __forceinline__ void leave(float *) const {}
+};
+template <> struct Problem<double> {   // crystal frame
+    Cubic<double> cu;
+    const double *R;
+    __device__ __forceinline__ void init(const LocalTab<double> &t, int g) {
+        cu = t.cub;
+        R = t.R + kFrameWords * (long)g;
+    }
+    __device__ __forceinline__ void enter(double etr[6], double sg[6]) const {
+        double r[9], e[6], s[6];
+        load_frame(R, r);
+        to_crystal(r, etr, e);
+        to_crystal(r, sg, s);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) { etr[i] = e[i]; sg[i] = s[i]; }
+    }
+    __device__ __forceinline__ void leave(double sg[6]) const {
+        double r[9], s[6];
+        load_frame(R, r);
+        to_sample(r, sg, s);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) sg[i] = s[i];
+    }
+};
+
 // Stored tangent factors (21 words per voxel): 16-byte vector planes, then one scalar plane for the last word.
 // FP32: planes 0-4 are float4 (words 4k..4k+3), plane 5 is float (word 20); FP64: planes 0-9 are double2 (words
 // 2k, 2k+1), plane 10 is double (word 20). Each plane holds N3 voxels, so a voxel's factors come in 5 (10)
@@ -168,9 +256,10 @@ template <typename TS> __device__ __forceinline__ void prefetched_factors(const 
     F[20] = sh[P * nt * W + t];
 }
 
-template <typename TA> struct Eval {
+// Residual r, tangent K (packed lower, in TK) and potential phi of a local problem at a stress.
+template <typename TA, typename TK = TA> struct Eval {
     TA r[6];
-    TA K[21];
+    TK K[21];
     TA phi;
 };
 
@@ -454,6 +543,165 @@ __device__ __forceinline__ void evaluate_r(const TA Sp[21], const TA *__restrict
     e.phi = phi;
 }
 
+// ---- residual, tangent and potential of one local problem, in the crystal frame ----
+// The 12 systems in three families of four, by the pair of axes (i, j) of their slip directions e_i -+ e_j: with
+// D = s_ii - s_jj and the family's two shears A, B, the systems' n.sigma.d are D + u, D - u, D + w and D - w
+// (u = A - B, w = A + B) up to a sign, which neither flow rule depends on. kFamSys gives their numbers in the
+// order of the density fields.
+__host__ __device__ constexpr int fam_sys(int f, int q) {
+    return f == 0 ? (q == 0 ? 0 : q == 1 ? 3 : q == 2 ? 9 : 6)
+         : f == 1 ? (q == 0 ? 1 : q == 1 ? 7 : q == 2 ? 10 : 4)
+                  : (q == 0 ? 2 : q == 1 ? 11 : q == 2 ? 8 : 5);
+}
+// The family's resolved stresses from h = (11, 22, 33, 23, 13, 12), normals scaled by 1/sqrt6, Mandel shears by
+// 1/sqrt12: families (2, 3) with A = 12, B = 13; (1, 3) with A = 12, B = 23; (1, 2) with A = 13, B = 23.
+template <typename T> __device__ __forceinline__ void fam_stress(int f, const T h[6], T t[4]) {
+    const T D = f == 0 ? h[1] - h[2] : f == 1 ? h[0] - h[2] : h[0] - h[1];
+    const T A = f == 2 ? h[4] : h[5], B = f == 0 ? h[4] : h[3];
+    const T u = A - B, w = A + B;
+    t[0] = D + u; t[1] = D - u; t[2] = D + w; t[3] = D - w;
+}
+
+// Rates of one family. Power law: t = tau / tau_c, gam = |t|^n sign(t), slope = |t|^(n-1), pot += |t|^(n+1), to be
+// scaled by the caller. Ma-Roters: t = tau, gam, slope and pot as in Eq. FlowRule. WK: slopes wanted, in TK; tk holds
+// the resolved stresses in TK (for an FP32 tangent they are formed in FP32: six conversions instead of twelve).
+template <bool WK, bool WP, typename TK, typename TA>
+__device__ __forceinline__ void fam_rates(TA, int, const TA t[4], const TK tk[4], const MatConst &mc, TA gam[4],
+                                          TK slope[4], TA &pot) {
+    if (mc.n_int == 10) {
+        // the workloads' exponent: |t|^9 = |t| ((t^2)^2)^2, the very products pow_nm1's bit loop forms
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const TA b2 = t[q] * t[q], b4 = b2 * b2, b8 = b4 * b4, ax = fabs(t[q]);
+            if constexpr (WK && sizeof(TK) == sizeof(TA)) {
+                const TA p9 = ax * b8;
+                slope[q] = p9;
+                gam[q] = p9 * t[q];
+            } else {
+                if constexpr (WK) {   // FP32 tangent of the FP64 residual
+                    const TK x = fabs(tk[q]), c2 = x * x, c4 = c2 * c2;
+                    slope[q] = x * (c4 * c4);
+                }
+                gam[q] = copysign(b8 * b2, t[q]);
+            }
+            if constexpr (WP) pot += gam[q] * t[q];
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const TA p = pow_nm1(fabs(t[q]), mc);
+            if constexpr (WK) slope[q] = (TK)p;
+            gam[q] = p * t[q];
+            if constexpr (WP) pot += gam[q] * t[q];
+        }
+    }
+}
+template <bool WK, bool WP, typename TK, typename TA>
+__device__ __forceinline__ void fam_rates(const FlowMR<TA> &hf, int f, const TA t[4], const TK *, const MatConst &mc,
+                                          TA gam[4], TK slope[4], TA &pot) {
+    const TA ga = mr_ga<TA>(mc);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        TA tp, itc, sl, psi;
+        mr_sys(hf, fam_sys(f, q), tp, itc);
+        mr_flow(t[q], tp, itc, ga, gam[q], sl, psi);
+        if constexpr (WK) slope[q] = (TK)sl;
+        if constexpr (WP) pot += psi;
+    }
+}
+// Scales of the sums above: stress -> t (a), rates -> strain over the step (g), slopes -> tangent (k), pot (p).
+template <typename TA>
+__device__ __forceinline__ void flow_scales(TA tauc, TA inv_tc, const MatConst &mc, TA &a, TA &g, TA &k, TA &p) {
+    TA dt, g0, nn;
+    flow_consts(mc, dt, g0, nn);
+    a = inv_tc;
+    g = dt * g0;
+    k = g * nn * inv_tc;
+    p = g * tauc / (nn + (TA)1);
+}
+template <typename TA>
+__device__ __forceinline__ void flow_scales(const FlowMR<TA> &, TA, const MatConst &mc, TA &a, TA &g, TA &k, TA &p) {
+    TA dt, g0, nn;
+    flow_consts(mc, dt, g0, nn);
+    a = (TA)1;
+    g = k = p = dt;
+}
+
+// r = S sigma + dt sum m gdot(sigma) - eps_tr, with its tangent K (packed lower, in TK; WK) and the potential phi of
+// which it is the gradient (WP). All Mandel vectors in the crystal frame.
+template <bool WK, bool WP, typename TK, typename TA, typename H>
+__device__ __forceinline__ void evaluate_crystal(const Cubic<TA> &cu, const TA etr[6], const H &hf, TA inv_tc,
+                                                 const TA sg[6], const MatConst &mc, TA r[6], TK K[21], TA &phi) {
+    const TA q6 = (TA)0.40824829046386301637, q12 = (TA)0.28867513459481288225;   // 1/sqrt6, 1/sqrt12
+    TA sa, gs, ks, ps;
+    flow_scales(hf, inv_tc, mc, sa, gs, ks, ps);
+    const TA an = sa * q6, as = sa * q12;
+    TA h[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) h[i] = (i < 3 ? an : as) * sg[i];
+    TK hk[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) hk[i] = (TK)h[i];
+    TA gD[3], gA[3], gB[3], pot = (TA)0;
+    TK W[3], kA[3], kB[3], kX[3];
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+        TA t[4], g[4];
+        TK w[4], tk[4];
+        fam_stress(f, h, t);
+        fam_stress(f, hk, tk);
+        fam_rates<WK, WP, TK>(hf, f, t, tk, mc, g, w, pot);
+        const TA gu = g[0] - g[1], gw = g[2] - g[3];
+        gD[f] = (g[0] + g[1]) + (g[2] + g[3]);
+        gA[f] = gu + gw;
+        gB[f] = gw - gu;
+        if constexpr (WK) {   // sum of w t t^T on (D, A, B): DD = AA = BB = W, DA, DB, AB
+            const TK p = w[0] + w[1], q = w[2] + w[3], m = w[0] - w[1], n = w[2] - w[3];
+            W[f] = p + q;
+            kA[f] = m + n;
+            kB[f] = n - m;
+            kX[f] = q - p;
+        }
+    }
+    const TA fn = gs * q6, fs = gs * q12, st = cu.s12 * (sg[0] + sg[1] + sg[2]);
+    const TA ep[6] = {fn * (gD[1] + gD[2]), fn * (gD[0] - gD[2]), -fn * (gD[0] + gD[1]),
+                      fs * (gB[1] + gB[2]), fs * (gB[0] + gA[2]), fs * (gA[0] + gA[1])};
+    TA el = (TA)0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const TA acc = i < 3 ? cu.d * sg[i] + st : cu.s44 * sg[i];
+        r[i] = (acc - etr[i]) + ep[i];
+        if constexpr (WP) el += sg[i] * ((TA)0.5 * acc - etr[i]);
+    }
+    if constexpr (WP) phi = el + ps * pot;
+    if constexpr (WK) {
+        const TK ksk = (TK)ks, kn = ksk * (TK)(1.0 / 6.0), kx = ksk * (TK)0.11785113019775792073, kt = ksk * (TK)(1.0 / 12.0);
+        const Cubic<TK> ck = cu.template as<TK>();
+        const TK s11 = ck.d + ck.s12;
+        K[pk(0, 0)] = s11 + kn * (W[1] + W[2]);
+        K[pk(1, 0)] = ck.s12 - kn * W[2];
+        K[pk(1, 1)] = s11 + kn * (W[0] + W[2]);
+        K[pk(2, 0)] = ck.s12 - kn * W[1];
+        K[pk(2, 1)] = ck.s12 - kn * W[0];
+        K[pk(2, 2)] = s11 + kn * (W[0] + W[1]);
+        K[pk(3, 0)] = kx * (kB[1] + kB[2]);
+        K[pk(3, 1)] = -kx * kB[2];
+        K[pk(3, 2)] = -kx * kB[1];
+        K[pk(3, 3)] = ck.s44 + kt * (W[1] + W[2]);
+        K[pk(4, 0)] = kx * kA[2];
+        K[pk(4, 1)] = kx * (kB[0] - kA[2]);
+        K[pk(4, 2)] = -kx * kB[0];
+        K[pk(4, 3)] = kt * kX[2];
+        K[pk(4, 4)] = ck.s44 + kt * (W[0] + W[2]);
+        K[pk(5, 0)] = kx * kA[1];
+        K[pk(5, 1)] = kx * kA[0];
+        K[pk(5, 2)] = -kx * (kA[0] + kA[1]);
+        K[pk(5, 3)] = kt * kX[1];
+        K[pk(5, 4)] = kt * kX[0];
+        K[pk(5, 5)] = ck.s44 + kt * (W[0] + W[1]);
+    }
+}
+
 // LDL^T factorisation kept for reuse: F[0..14] = strict lower L (row-major by packed index, diagonal
 // slots skipped), F[15..20] = 1/D. Returns false if a pivot is not positive.
 template <typename TS, typename TA> __device__ __forceinline__ bool ldl_factor(const TA Kin[21], TS F[21]) {
@@ -510,62 +758,27 @@ template <typename TS, typename TA> __device__ __forceinline__ void ldl_apply(co
     for (int i = 0; i < 6; ++i) dout[i] = (TA)y[i];
 }
 
-// FP64 residual and potential with the tangent assembled in FP32 (the tangent only steers the
-// iteration; the converged stress is fixed by the FP64 residual). Sf / Mf are FP32 copies of the
-// per-grain compliance and Schmid tables.
-struct EvalDF {
-    double r[6];
-    float K[21];
-    double phi;
-};
-__device__ __forceinline__ void evaluate_df(const double Sp[21], const double *__restrict__ M, const float Spf[21],
-                                            const float *__restrict__ Mf, const double etr[6], double tauc,
-                                            double inv_tc, const double sg[6], const MatConst &mc, EvalDF &e) {
-    const double dt = mc.dt, g0 = mc.gdot0, nn = mc.n;
-    double phi = 0.0;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        double acc = 0.0;
-#pragma unroll
-        for (int j = 0; j < 6; ++j) acc += Sp[i >= j ? pk(i, j) : pk(j, i)] * sg[j];
-        e.r[i] = acc - etr[i];
-        phi += sg[i] * (0.5 * acc - etr[i]);
-    }
-#pragma unroll
-    for (int q = 0; q < 21; ++q) e.K[q] = Spf[q];
-    const double cphi = dt * g0 * tauc / (nn + 1.0);
-    const float cslope = (float)(dt * nn * g0 * inv_tc);
-#pragma unroll 1
-    for (int p = 0; p < 6; ++p) {
-      double mm[12];
-      float mmf[12];
-      load_slip_pair(M, p, mm);
-      load_slip_pair(Mf, p, mmf);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const double *m = mm + 6 * h;
-        const float *mf = mmf + 6 * h;
-        double tau = 0.0;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) tau += m[i] * sg[i];
-        const double x = tau * inv_tc, ax = fabs(x);
-        const double p9 = pow_nm1(ax, mc);
-        const double p10 = p9 * ax;
-        const double dg = x < 0.0 ? -dt * g0 * p10 : dt * g0 * p10;
-#pragma unroll
-        for (int i = 0; i < 6; ++i) e.r[i] += dg * m[i];
-        phi += cphi * p10 * ax;
-        const float slope = cslope * (float)p9;
-        float sm[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) sm[i] = slope * mf[i];
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-#pragma unroll
-            for (int j = 0; j <= i; ++j) e.K[pk(i, j)] += sm[i] * mf[j];
-      }
-    }
-    e.phi = phi;
+// The forms the solvers call: with the tangent (FP64 residuals may take it in FP32), or without it (the cost of a
+// chord step); UNROLL as in evaluate_r.
+template <typename TK, typename H>
+__device__ __forceinline__ void evaluate(const Problem<double> &p, const double etr[6], const H &hf, double inv_tc,
+                                         const double sg[6], const MatConst &mc, Eval<double, TK> &e) {
+    evaluate_crystal<true, true, TK>(p.cu, etr, hf, inv_tc, sg, mc, e.r, e.K, e.phi);
+}
+template <typename H>
+__device__ __forceinline__ void evaluate(const Problem<float> &p, const float etr[6], const H &hf, float inv_tc,
+                                         const float sg[6], const MatConst &mc, Eval<float> &e) {
+    evaluate(p.Sp, p.M, etr, hf, inv_tc, sg, mc, e);
+}
+template <int UNROLL = 1, typename H>
+__device__ __forceinline__ void evaluate_r(const Problem<double> &p, const double etr[6], const H &hf, double inv_tc,
+                                           const double sg[6], const MatConst &mc, EvalR<double> &e) {
+    evaluate_crystal<false, true, double>(p.cu, etr, hf, inv_tc, sg, mc, e.r, nullptr, e.phi);
+}
+template <int UNROLL = 1, typename H>
+__device__ __forceinline__ void evaluate_r(const Problem<float> &p, const float etr[6], const H &hf, float inv_tc,
+                                           const float sg[6], const MatConst &mc, EvalR<float> &e) {
+    evaluate_r<float, UNROLL>(p.Sp, p.M, etr, hf, inv_tc, sg, mc, e);
 }
 
 }  // namespace evp

@@ -58,12 +58,12 @@ __device__ __forceinline__ void block_solve_stats(int fail, int maxit, int it, i
 // Damped Newton on one voxel. Returns the iteration count (> 0) or minus it on failure.
 // H: the power law's tau_c (TA) or the Ma-Roters flow data (FlowMR<TA>, Sec. 2.2).
 template <typename TA, typename TS, typename H>
-__device__ int newton_voxel(const TA Sp[21], const TA *__restrict__ M, const TA etr[6], const H &hf, TA sg[6],
+__device__ int newton_voxel(const Problem<TA> &pb, const TA etr[6], const H &hf, TA sg[6],
                             const MatConst &mc, TA tol, int maxit, TA ls_free, int &nevals) {
     const TA tauc = flow_ref(hf);
     const TA inv_tc = drcp(tauc);
     Eval<TA> e;
-    evaluate(Sp, M, etr, hf, inv_tc, sg, mc, e);
+    evaluate(pb, etr, hf, inv_tc, sg, mc, e);
     nevals = 1;
     for (int it = 1; it <= maxit; ++it) {
         TA d[6];
@@ -90,7 +90,7 @@ __device__ int newton_voxel(const TA Sp[21], const TA *__restrict__ M, const TA 
         for (int h = 0; h < 60; ++h) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) st[i] = sg[i] - s * d[i];
-            evaluate(Sp, M, etr, hf, inv_tc, st, mc, e);
+            evaluate(pb, etr, hf, inv_tc, st, mc, e);
             ++nevals;
             if (e.phi <= phi0 - (TA)1e-4 * s * rd || s * dn <= ls_free * scale) {
                 ok = true;
@@ -109,7 +109,7 @@ __device__ int newton_voxel(const TA Sp[21], const TA *__restrict__ M, const TA 
 template <typename TA, typename TS, bool MR = false>
 __global__ void __launch_bounds__(kThreads) k_newton(long N3, const TA *__restrict__ epst, const TA *__restrict__ tauc,
                                                     const int32_t *__restrict__ g0, TA *__restrict__ sig,
-                                                    const TA *__restrict__ Stab, const TA *__restrict__ Mtab, MatConst mc,
+                                                    LocalTab<TA> tab, MatConst mc,
                                                     TA tol, int maxit, TA ls_free, int *__restrict__ flags, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
     pdl_wait();
@@ -120,20 +120,21 @@ __global__ void __launch_bounds__(kThreads) k_newton(long N3, const TA *__restri
     const bool valid = v < N3;
     int r = 1, nev = 0;
     if (valid) {
-        const int g = g0[v];
-        TA Sp[21];
-        load_compliance(Stab + 36 * (long)g, Sp);
+        Problem<TA> pb;
+        pb.init(tab, g0[v]);
         TA etr[6], sg[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             etr[c] = epst[c * N3 + v];
             sg[c] = sig[c * N3 + v];
         }
+        pb.enter(etr, sg);
         if constexpr (MR)
-            r = newton_voxel<TA, TS>(Sp, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]}, sg, mc,
+            r = newton_voxel<TA, TS>(pb, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]}, sg, mc,
                                      tol, maxit, ls_free, nev);
         else
-            r = newton_voxel<TA, TS>(Sp, Mtab + 72 * (long)g, etr, tauc[v], sg, mc, tol, maxit, ls_free, nev);
+            r = newton_voxel<TA, TS>(pb, etr, tauc[v], sg, mc, tol, maxit, ls_free, nev);
+        pb.leave(sg);
 #pragma unroll
         for (int c = 0; c < 6; ++c) sig[c * N3 + v] = sg[c];
     }
@@ -145,28 +146,41 @@ __global__ void __launch_bounds__(kThreads) k_newton(long N3, const TA *__restri
 // slightly inexact Newton step (relative tangent error ~1e-7), so the iteration contracts at least
 // ~1e-6 per step near the solution and stops on the same step-size test; Armijo backtracking on
 // the FP64 potential keeps it globally convergent.
-__device__ int newton_voxel_df(const double Sp[21], const double *__restrict__ M, const float Spf[21],
-                               const float *__restrict__ Mf, const double etr[6], double tauc, double sg[6],
+__device__ int newton_voxel_df(const Problem<double> &pb, const double etr[6], double tauc, double sg[6],
                                const MatConst &mc, double tol, int maxit, double ls_free, int &nevals) {
     const double inv_tc = drcp(tauc);
-    EvalDF e;
-    evaluate_df(Sp, M, Spf, Mf, etr, tauc, inv_tc, sg, mc, e);
+    Eval<double, float> e;
+    evaluate(pb, etr, tauc, inv_tc, sg, mc, e);
     nevals = 1;
     for (int it = 1; it <= maxit; ++it) {
         float rf[6], df[6];
 #pragma unroll
         for (int i = 0; i < 6; ++i) rf[i] = (float)e.r[i];
         if (!ldl_solve<float, float>(e.K, rf, df)) return -it;
-        double d[6], rd = 0.0, dn = 0.0, sn = 0.0;
+        double d[6], rd = 0.0, sn = 0.0;
+        float dn2 = 0.f;
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
             d[i] = (double)df[i];
             rd += e.r[i] * d[i];
-            dn += d[i] * d[i];
+            dn2 += df[i] * df[i];
             sn += sg[i] * sg[i];
         }
-        dn = dsqrt(dn);
-        const double scale = dsqrt(sn) + tauc;
+        // the two norms steer the stopping and line-search tests only: their roots in FP32 (the step is an FP32 vector),
+        // in FP64 where a square leaves the range of FP32
+        const float snf = (float)sn;
+        const bool in_range = dn2 > 1e-30f && dn2 < 1e30f && snf < 1e30f;
+        double dn, scale;
+        if (in_range) {
+            dn = (double)sqrtf(dn2);
+            scale = (double)sqrtf(snf) + tauc;
+        } else {
+            dn = 0.0;
+#pragma unroll
+            for (int i = 0; i < 6; ++i) dn += d[i] * d[i];
+            dn = dsqrt(dn);
+            scale = dsqrt(sn) + tauc;
+        }
         if (dn <= tol * scale && rd >= 0.0) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) sg[i] -= d[i];
@@ -178,7 +192,7 @@ __device__ int newton_voxel_df(const double Sp[21], const double *__restrict__ M
         for (int h = 0; h < 60; ++h) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) st[i] = sg[i] - s * d[i];
-            evaluate_df(Sp, M, Spf, Mf, etr, tauc, inv_tc, st, mc, e);
+            evaluate(pb, etr, tauc, inv_tc, st, mc, e);
             ++nevals;
             if (e.phi <= phi0 - 1e-4 * s * rd || s * dn <= ls_free * scale) {
                 ok = true;
@@ -196,9 +210,8 @@ __device__ int newton_voxel_df(const double Sp[21], const double *__restrict__ M
 
 __global__ void __launch_bounds__(kThreads) k_newton_df(long N3, const double *__restrict__ epst,
                                                        const double *__restrict__ tauc, const int32_t *__restrict__ g0,
-                                                       double *__restrict__ sig, const double *__restrict__ Stab,
-                                                       const double *__restrict__ Mtab, const float *__restrict__ Stabf,
-                                                       const float *__restrict__ Mtabf, MatConst mc, double tol,
+                                                       double *__restrict__ sig, LocalTab<double> tab,
+                                                       MatConst mc, double tol,
                                                        int maxit, int *__restrict__ flags, const int *__restrict__ skip,
     const double *__restrict__ tol_dev) {
     pdl_wait();
@@ -209,19 +222,17 @@ __global__ void __launch_bounds__(kThreads) k_newton_df(long N3, const double *_
     const bool valid = v < N3;
     int r = 1, nev = 0;
     if (valid) {
-        const int g = g0[v];
-        double Sp[21];
-        float Spf[21];
-        load_compliance(Stab + 36 * (long)g, Sp);
-        load_compliance(Stabf + 36 * (long)g, Spf);
+        Problem<double> pb;
+        pb.init(tab, g0[v]);
         double etr[6], sg[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             etr[c] = epst[c * N3 + v];
             sg[c] = sig[c * N3 + v];
         }
-        r = newton_voxel_df(Sp, Mtab + 72 * (long)g, Spf, Mtabf + 72 * (long)g, etr, tauc[v], sg, mc, tol, maxit,
-                            1e-6, nev);
+        pb.enter(etr, sg);
+        r = newton_voxel_df(pb, etr, tauc[v], sg, mc, tol, maxit, 1e-6, nev);
+        pb.leave(sg);
 #pragma unroll
         for (int c = 0; c < 6; ++c) sig[c * N3 + v] = sg[c];
     }
@@ -242,13 +253,13 @@ __global__ void __launch_bounds__(kThreads) k_newton_df(long N3, const double *_
 // FP32 afterwards are a componentwise perturbation and keep the Newton direction within about 1e-4
 // relative even there, so the reused step runs on the FP32 pipe and reads half the bytes.
 template <typename TA, typename TS, typename TF, typename H>
-__device__ int chord_voxel(const TA Sp[21], const TA *__restrict__ M, const TA etr[6], const H &hf, TA sg[6],
+__device__ int chord_voxel(const Problem<TA> &pb, const TA etr[6], const H &hf, TA sg[6],
                            const MatConst &mc, TA tol, int maxit, TA ls_free, TS F[21], bool refresh, int &nevals,
                            int &nref) {
     const TA tauc = flow_ref(hf);
     const TA inv_tc = drcp(tauc);
     EvalR<TA> e;
-    evaluate_r(Sp, M, etr, hf, inv_tc, sg, mc, e);
+    evaluate_r(pb, etr, hf, inv_tc, sg, mc, e);
     nevals = 1;
     nref = 0;
     TA prev_step = (TA)-1;
@@ -256,7 +267,7 @@ __device__ int chord_voxel(const TA Sp[21], const TA *__restrict__ M, const TA e
     for (int it = 1; it <= maxit; ++it) {
         if (refresh) {
             Eval<TA> full;
-            evaluate(Sp, M, etr, hf, inv_tc, sg, mc, full);
+            evaluate(pb, etr, hf, inv_tc, sg, mc, full);
             ++nevals;
             TF Ff[21];
             if (!ldl_factor<TF, TA>(full.K, Ff)) return -it;
@@ -292,7 +303,7 @@ __device__ int chord_voxel(const TA Sp[21], const TA *__restrict__ M, const TA e
         for (int h = 0; h < 60; ++h) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) st[i] = sg[i] - s * d[i];
-            evaluate_r(Sp, M, etr, hf, inv_tc, st, mc, e);
+            evaluate_r(pb, etr, hf, inv_tc, st, mc, e);
             ++nevals;
             if (e.phi <= phi0 - (TA)1e-4 * s * rd || s * dn <= ls_free * scale) {
                 ok = true;
@@ -314,7 +325,7 @@ __device__ int chord_voxel(const TA Sp[21], const TA *__restrict__ M, const TA e
 template <typename TA, typename TS, typename TF, bool MR = false>
 __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_newton_chord(long N3, const TA *__restrict__ epst, const TA *__restrict__ tauc,
                                                           const int32_t *__restrict__ g0, TA *__restrict__ sig,
-                                                          const TA *__restrict__ Stab, const TA *__restrict__ Mtab,
+                                                          LocalTab<TA> tab,
                                                           TS *__restrict__ fac, MatConst mc, TA tol, int maxit,
                                                           TA ls_free, int force_refresh, int *__restrict__ flags, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
@@ -326,25 +337,26 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_newton_ch
     const bool valid = v < N3;
     int r = 1, nev = 0, nref = 0;
     if (valid) {
-        const int g = g0[v];
-        TA Sp[21];
-        load_compliance(Stab + 36 * (long)g, Sp);
+        Problem<TA> pb;
+        pb.init(tab, g0[v]);
         TA etr[6], sg[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             etr[c] = epst[c * N3 + v];
             sg[c] = sig[c * N3 + v];
         }
+        pb.enter(etr, sg);
         TS F[21];
         if (!force_refresh) {
             load_factors(fac, N3, v, F);
         }
         if constexpr (MR)
-            r = chord_voxel<TA, TS, TF>(Sp, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]}, sg,
+            r = chord_voxel<TA, TS, TF>(pb, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]}, sg,
                                         mc, tol, maxit, ls_free, F, force_refresh != 0, nev, nref);
         else
-            r = chord_voxel<TA, TS, TF>(Sp, Mtab + 72 * (long)g, etr, tauc[v], sg, mc, tol, maxit, ls_free, F,
+            r = chord_voxel<TA, TS, TF>(pb, etr, tauc[v], sg, mc, tol, maxit, ls_free, F,
                                         force_refresh != 0, nev, nref);
+        pb.leave(sg);
 #pragma unroll
         for (int c = 0; c < 6; ++c) sig[c * N3 + v] = sg[c];
         if (nref) {
@@ -366,8 +378,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_newton_ch
 template <typename TA, typename TS, bool MR = false, bool TWO = true>
 __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1) k_chord_first(long N3, const TA *__restrict__ epst,
                                                          const TA *__restrict__ tauc, const int32_t *__restrict__ g0,
-                                                         TA *__restrict__ sig, const TA *__restrict__ Stab,
-                                                         const TA *__restrict__ Mtab, const TS *__restrict__ fac,
+                                                         TA *__restrict__ sig, LocalTab<TA> tab,
+                                                         const TS *__restrict__ fac,
                                                          MatConst mc, TA tol, TA ls_free, int *__restrict__ flags,
                                                          int32_t *__restrict__ wl, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
@@ -384,8 +396,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
     if (valid) prefetch_factors(fac, N3, v, fsh);
     if (valid) {
         const int g = g0[v];
-        TA Sp[21];
-        load_compliance(Stab + 36 * (long)g, Sp);
+        Problem<TA> pb;
+        pb.init(tab, g);
         TA etr[6], sg[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
@@ -393,11 +405,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
             sg[c] = sig[c * N3 + v];
         }
         const TA tc = tauc[v];
+        pb.enter(etr, sg);
         EvalR<TA> e;
         if constexpr (MR)
-            evaluate_r<TA, 6>(Sp, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tc}, (TA)0, sg, mc, e);
+            evaluate_r<6>(pb, etr, FlowMR<TA>{mrp.tpi, N3, v, tc}, (TA)0, sg, mc, e);
         else
-            evaluate_r<TA, 6>(Sp, Mtab + 72 * (long)g, etr, tc, drcp(tc), sg, mc, e);
+            evaluate_r<6>(pb, etr, tc, drcp(tc), sg, mc, e);
         TS F[21];
         prefetched_factors(fsh, F);
         TA d[6];
@@ -412,8 +425,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
         dn = dsqrt(dn);
         const TA scale = dsqrt(sn) + tc;
         if (dn <= tol * scale && rd >= (TA)0) {   // the acceptance test of chord_voxel
+            TA sn6[6];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) sig[c * N3 + v] = sg[c] - d[c];
+            for (int c = 0; c < 6; ++c) sn6[c] = sg[c] - d[c];
+            pb.leave(sn6);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) sig[c * N3 + v] = sn6[c];
             done = true;
         } else if (TWO && rd > (TA)0) {
             // chord_voxel's next moves while they stay on its common path, with its operations in its order: the
@@ -427,12 +444,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
 #pragma unroll
             for (int i = 0; i < 6; ++i) st[i] = sg[i] - s1 * d[i];
             asm volatile("" ::: "memory");
-            TA Sp2[21];
-            load_compliance(Stab + 36 * (long)g, Sp2);
+            Problem<TA> pb2;
+            pb2.init(tab, g);
             if constexpr (MR)
-                evaluate_r<TA>(Sp2, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tc}, (TA)0, st, mc, e);
+                evaluate_r(pb2, etr, FlowMR<TA>{mrp.tpi, N3, v, tc}, (TA)0, st, mc, e);
             else
-                evaluate_r<TA>(Sp2, Mtab + 72 * (long)g, etr, tc, drcp(tc), st, mc, e);
+                evaluate_r(pb2, etr, tc, drcp(tc), st, mc, e);
             if (e.phi <= phi0 - (TA)1e-4 * s1 * rd || s1 * dn <= ls_free * scale) {
                 prefetched_factors(fsh, F);
                 ldl_apply<TS, TA>(F, e.r, d);
@@ -446,7 +463,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
                 dn2 = dsqrt(dn2);
                 if (dn2 <= tol * (dsqrt(sn2) + tc) && rd2 >= (TA)0) {
 #pragma unroll
-                    for (int c = 0; c < 6; ++c) sig[c * N3 + v] = st[c] - d[c];
+                    for (int c = 0; c < 6; ++c) st[c] -= d[c];
+                    pb2.leave(st);
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) sig[c * N3 + v] = st[c];
                     done = true;
                     two = true;
                 }
@@ -468,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
 template <typename TA, typename TS, typename TF, bool MR = false>
 __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_chord_rest(
     long N3, const TA *__restrict__ epst, const TA *__restrict__ tauc, const int32_t *__restrict__ g0,
-    TA *__restrict__ sig, const TA *__restrict__ Stab, const TA *__restrict__ Mtab, TS *__restrict__ fac, MatConst mc,
+    TA *__restrict__ sig, LocalTab<TA> tab, TS *__restrict__ fac, MatConst mc,
     TA tol, int maxit, TA ls_free, int *__restrict__ flags, const int32_t *__restrict__ wl, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
     pdl_wait();
@@ -490,23 +510,24 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_chord_res
         int r = 1, nev = 0, nref = 0;
         if (valid) {
             const long v = wl[w];
-            const int g = g0[v];
-            TA Sp[21];
-            load_compliance(Stab + 36 * (long)g, Sp);
+            Problem<TA> pb;
+            pb.init(tab, g0[v]);
             TA etr[6], sg[6];
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 etr[c] = epst[c * N3 + v];
                 sg[c] = sig[c * N3 + v];
             }
+            pb.enter(etr, sg);
             TS F[21];
             load_factors(fac, N3, v, F);
             if constexpr (MR)
-                r = chord_voxel<TA, TS, TF>(Sp, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]},
+                r = chord_voxel<TA, TS, TF>(pb, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]},
                                             sg, mc, tol, maxit, ls_free, F, false, nev, nref);
             else
-                r = chord_voxel<TA, TS, TF>(Sp, Mtab + 72 * (long)g, etr, tauc[v], sg, mc, tol, maxit, ls_free, F, false,
+                r = chord_voxel<TA, TS, TF>(pb, etr, tauc[v], sg, mc, tol, maxit, ls_free, F, false,
                                             nev, nref);
+            pb.leave(sg);
 #pragma unroll
             for (int c = 0; c < 6; ++c) sig[c * N3 + v] = sg[c];
             if (nref) {
@@ -592,8 +613,7 @@ template <typename TA, typename TS, typename TF, bool MR = false>
 __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(long N3, const TA *__restrict__ epst, const TA *__restrict__ epse,
                                                       const TA *__restrict__ tauc, const int32_t *__restrict__ g0,
                                                       TA *__restrict__ sig, TA *__restrict__ lam, TA *__restrict__ pout,
-                                                      const TA *__restrict__ Stab, const TA *__restrict__ Sal,
-                                                      const TA *__restrict__ Mtab, MatConst mc, TA l0, TA m0, TA sa,
+                                                      LocalTab<TA> tab, MatConst mc, TA l0, TA m0, TA sa,
                                                       TA sb, TA sa_lo, TA sb_lo, double sad, double sbd, TA tol,
                                                       int maxit, TA ls_free, int init,
                                                       int *__restrict__ flags, double *__restrict__ part,
@@ -615,9 +635,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
 #pragma unroll
     for (int q = 0; q < NV; ++q) sums[q] = (TA)0;
     if (valid) {
-        const int g = g0[v];
-        TA Sp[21];
-        load_compliance((init ? Stab : Sal) + 36 * (long)g, Sp);
+        Problem<TA> pb;
+        pb.init(tab, g0[v]);
         // isotropic S0 = C0^-1 = sa I - sb J (Mandel), sa = 1/(2 m0), sb = l0 / (2 m0 (3 l0 + 2 m0))
         TA et[6], lm[6], ee[6], etr[6], sg[6];
 #pragma unroll
@@ -630,6 +649,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
         const TA ltr = lm[0] + lm[1] + lm[2];
 #pragma unroll
         for (int c = 0; c < 6; ++c) etr[c] = et[c] + sa * lm[c] - (c < 3 ? sb * ltr : (TA)0);
+        TA el6[6];   // the trial strain in the frame the problem is solved in
+#pragma unroll
+        for (int c = 0; c < 6; ++c) el6[c] = etr[c];
+        pb.enter(el6, sg);
         if (fac) {   // tangent reuse: factors refreshed on request or when a step stalls
             TS F[21];
             if (!refresh) {
@@ -637,21 +660,22 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
             }
             int nref = 0;
             if constexpr (MR)
-                r = chord_voxel<TA, TS, TF>(Sp, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]},
+                r = chord_voxel<TA, TS, TF>(pb, el6, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]},
                                             sg, mc, tol, maxit, ls_free, F, refresh != 0, nev, nref);
             else
-                r = chord_voxel<TA, TS, TF>(Sp, Mtab + 72 * (long)g, etr, tauc[v], sg, mc, tol, maxit, ls_free, F,
+                r = chord_voxel<TA, TS, TF>(pb, el6, tauc[v], sg, mc, tol, maxit, ls_free, F,
                                             refresh != 0, nev, nref);
             if (nref) {
                 store_factors(fac, N3, v, F);
             }
         } else {
             if constexpr (MR)
-                r = newton_voxel<TA, TF>(Sp, Mtab + 72 * (long)g, etr, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]}, sg,
+                r = newton_voxel<TA, TF>(pb, el6, FlowMR<TA>{mrp.tpi, N3, v, tauc[v]}, sg,
                                          mc, tol, maxit, ls_free, nev);
             else
-                r = newton_voxel<TA, TF>(Sp, Mtab + 72 * (long)g, etr, tauc[v], sg, mc, tol, maxit, ls_free, nev);
+                r = newton_voxel<TA, TF>(pb, el6, tauc[v], sg, mc, tol, maxit, ls_free, nev);
         }
+        pb.leave(sg);
         // local strain e_tr = eps_tr' - S0 sigma and the gap d = eps_tr - e_tr to about twice the field
         // precision: near convergence eps_tr and e_tr agree to many digits, and forming them in plain FP32
         // leaves rounding noise in d (hence in the multiplier update) that keeps the iteration from
@@ -872,24 +896,24 @@ template <typename TA, typename F> cudaError_t by_law(MRPtr<TA> mrp, F &&go) {
 }
 
 template <typename TA>
-cudaError_t newton_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, const TA *Stab,
-                         const TA *Mtab, MatConst mc, double tol, int maxit, int solve_fp64, int *flags,
+cudaError_t newton_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, LocalTab<TA> tab,
+                         MatConst mc, double tol, int maxit, int solve_fp64, int *flags,
                          cudaStream_t s, const int *skip, const TA *tol_dev, MRPtr<TA> mrp) {
     const int blocks = (int)((N3 + kThreads - 1) / kThreads);
     return by_law(mrp, [&](auto law) {
         constexpr bool MR = decltype(law)::value;
         if (solve_fp64)
-            k_newton<TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, Stab, Mtab, mc, (TA)tol,
+            k_newton<TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, tab, mc, (TA)tol,
                                                                  maxit, ls_free_of<TA>(), flags, skip, tol_dev, mrp);
         else
-            k_newton<TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, Stab, Mtab, mc, (TA)tol, maxit,
+            k_newton<TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, tab, mc, (TA)tol, maxit,
                                                              ls_free_of<TA>(), flags, skip, tol_dev, mrp);
     });
 }
 
 template <typename TA>
-cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, const TA *Stab,
-                               const TA *Mtab, void *fac, MatConst mc, double tol, int maxit, int solve_fp64,
+cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const int32_t *g0, TA *sig, LocalTab<TA> tab,
+                               void *fac, MatConst mc, double tol, int maxit, int solve_fp64,
                                int force_refresh, int *flags, int32_t *wl, int nsm, cudaStream_t s, const int *skip,
                                const TA *tol_dev, MRPtr<TA> mrp, int two_step) {
     const int blocks = (int)((N3 + kThreads - 1) / kThreads);
@@ -909,20 +933,20 @@ cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const in
             constexpr bool MR = decltype(law)::value;
             if (two_step)
                 err = launch_k(pdl, k_chord_first<TA, TA, MR, true>, dim3(blocks), dim3(kThreads), 0, s, N3, epst, tauc,
-                               g0, sig, Stab, Mtab, (const TA *)fac, mc, (TA)tol, ls_free_of<TA>(), flags, wl, skip,
+                               g0, sig, tab, (const TA *)fac, mc, (TA)tol, ls_free_of<TA>(), flags, wl, skip,
                                tol_dev, mrp);
             else
                 err = launch_k(pdl, k_chord_first<TA, TA, MR, false>, dim3(blocks), dim3(kThreads), 0, s, N3, epst,
-                               tauc, g0, sig, Stab, Mtab, (const TA *)fac, mc, (TA)tol, ls_free_of<TA>(), flags, wl,
+                               tauc, g0, sig, tab, (const TA *)fac, mc, (TA)tol, ls_free_of<TA>(), flags, wl,
                                skip, tol_dev, mrp);
             if (err != cudaSuccess) return;
             if (solve_fp64)
                 err = launch_k(pdl, k_chord_rest<TA, TA, double, MR>, dim3(rb), dim3(kThreads), 0, s, N3, epst, tauc,
-                               g0, sig, Stab, Mtab, (TA *)fac, mc, (TA)tol, maxit, ls_free_of<TA>(), flags,
+                               g0, sig, tab, (TA *)fac, mc, (TA)tol, maxit, ls_free_of<TA>(), flags,
                                (const int32_t *)wl, skip, tol_dev, mrp);
             else
                 err = launch_k(pdl, k_chord_rest<TA, TA, TA, MR>, dim3(rb), dim3(kThreads), 0, s, N3, epst, tauc, g0,
-                               sig, Stab, Mtab, (TA *)fac, mc, (TA)tol, maxit, ls_free_of<TA>(), flags,
+                               sig, tab, (TA *)fac, mc, (TA)tol, maxit, ls_free_of<TA>(), flags,
                                (const int32_t *)wl, skip, tol_dev, mrp);
         });
         return err != cudaSuccess ? err : cudaGetLastError();
@@ -931,12 +955,12 @@ cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const in
     return by_law(mrp, [&](auto law) {
         constexpr bool MR = decltype(law)::value;
         if (solve_fp64)
-            k_newton_chord<TA, TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, Stab, Mtab,
+            k_newton_chord<TA, TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, tab,
                                                                            (TA *)fac, mc, (TA)tol, maxit,
                                                                            ls_free_of<TA>(), force_refresh, flags,
                                                                            skip, tol_dev, mrp);
         else
-            k_newton_chord<TA, TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, Stab, Mtab, (TA *)fac,
+            k_newton_chord<TA, TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, tab, (TA *)fac,
                                                                        mc, (TA)tol, maxit, ls_free_of<TA>(),
                                                                        force_refresh, flags, skip, tol_dev, mrp);
     });
@@ -946,18 +970,17 @@ int al_blocks(long N3) { return (int)((N3 + kThreads - 1) / kThreads); }
 int al_grid(long N3, int nsm, int tsize) { return std::min(al_blocks(N3), std::max(nsm, 1) * (tsize == 4 ? 3 : 2)); }
 
 cudaError_t newton_field_df(long N3, const double *epst, const double *tauc, const int32_t *g0, double *sig,
-                            const double *Stab, const double *Mtab, const float *Stabf, const float *Mtabf,
-                            MatConst mc, double tol, int maxit, int *flags, cudaStream_t s, const int *skip,
+                            LocalTab<double> tab, MatConst mc, double tol, int maxit, int *flags, cudaStream_t s, const int *skip,
                             const double *tol_dev) {
     const int blocks = (int)((N3 + kThreads - 1) / kThreads);
-    k_newton_df<<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, Stab, Mtab, Stabf, Mtabf, mc, tol, maxit, flags,
+    k_newton_df<<<blocks, kThreads, 0, s>>>(N3, epst, tauc, g0, sig, tab, mc, tol, maxit, flags,
                                             skip, tol_dev);
     return cudaGetLastError();
 }
 
 template <typename TA>
 cudaError_t al_local(long N3, const TA *epst, const TA *epse, const TA *tauc, const int32_t *g0, TA *sig, TA *lam, TA *p,
-                     const TA *Stab, const TA *Sal, const TA *Mtab, MatConst mc, double lam0, double mu0, double tol,
+                     LocalTab<TA> tab, MatConst mc, double lam0, double mu0, double tol,
                      int maxit, int solve_fp64, int init, int *flags, double *part, void *fac, int refresh,
                      cudaStream_t s, int nsm, MRPtr<TA> mrp) {
     const int blocks = al_grid(N3, nsm, (int)sizeof(TA));
@@ -967,14 +990,14 @@ cudaError_t al_local(long N3, const TA *epst, const TA *epse, const TA *tauc, co
     return by_law(mrp, [&](auto law) {
         constexpr bool MR = decltype(law)::value;
         if (solve_fp64)
-            k_al_local<TA, TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, epse, tauc, g0, sig, lam, p, Stab, Sal,
-                                                                       Mtab, mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo,
+            k_al_local<TA, TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, epse, tauc, g0, sig, lam, p, tab,
+                                                                       mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo,
                                                                        sb_lo, sad, sbd, (TA)tol, maxit,
                                                                        ls_free_of<TA>(), init, flags, part, (TA *)fac,
                                                                        refresh, mrp);
         else
-            k_al_local<TA, TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, epse, tauc, g0, sig, lam, p, Stab, Sal,
-                                                                   Mtab, mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo, sb_lo,
+            k_al_local<TA, TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, epse, tauc, g0, sig, lam, p, tab,
+                                                                   mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo, sb_lo,
                                                                    sad, sbd, (TA)tol, maxit, ls_free_of<TA>(), init,
                                                                    flags, part, (TA *)fac, refresh, mrp);
     });
@@ -1005,14 +1028,14 @@ template <typename TA> cudaError_t total_strain(long N3, const TA *epse, const T
 }
 
 #define EVP_INST(TA)                                                                                              \
-    template cudaError_t newton_field<TA>(long, const TA *, const TA *, const int32_t *, TA *, const TA *,        \
-                                          const TA *, MatConst, double, int, int, int *, cudaStream_t,           \
+    template cudaError_t newton_field<TA>(long, const TA *, const TA *, const int32_t *, TA *, LocalTab<TA>,      \
+                                          MatConst, double, int, int, int *, cudaStream_t,           \
                                           const int *, const TA *, MRPtr<TA>);                                   \
-    template cudaError_t newton_chord_field<TA>(long, const TA *, const TA *, const int32_t *, TA *, const TA *,  \
-                                                const TA *, void *, MatConst, double, int, int, int, int *,       \
+    template cudaError_t newton_chord_field<TA>(long, const TA *, const TA *, const int32_t *, TA *, LocalTab<TA>, \
+                                                void *, MatConst, double, int, int, int, int *,       \
                                                 int32_t *, int, cudaStream_t, const int *, const TA *, MRPtr<TA>, int); \
     template cudaError_t al_local<TA>(long, const TA *, const TA *, const TA *, const int32_t *, TA *, TA *, TA *, \
-                                      const TA *, const TA *, const TA *, MatConst, double, double, double, int, int, \
+                                      LocalTab<TA>, MatConst, double, double, double, int, int, \
                                       int, int *, double *, void *, int, cudaStream_t, int, MRPtr<TA>);           \
     template cudaError_t predictor<TA>(long, const TA *, const TA *, const TA *, TA *, TA *, MatConst, double,    \
                                        const double *, int, cudaStream_t);                                        \
