@@ -495,8 +495,8 @@ double vm_strain(const double e[6]) {
 // Returns a status; fills the iteration count, residuals, mean stress and the macro strain increment.
 static_assert(sizeof(FpCtl) <= 256, "FpCtl must fit its workspace slot");
 constexpr int kFpBatch = 16;   // iterations queued between host reads of the control block
-constexpr int kTwoStepIters = 40;   // iterations of an increment whose first local-solve pass takes two chord steps
 const double kZero6[6] = {0, 0, 0, 0, 0, 0};
+constexpr int kTwoStepIters = 40;   // iterations of an increment whose first local-solve pass takes two chord steps
 
 // The x and y passes of the fixed point's transforms, forward and inverse: one launch each where the (field, z)
 // plane fits shared memory (timed as classes 1 and 5), else the two passes (classes 1, 2 and 4, 5).
@@ -515,14 +515,15 @@ template <typename T> cudaError_t fwd_xy(evp_handle *h, const T *in, const int *
     return fft_y<T>(h->spec, h->n, 6, 0, h->st, skip);
 }
 template <typename T>
-cudaError_t inv_xy(evp_handle *h, T *out, T scale, const double *add6, const T *base, const int *skip = nullptr) {
+cudaError_t inv_xy(evp_handle *h, T *out, T scale, const double *add6, const T *base, const int *skip = nullptr,
+                   const InvCtl *ic = nullptr) {
     if (fft_xy_fused(h->n, h->dbl)) {
         PROF(5, 1);
-        return fft_xy_c2r<T>(h->spec, out, h->n, 6, scale, add6, h->st, base, skip);
+        return fft_xy_c2r<T>(h->spec, out, h->n, 6, scale, add6, h->st, base, skip, ic);
     }
     {
         PROF(4, 1);
-        const cudaError_t e = fft_y<T>(h->spec, h->n, 6, 1, h->st, skip);
+        const cudaError_t e = fft_y<T>(h->spec, h->n, 6, 1, h->st, skip, ic);
         if (e != cudaSuccess) return e;
     }
     PROF(5, 1);
@@ -907,8 +908,11 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
         zc.ctl = dc;
         zc.flags = h->flags;
         zc.scal = h->scal;
-        zc.p.N3 = (double)N3; zc.p.tau0 = h->p.tau0; zc.p.tol = h->cfg.tol; zc.p.a = a; zc.p.b = b; zc.p.det = det;
-        zc.p.mu0 = mu0r; zc.p.ntol = ntol; zc.p.eta = h->cfg.newton_adapt; zc.p.max_iter = h->cfg.max_iter;
+        zc.p.n6 = (double)N3 * (double)N3; zc.p.tau02 = h->p.tau0 * h->p.tau0;
+        zc.p.tol2 = h->cfg.tol * h->cfg.tol;
+        zc.p.ca = a / det; zc.p.cb = b / det; zc.p.cs = 1.0 / (2.0 * mu0r);
+        zc.p.max_iter = h->cfg.max_iter;
+        const InvCtl ic{dc, h->scal, (double)N3, h->p.tau0, ntol, h->cfg.newton_adapt};
         int queued = 0;
         while (true) {
             const int nb = std::min(kFpBatch, h->cfg.max_iter - queued);
@@ -954,9 +958,9 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
                 }
                 // the strain correction arrives through the zero-frequency term: no offsets here
                 if (h->dbl) {
-                    CK(inv_xy<double>(h, (double *)h->epst, inv, kZero6, nullptr, skip));
+                    CK(inv_xy<double>(h, (double *)h->epst, inv, kZero6, nullptr, skip, &ic));
                 } else {
-                    CK(inv_xy<float>(h, (float *)h->epst, (float)inv, kZero6, nullptr, skip));
+                    CK(inv_xy<float>(h, (float *)h->epst, (float)inv, kZero6, nullptr, skip, &ic));
                 }
             }
             queued += nb;
@@ -969,12 +973,16 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
         it = hc.it;
         conv = hc.conv;
         nmax = hc.nmax;
-        err_eq = hc.err_eq;
-        err_bc = hc.err_bc;
+        double mn = 0.0, mu_n = 0.0;
         for (int i = 0; i < 6; ++i) {
             dE[i] = hc.dE[i];
             mean[i] = hs[i];
+            mn += hs[i] * hs[i];
+            if (i != 2) mu_n += hs[i] * hs[i];
         }
+        const double den = std::fmax(std::sqrt(mn), h->p.tau0);
+        err_eq = std::sqrt(hs[6]) / ((double)N3 * den);
+        err_bc = std::sqrt(mu_n) / den;
         if (hc.status == EVP_ERR_NEWTON)
             status = fail(h, EVP_ERR_NEWTON, "local Newton failed in %d voxels at iteration %d", hc.nfail, it);
         else if (hc.status == EVP_ERR_NONFINITE)

@@ -11,9 +11,9 @@
 // per direction over whole planes (k_fft_xy_r2c, k_fft_xy_c2r), so an iteration crosses HBM three times.
 // Spectra are [field][z|kz][ky][kx] with kx = 0..N/2 (row length N/2+1).
 //
-// Line transforms: Stockham auto-sort with register butterflies. N = R1 * R2 with R1 = min(N, 16)
+// Line transforms: Stockham auto-sort with register butterflies. N = R1 * R2 with R1 = 16 (8 for N <= 32, see Shape)
 // and R2 = N / R1 <= 16: a radix-R1 pass (no twiddles) and a radix-R2 pass (twiddles W_N^{r j}),
-// natural order in and out. Shared-memory lines are padded (one slot per 16) so that the strided
+// natural order in and out. Shared-memory lines are padded (one slot per R1) so that the strided
 // pass-1 writes hit distinct banks.
 #include <cmath>
 #include <cstdint>
@@ -39,12 +39,19 @@ template <int B> __device__ __forceinline__ void cp_async(void *smem, const void
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// Radices and padded line stride. N = 16 and 32 take R1 = 8: a plane or a slab of such a grid is small, its transform is
+// bound by the latency of each thread's chain and by the threads it occupies, and radix-8 items are twice as many and
+// half as long as radix-16 ones (32^3 FP32 plane of 16 packed lines: 64 items instead of 32). Their second pass starts
+// with the last stage of the radix-16 network (pass2_tail), so the arithmetic is that of the radix-16 split,
+// operation by operation. The line strides keep both ways a warp walks a tile (along lines, across lines) at most
+// two-way bank-conflicted. NTW: slots of the twiddle table (load_tw).
 template <int N> struct Shape {
-    static constexpr int R1 = N < 16 ? N : 16;
+    static constexpr int R1 = N < 16 ? N : N <= 32 ? 8 : 16;
     static constexpr int R2 = N / R1;
-    static constexpr int LS = N + N / 16 + 1;   // padded line stride
+    static constexpr int LS = N >= 64 ? N + N / 16 + 1 : N == 32 ? 38 : N == 16 ? 22 : N + 1;
+    static constexpr int NTW = R1 == 8 && R2 > 1 ? N + 8 : N;
 };
-__device__ __forceinline__ int pad16(int i) { return i + (i >> 4); }
+template <int N> __host__ __device__ constexpr int padn(int i) { return N < 16 ? i : i + i / Shape<N>::R1; }
 
 template <int L> struct Log2 { static constexpr int v = 1 + Log2<L / 2>::v; };
 template <> struct Log2<1> { static constexpr int v = 0; };
@@ -139,13 +146,13 @@ template <int N, int TX> __device__ __forceinline__ void slab_item(int r, int &z
 
 // The two passes of block_fft (R2 > 1), also called on their own by the z pass.
 // pass 1: radix R1, Ns = 1: item (l, j < M1) reads slots j + M1 r and writes j R1 + r, so
-// every read completes before any write (held in registers across a barrier). With j < M1 and M1 | 16
-// the padded slots are pad16(j + M1 r) = j + pad16(M1 r) and pad16(16 j + r) = 17 j + r (r < 16): one base
+// every read completes before any write (held in registers across a barrier). With j < M1 and M1 | R1
+// the padded slots are padn(j + M1 r) = j + padn(M1 r) and padn(R1 j + r) = (R1 + 1) j + r (r < R1): one base
 // address per item and compile-time offsets. Ends with a barrier.
 template <int N, bool INV, int MAXIT, typename C> __device__ void bfft_pass1(C *buf, int nlines) {
     constexpr int R1 = Shape<N>::R1, LS = Shape<N>::LS;
     constexpr int M1 = N / R1;
-    static_assert(16 % M1 == 0 || M1 % 16 == 0, "pass-1 stride");
+    static_assert(R1 % M1 == 0, "pass-1 stride");
     const int items = nlines * M1;
     C v[MAXIT][R1];
 #pragma unroll
@@ -154,9 +161,9 @@ template <int N, bool INV, int MAXIT, typename C> __device__ void bfft_pass1(C *
         if (t < items) {
             int l, j;
             pass1_item<N>(t, nlines, l, j);
-            const C *src = buf + l * LS + (M1 <= 16 ? j : pad16(j));
+            const C *src = buf + l * LS + j;
 #pragma unroll
-            for (int r = 0; r < R1; ++r) v[it][r] = src[M1 <= 16 ? pad16(r * M1) : r * (M1 + M1 / 16)];
+            for (int r = 0; r < R1; ++r) v[it][r] = src[padn<N>(r * M1)];
         }
     }
     __syncthreads();
@@ -167,7 +174,7 @@ template <int N, bool INV, int MAXIT, typename C> __device__ void bfft_pass1(C *
             int l, j;
             pass1_item<N>(t, nlines, l, j);
             dft_reg<R1, INV>(v[it]);
-            C *dst = buf + l * LS + 17 * j;
+            C *dst = buf + l * LS + (R1 + 1) * j;
 #pragma unroll
             for (int r = 0; r < R1; ++r) dst[r] = v[it][r];
         }
@@ -175,49 +182,121 @@ template <int N, bool INV, int MAXIT, typename C> __device__ void bfft_pass1(C *
     __syncthreads();
 }
 
-// pass 2: radix R2, Ns = R1 = 16: item (l, j < 16) reads and writes slots j + 16 r only, which are
-// pad16(j + 16 r) = j + 17 r
-// Every CTA has a multiple of 16 threads, so a thread's items share one j = threadIdx.x mod 16 and its
-// twiddles tw[16 r + j] = exp(-2 pi i r j / N) are loaded once, into registers. Ends with a barrier.
-template <int N, bool INV, typename C> __device__ void bfft_pass2(C *buf, int nlines, const C *tw) {
-    constexpr int R2 = Shape<N>::R2, LS = Shape<N>::LS;
-    const int jt = threadIdx.x & 15;
-    C wr[R2];
+// a * w with the rounding of the FP32 product written out (which product of each sum is fused): FY fuses a.y w.x into the
+// imaginary part, else a.x w.y.
+template <bool FY> __device__ __forceinline__ float2 cmul_r(float2 a, float2 w) {
+    return make_float2(fmaf(a.x, w.x, -__fmul_rn(a.y, w.y)),
+                       FY ? fmaf(a.y, w.x, __fmul_rn(a.x, w.y)) : fmaf(a.x, w.y, __fmul_rn(a.y, w.x)));
+}
+template <bool FY> __device__ __forceinline__ double2 cmul_r(double2 a, double2 w) { return cmul(a, w); }
+
+// The arithmetic of the second pass on the R2 values u[r] of slots j + R1 r, in place. N >= 64: twiddles
+// tw[R1 r + j], then a radix-R2 DFT. N <= 32: values r and r + R2/2 are the even and odd halves of a radix-16 DFT, so
+// its last stage (W16^j, at tw[N + j]) gives its outputs j and j + 8, which then take the twiddles and the radix-R2/2
+// DFT of the 16 x R2/2 split; slot j + 8 q holds its output q.
+// FY (cmul_r): chosen so that FP32 transforms of 16 and 32 points give the bits of the radix-16 form.
+template <int N, bool INV, bool FY = true, typename C> __device__ __forceinline__ void pass2_tail(C (&u)[Shape<N>::R2], int j, const C *tw) {
+    constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2;
+    auto tw_at = [&](int i) {
+        C w = tw[i];
+        if (INV) w.y = -w.y;
+        return w;
+    };
+    if constexpr (R1 == 16) {
 #pragma unroll
-    for (int r = 1; r < R2; ++r) {
-        wr[r] = tw[16 * r + jt];   // r-major: a half-warp reads 16 in a row
-        if (INV) wr[r].y = -wr[r].y;
-    }
-    for (int t = threadIdx.x; t < nlines * 16; t += blockDim.x) {
-        const int l = t >> 4;
-        C *line = buf + l * LS + jt;
-        C u[R2];
-#pragma unroll
-        for (int r = 0; r < R2; ++r) {
-            C a = line[17 * r];
-            if (r > 0) a = cmul(a, wr[r]);
-            u[r] = a;
-        }
+        for (int r = 1; r < R2; ++r) u[r] = cmul(u[r], tw_at(16 * r + j));
         dft_reg<R2, INV>(u);
+    } else {
+        constexpr int Q = R2 / 2;
+        const C w = tw_at(N + j);
+        C a[Q], b[Q];
 #pragma unroll
-        for (int r = 0; r < R2; ++r) line[17 * r] = u[r];
+        for (int r = 0; r < Q; ++r) {
+            const C y = u[r + Q];
+            C z;
+            if constexpr (sizeof(C) == 8) {
+                // rounded as dft_reg's products by constants are (which product of a sum is fused)
+                const bool fx = !(j == 6 && !INV), fy = j == 2;
+                const float px = fx ? y.x : -y.y, qx = fx ? w.x : w.y, rx = fx ? -y.y : y.x, tx = fx ? w.y : w.x;
+                const float py = fy ? y.x : y.y, qy = fy ? w.y : w.x, ry = fy ? y.y : y.x, ty = fy ? w.x : w.y;
+                z.x = fmaf(px, qx, __fmul_rn(rx, tx));
+                z.y = fmaf(py, qy, __fmul_rn(ry, ty));
+            } else {
+                z = cmk<C>(y.x * w.x - y.y * w.y, y.x * w.y + y.y * w.x);
+            }
+            if (j == 0) z = y;   // as in dft_reg: the twiddles 1 and -i (+i inverse) are not multiplied
+            if (j == 4) z = INV ? cmk<C>(-y.y, y.x) : cmk<C>(y.y, -y.x);
+            a[r] = cadd(u[r], z);
+            b[r] = csub(u[r], z);
+        }
+        if constexpr (Q > 1) {
+#pragma unroll
+            for (int r = 1; r < Q; ++r) {
+                a[r] = cmul_r<FY>(a[r], tw_at(16 * r + j));
+                b[r] = cmul_r<FY>(b[r], tw_at(16 * r + j + 8));
+            }
+            dft_reg<Q, INV>(a);
+            dft_reg<Q, INV>(b);
+        }
+#pragma unroll
+        for (int r = 0; r < Q; ++r) {
+            u[2 * r] = a[r];
+            u[2 * r + 1] = b[r];
+        }
+    }
+}
+
+// pass 2: item (l, j < R1) reads and writes slots j + R1 r only, which are padn(j + R1 r) = j + (R1 + 1) r.
+// Every CTA has a multiple of R1 threads, so a thread's items share one j = threadIdx.x mod R1; at N >= 64 its
+// twiddles tw[R1 r + j] = exp(-2 pi i r j / N) are loaded once, into registers. Ends with a barrier.
+template <int N, bool INV, typename C> __device__ void bfft_pass2(C *buf, int nlines, const C *tw) {
+    constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2, LS = Shape<N>::LS;
+    const int jt = threadIdx.x & (R1 - 1);
+    if constexpr (R1 == 16) {
+        C wr[R2];
+#pragma unroll
+        for (int r = 1; r < R2; ++r) {
+            wr[r] = tw[R1 * r + jt];   // r-major: R1 lanes read R1 in a row
+            if (INV) wr[r].y = -wr[r].y;
+        }
+        for (int t = threadIdx.x; t < nlines * R1; t += blockDim.x) {
+            C *line = buf + (t / R1) * LS + jt;
+            C u[R2];
+#pragma unroll
+            for (int r = 0; r < R2; ++r) {
+                C a = line[(R1 + 1) * r];
+                if (r > 0) a = cmul(a, wr[r]);
+                u[r] = a;
+            }
+            dft_reg<R2, INV>(u);
+#pragma unroll
+            for (int r = 0; r < R2; ++r) line[(R1 + 1) * r] = u[r];
+        }
+    } else {
+        for (int t = threadIdx.x; t < nlines * R1; t += blockDim.x) {
+            C *line = buf + (t / R1) * LS + jt;
+            C u[R2];
+#pragma unroll
+            for (int r = 0; r < R2; ++r) u[r] = line[(R1 + 1) * r];
+            pass2_tail<N, INV, !(N == 32 && !INV)>(u, jt, tw);
+#pragma unroll
+            for (int r = 0; r < R2; ++r) line[(R1 + 1) * r] = u[r];
+        }
     }
     __syncthreads();
 }
 
-// In-place transform of nlines padded lines (line l at buf + l*LS). tw[16 r + j] = exp(-2 pi i r j / N)
-// (see load_tw),
-// m < N. Starts after and ends with a barrier. MAXIT >= ceil(nlines * (N/R1) / blockDim).
+// In-place transform of nlines padded lines (line l at buf + l*LS). tw: see load_tw. Starts after and ends with a barrier. MAXIT >= ceil(nlines * (N/R1) / blockDim).
 template <int N, bool INV, int MAXIT, typename C> __device__ void block_fft(C *buf, int nlines, const C *tw) {
     constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2, LS = Shape<N>::LS;
     if constexpr (R2 == 1) {   // a single radix-N pass; every line is owned by one thread
         for (int l = threadIdx.x; l < nlines; l += blockDim.x) {
             C v[R1];
 #pragma unroll
-            for (int r = 0; r < R1; ++r) v[r] = buf[l * LS + pad16(r)];
+            for (int r = 0; r < R1; ++r) v[r] = buf[l * LS + padn<N>(r)];
             dft_reg<R1, INV>(v);
 #pragma unroll
-            for (int r = 0; r < R1; ++r) buf[l * LS + pad16(r)] = v[r];
+            for (int r = 0; r < R1; ++r) buf[l * LS + padn<N>(r)] = v[r];
         }
         __syncthreads();
     } else {
@@ -226,22 +305,47 @@ template <int N, bool INV, int MAXIT, typename C> __device__ void block_fft(C *b
     }
 }
 
-// Twiddles of the radix-R2 pass, computed once per CTA into shared memory in the precision of the transform
-// (the FP64 pipe is 1/58 of the FP32 rate on this GPU, so FP32 transforms avoid it): slot k = 16 r + j holds
-// exp(-2 pi i r j / N) for r < N/16, j < 16 (r j < N), so the 16 lanes of a half-warp, which differ in j, read
-// 16 consecutive slots (indexed by the product r j the stride-r reads hit the same banks).
-__device__ __forceinline__ void load_tw(float2 *tw_s, int N) {
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        float sn, cs;
-        sincospif(-2.0f * (float)((k >> 4) * (k & 15)) / (float)N, &sn, &cs);
-        tw_s[k] = make_float2(cs, sn);
-    }
+// cos(2 pi k / 256), k = 0 .. 64, rounded to nearest: the FP64 twiddles of every N <= 256 by symmetry. Reading them
+// replaces a sincospi per CTA and twiddle: 128 of them were about a tenth of an FP64 z-pass CTA's FP64 operations.
+// (The FP32 twiddles stay sincospif's, on the FP32 pipe.)
+__device__ const double kCos256[65] = {
+    1.0, 0.9996988186962042, 0.9987954562051724, 0.9972904566786902, 0.9951847266721969,
+    0.99247953459871, 0.989176509964781, 0.9852776423889412, 0.9807852804032304, 0.9757021300385286,
+    0.970031253194544, 0.9637760657954398, 0.9569403357322088, 0.9495281805930367, 0.9415440651830208,
+    0.9329927988347388, 0.9238795325112867, 0.9142097557035307, 0.9039892931234433, 0.8932243011955153,
+    0.881921264348355, 0.8700869911087115, 0.8577286100002721, 0.8448535652497071, 0.8314696123025452,
+    0.8175848131515837, 0.8032075314806449, 0.7883464276266062, 0.773010453362737, 0.7572088465064846,
+    0.7409511253549591, 0.7242470829514669, 0.7071067811865476, 0.6895405447370669, 0.6715589548470184,
+    0.6531728429537768, 0.6343932841636455, 0.6152315905806268, 0.5956993044924334, 0.5758081914178453,
+    0.5555702330196022, 0.5349976198870973, 0.5141027441932218, 0.49289819222978404, 0.47139673682599764,
+    0.4496113296546066, 0.4275550934302821, 0.40524131400498986, 0.3826834323650898, 0.35989503653498817,
+    0.33688985339222005, 0.31368174039889146, 0.2902846772544624, 0.26671275747489837, 0.2429801799032639,
+    0.2191012401568698, 0.19509032201612828, 0.17096188876030122, 0.14673047445536175, 0.1224106751992162,
+    0.0980171403295606, 0.07356456359966743, 0.049067674327418015, 0.024541228522912288, 0.0,
+};
+// exp(-2 pi i k / 256), 0 <= k < 256
+__device__ __forceinline__ double2 root256(int k) {
+    const int q = k >> 6, m = k & 63;
+    const double c = __ldg(kCos256 + m), d = __ldg(kCos256 + 64 - m);   // cos, sin of the angle within its quarter
+    return q == 0 ? make_double2(c, -d) : q == 1 ? make_double2(-d, -c) : q == 2 ? make_double2(-c, d) : make_double2(d, c);
 }
-__device__ __forceinline__ void load_tw(double2 *tw_s, int N) {
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        double sn, cs;
-        sincospi(-2.0 * (double)((k >> 4) * (k & 15)) / (double)N, &sn, &cs);
-        tw_s[k] = make_double2(cs, sn);
+__device__ __forceinline__ float2 root_of(float2, int k, int N) {   // exp(-2 pi i k / N)
+    float sn, cs;
+    sincospif(-2.0f * (float)k / (float)N, &sn, &cs);
+    return make_float2(cs, sn);
+}
+__device__ __forceinline__ double2 root_of(double2, int k, int N) { return root256(k * (256 / N)); }
+// Twiddles into shared memory, once per CTA: slot 16 r + j holds exp(-2 pi i r j / N) for r < N / 16, j < 16 (r j < N),
+// so lanes that differ in j read consecutive slots; with radix-8 first passes slots N .. N + 7 hold W16^0 .. W16^7.
+template <int N, typename C> __device__ __forceinline__ void load_tw(C *tw_s) {
+    using T = decltype(C::x);
+    for (int k = threadIdx.x; k < Shape<N>::NTW; k += blockDim.x) {
+        if (k < N) {
+            tw_s[k] = root_of(C{}, (k >> 4) * (k & 15), N);
+        } else {
+            const double2 w = root256(16 * (k - N));
+            tw_s[k] = cmk<C>((T)w.x, (T)w.y);
+        }
     }
 }
 
@@ -251,9 +355,12 @@ template <int N> __host__ __device__ constexpr int rowpairs() { return N >= 64 ?
 template <int N, typename T> __host__ __device__ constexpr int tx_y() {
     return (sizeof(T) == 4 ? 32 : 16) < N / 2 ? (sizeof(T) == 4 ? 32 : 16) : N / 2;
 }
-template <int N, typename T> __host__ __device__ constexpr int tx_z() {
-    return (sizeof(T) == 4 ? 8 : 4) < N / 2 ? (sizeof(T) == 4 ? 8 : 4) : N / 2;
+// z-pass tiles: 64-byte column segments; two columns on grids of 16 and 32, where wider tiles would leave most of the
+// chip idle (32^3 FP32: 256 CTAs instead of 64).
+__host__ __device__ constexpr int tx_z_of(int n, int tsize) {
+    return n <= 8 ? n / 2 : n <= 32 ? 2 : 32 / tsize;
 }
+template <int N, typename T> __host__ __device__ constexpr int tx_z() { return tx_z_of(N, sizeof(T)); }
 template <int N> __host__ __device__ constexpr int maxit(int lines, int threads = kThreads) {
     return (lines * (N / Shape<N>::R1) + threads - 1) / threads < 1 ? 1
                                                                    : (lines * (N / Shape<N>::R1) + threads - 1) / threads;
@@ -267,7 +374,9 @@ template <int N> __host__ __device__ constexpr int tile_threads(int lines, int e
                : ((((lines + extra) * (N / Shape<N>::R1) + maxit<N>(lines) - 1) / maxit<N>(lines) + 31) / 32) * 32;
 }
 template <int N, typename T> __host__ __device__ constexpr int y_threads() { return tile_threads<N>(tx_y<N, T>(), 1); }
-template <int N, typename T> __host__ __device__ constexpr int z_threads() { return tile_threads<N>(6 * tx_z<N, T>(), 6); }
+template <int N, typename T> __host__ __device__ constexpr int z_threads() {
+    return N == 16 || N == 32 ? 128 : tile_threads<N>(6 * tx_z<N, T>(), 6);
+}
 
 // ---------------------------------------------------------------------------------------------
 // x pass, real -> half spectrum. CTA = RP pairs of rows (y even, y+1) of one (field, z).
@@ -275,21 +384,21 @@ template <int N, typename T> __host__ __device__ constexpr int z_threads() { ret
 template <typename T, int N>
 __global__ void __launch_bounds__(kThreads, N >= 64 && N <= 128 ? (sizeof(T) == 4 ? 6 : 3) : 1) k_fft_x_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out,
                                                        long npairs, const int *__restrict__ skip) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    using C = typename CT<T>::type;
     constexpr int RP = rowpairs<N>(), LS = Shape<N>::LS, Hx = N / 2 + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw = reinterpret_cast<C *>(smem_raw);
-    C *buf = tw + N;
-    load_tw(tw, N);
     const long p0 = (long)blockIdx.x * RP;
     const int np = (int)min((long)RP, npairs - p0);
     for (int t = threadIdx.x; t < np * N; t += blockDim.x) {
         const int pl = t / N, j = t - pl * N;
         const long row0 = 2 * (p0 + pl);            // global row index = (field*N + z)*N + y
-        T *slot = reinterpret_cast<T *>(buf + pl * LS + pad16(j));
+        T *slot = reinterpret_cast<T *>(buf + pl * LS + padn<N>(j));
         cp_async<sizeof(T)>(slot, in + row0 * N + j);
         cp_async<sizeof(T)>(slot + 1, in + (row0 + 1) * N + j);
     }
@@ -299,8 +408,8 @@ __global__ void __launch_bounds__(kThreads, N >= 64 && N <= 128 ? (sizeof(T) == 
     const T h = (T)0.5;
     for (int t = threadIdx.x; t < np * Hx; t += blockDim.x) {
         const int pl = t / Hx, k = t - pl * Hx;
-        const C zk = buf[pl * LS + pad16(k & (N - 1))];
-        const C zc = cconj(buf[pl * LS + pad16((N - k) & (N - 1))]);
+        const C zk = buf[pl * LS + padn<N>(k & (N - 1))];
+        const C zc = cconj(buf[pl * LS + padn<N>((N - k) & (N - 1))]);
         const long row0 = 2 * (p0 + pl);
         out[row0 * Hx + k] = cmk<C>(h * (zk.x + zc.x), h * (zk.y + zc.y));
         out[(row0 + 1) * Hx + k] = cmk<C>(h * (zk.y - zc.y), -h * (zk.x - zc.x));   // (zk - zc) / 2i
@@ -318,14 +427,15 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
                                                        long npairs, T scale, int has_add, T a0, T a1, T a2, T a3, T a4,
                                                        T a5, const T *__restrict__ base, const int *__restrict__ skip) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;                          // RP packed lines
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    using C = typename CT<T>::type;
     constexpr int RP = rowpairs_c2r<N>(), LS = Shape<N>::LS, Hx = N / 2 + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw = reinterpret_cast<C *>(smem_raw);
-    C *buf = tw + N;                          // RP packed lines
     C *hs = buf + RP * LS;                    // 2 RP half-spectrum rows, row-major
     T *bs = reinterpret_cast<T *>(hs + 2 * RP * Hx);   // 2 RP strain rows (with has_add)
     const long p0 = (long)blockIdx.x * RP;
@@ -343,7 +453,6 @@ __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::ty
             for (int t = threadIdx.x; t < nchunk2; t += blockDim.x) cp_async<16>(dst2 + t, src2 + t);
         }
     }
-    load_tw(tw, N);
     cp_async_wait_all();
     __syncthreads();
     for (int t = threadIdx.x; t < np * N; t += blockDim.x) {
@@ -357,18 +466,24 @@ __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::ty
             A = cconj(ra[N - k]);
             B = cconj(rb[N - k]);
         }
-        buf[pl * LS + pad16(k)] = cmk<C>(A.x - B.y, A.y + B.x);   // A + iB
+        buf[pl * LS + padn<N>(k)] = cmk<C>(A.x - B.y, A.y + B.x);   // A + iB
     }
     __syncthreads();
     block_fft<N, true, maxit<N>(RP)>(buf, np, tw);
-    const long rows_per_field = (long)N * N;
+    // the offset of a row's field, formed once where the CTA's rows belong to one field (256^3 FP32: 246 us a pass, 287
+    // with the selection in the loop)
+    auto add_of = [&](long row) -> T {
+        const int f = (int)(row / ((long)N * N));
+        return f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
+    };
+    constexpr bool one_field = (N * N) % (2 * RP) == 0;
+    const T add_cta = one_field ? add_of(2 * p0) : (T)0;
     for (int t = threadIdx.x; t < np * N; t += blockDim.x) {
         const int pl = t / N, j = t - pl * N;
         const long row0 = 2 * (p0 + pl);
-        const C z = buf[pl * LS + pad16(j)];
+        const C z = buf[pl * LS + padn<N>(j)];
         if (has_add) {
-            const int f = (int)(row0 / rows_per_field);
-            const T add = f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
+            const T add = one_field ? add_cta : add_of(row0);
             out[row0 * N + j] = bs[2 * pl * N + j] + (z.x * scale + add);
             out[(row0 + 1) * N + j] = bs[(2 * pl + 1) * N + j] + (z.y * scale + add);
         } else {
@@ -383,38 +498,44 @@ __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::ty
 // ---------------------------------------------------------------------------------------------
 template <typename T, int N, bool INV>
 __global__ void __launch_bounds__(y_threads<N, T>(), sizeof(T) == 4 && N >= 64 && N <= 128 ? 5 : 1)
-k_fft_y(typename CT<T>::type *__restrict__ spec, const int *__restrict__ skip) {
+k_fft_y(typename CT<T>::type *__restrict__ spec, const int *__restrict__ skip, InvCtl ic) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    using C = typename CT<T>::type;
     constexpr int TX = tx_y<N, T>(), LS = Shape<N>::LS, Hx = N / 2 + 1;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw = reinterpret_cast<C *>(smem_raw);
-    C *buf = tw + N;
+    if (INV && ic.ctl != nullptr && blockIdx.x == gridDim.x - 1) {   // as in k_fft_xy_c2r
+        if (threadIdx.x == 0) fp_next_tolerance(ic);
+        return;
+    }
     constexpr int ntiles = (N / 2) / TX;
     const int tile = blockIdx.x % ntiles;
     const long plane = blockIdx.x / ntiles;        // field*N + z
     const bool nyq = tile == 0;                    // tile 0 also carries the column kx = N/2 as line TX
     C *base = spec + plane * (long)N * Hx;
     const int kx0 = tile * TX;
-    load_tw(tw, N);
     for (int t = threadIdx.x; t < TX * N; t += blockDim.x) {   // TX, N powers of two: shifts, no division
         const int y = t / TX, xl = t % TX;
-        cp_async<sizeof(C)>(buf + xl * LS + pad16(y), base + (long)y * Hx + kx0 + xl);
+        cp_async<sizeof(C)>(buf + xl * LS + padn<N>(y), base + (long)y * Hx + kx0 + xl);
     }
     if (nyq)
         for (int y = threadIdx.x; y < N; y += blockDim.x)
-            cp_async<sizeof(C)>(buf + TX * LS + pad16(y), base + (long)y * Hx + N / 2);
+            cp_async<sizeof(C)>(buf + TX * LS + padn<N>(y), base + (long)y * Hx + N / 2);
     cp_async_wait_all();
+    // the macroscopic strain correction goes into the zero-frequency term (this thread copied it)
+    if (INV && ic.ctl != nullptr && tile == 0 && threadIdx.x == 0) buf[0].x += (T)(ic.ctl->corr[plane / N] * ic.n3);
     __syncthreads();
     block_fft<N, INV, maxit<N>(TX + 1, y_threads<N, T>())>(buf, TX + (nyq ? 1 : 0), tw);
     for (int t = threadIdx.x; t < TX * N; t += blockDim.x) {
         const int y = t / TX, xl = t % TX;
-        base[(long)y * Hx + kx0 + xl] = buf[xl * LS + pad16(y)];
+        base[(long)y * Hx + kx0 + xl] = buf[xl * LS + padn<N>(y)];
     }
     if (nyq)
-        for (int y = threadIdx.x; y < N; y += blockDim.x) base[(long)y * Hx + N / 2] = buf[TX * LS + pad16(y)];
+        for (int y = threadIdx.x; y < N; y += blockDim.x) base[(long)y * Hx + N / 2] = buf[TX * LS + padn<N>(y)];
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -428,18 +549,18 @@ k_fft_y(typename CT<T>::type *__restrict__ spec, const int *__restrict__ skip) {
 // One thread per pass-1 item of the N/2 row-pair lines (x) and of the N/2 regular columns (y); the Nyquist
 // column's few pass-1 items run on lanes of warp 0 (col_pass1).
 template <int N> __host__ __device__ constexpr int xy_threads() {
-    return (((N / 2) * (N / Shape<N>::R1) + 31) / 32) * 32;
+    return N == 16 ? 64 : N == 32 ? 128 : (((N / 2) * (N / Shape<N>::R1) + 31) / 32) * 32;
 }
 template <typename T, int N> __host__ __device__ constexpr size_t smem_xy() {
-    return sizeof(typename CT<T>::type) * (N + (size_t)(N / 2) * Shape<N>::LS);
+    return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)(N / 2) * Shape<N>::LS);
 }
 // The plane fits next to two others on one SM (FP32 up to N = 128, FP64 up to N = 64), the row pair of the
 // half spectrum fits in a padded line (2 (N/2+1) <= LS), and both passes are two-radix Stockham passes.
 template <typename T, int N> __host__ __device__ constexpr bool xy_fused() {
-    return N >= 32 && Shape<N>::R2 > 1 && 2 * (N / 2 + 1) <= Shape<N>::LS && smem_xy<T, N>() <= 72 * 1024;
+    return N >= 16 && Shape<N>::R2 > 1 && 2 * (N / 2 + 1) <= Shape<N>::LS && smem_xy<T, N>() <= 72 * 1024;
 }
 template <typename T, int N> __host__ __device__ constexpr int xy_ctas() {
-    return sizeof(T) == 4 ? (N >= 128 ? 3 : N == 64 ? 8 : 1) : 1;
+    return sizeof(T) == 4 ? (N >= 128 ? 3 : N == 64 ? 8 : 4) : 1;
 }
 
 // Slot of half-spectrum row y, column kx in the row-major plane (rows 2p and 2p+1 share line p).
@@ -458,7 +579,7 @@ template <int N> __device__ __forceinline__ int xy_at(int y, int kx) {
 // pass writes, so every read comes before any write (a barrier between); otherwise it reads HBM. Ends with a barrier.
 template <int N, bool INV, bool IN_PLACE, typename C, typename Ld> __device__ void x_pass1_ld(C *buf, int nlines, Ld ld) {
     constexpr int R1 = Shape<N>::R1, LS = Shape<N>::LS, M1 = N / R1;
-    static_assert(M1 <= 16 && 16 % M1 == 0, "pass-1 stride");
+    static_assert(R1 % M1 == 0, "pass-1 stride");
     const int t = threadIdx.x;
     const bool on = t < nlines * M1;
     int l = 0, j = 0;
@@ -471,7 +592,7 @@ template <int N, bool INV, bool IN_PLACE, typename C, typename Ld> __device__ vo
     if constexpr (IN_PLACE) __syncthreads();
     if (on) {
         dft_reg<R1, INV>(v);
-        C *dst = buf + l * LS + 17 * j;
+        C *dst = buf + l * LS + (R1 + 1) * j;
 #pragma unroll
         for (int r = 0; r < R1; ++r) dst[r] = v[r];
     }
@@ -514,8 +635,8 @@ __device__ void col_pass1(C *buf, Ld ld, Pre pre, LdN ldn) {
     __syncthreads();
 }
 
-// y pass 2: item (kx, j < 16) transforms rows j + 16 r (line (j >> 1) + 8 r, half j & 1) and hands its outputs
-// (row j + 16 r in u[r]) to st(j, kx, slot of row j, u). Ends with a barrier.
+// y pass 2: item (kx, j < R1) transforms rows j + R1 r (line (j >> 1) + R1 / 2 r, half j & 1) and hands its outputs
+// (row j + R1 r in u[r]) to st(j, kx, slot of row j, u). Ends with a barrier.
 template <int N, bool INV, typename C, typename St> __device__ void col_pass2(C *buf, const C *tw, St st) {
     constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2, Hx = N / 2 + 1, LS = Shape<N>::LS;
     for (int t = threadIdx.x; t < Hx * R1; t += blockDim.x) {
@@ -523,16 +644,8 @@ template <int N, bool INV, typename C, typename St> __device__ void col_pass2(C 
         C *line = buf + xy_at<N>(j, kx);
         C u[R2];
 #pragma unroll
-        for (int r = 0; r < R2; ++r) {
-            C a = line[r * (R1 / 2) * LS];
-            if (r > 0) {
-                C w = tw[16 * r + j];
-                if (INV) w.y = -w.y;
-                a = cmul(a, w);
-            }
-            u[r] = a;
-        }
-        dft_reg<R2, INV>(u);
+        for (int r = 0; r < R2; ++r) u[r] = line[r * (R1 / 2) * LS];
+        pass2_tail<N, INV>(u, j, tw);
         st(j, kx, line, u);
     }
     __syncthreads();
@@ -541,17 +654,17 @@ template <int N, bool INV, typename C, typename St> __device__ void col_pass2(C 
 template <typename T, int N>
 __global__ void __launch_bounds__(xy_threads<N>(), xy_ctas<T, N>())
 k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, const int *__restrict__ skip) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    using C = typename CT<T>::type;
     constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, NP = N / 2, KU = (Hx + 31) / 32, R2 = Shape<N>::R2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw = reinterpret_cast<C *>(smem_raw);
-    C *buf = tw + N;
     const T *src = in + (long)blockIdx.x * N * N;   // plane = field * N + z
     C *dst = out + (long)blockIdx.x * N * Hx;
-    load_tw(tw, N);
     // x: line p packs rows 2p and 2p+1 as one complex row; pass 1 reads them from HBM
     x_pass1_ld<N, false, false>(buf, NP, [&](int p, int e) { return cmk<C>(src[(2 * p) * N + e], src[(2 * p + 1) * N + e]); });
     bfft_pass2<N, false>(buf, NP, tw);
@@ -565,8 +678,8 @@ k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, c
             for (int u = 0; u < KU; ++u) {
                 const int k = lane + 32 * u;
                 if (k < Hx) {
-                    const C zk = line[pad16(k & (N - 1))];
-                    const C zc = cconj(line[pad16((N - k) & (N - 1))]);
+                    const C zk = line[padn<N>(k & (N - 1))];
+                    const C zc = cconj(line[padn<N>((N - k) & (N - 1))]);
                     a[u] = cmk<C>(h * (zk.x + zc.x), h * (zk.y + zc.y));
                     b[u] = cmk<C>(h * (zk.y - zc.y), -h * (zk.x - zc.x));   // (zk - zc) / 2i
                 }
@@ -584,13 +697,12 @@ k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, c
         }
     }
     __syncthreads();
-    // y: down the columns of the row-major plane; pass 2 stores rows j + 16 r to HBM
-    // y: down the columns of the row-major plane; pass 2 stores rows j + 16 r to HBM
+    // y: down the columns of the row-major plane; pass 2 stores rows j + R1 r to HBM
     col_pass1<N, false, true>(
         buf, [&](int y, int kx) { return buf[xy_at<N>(y, kx)]; }, [] {}, [&](int y) { return buf[xy_at<N>(y, N / 2)]; });
     col_pass2<N, false>(buf, tw, [&](int j, int kx, C *, const C (&u)[R2]) {
 #pragma unroll
-        for (int r = 0; r < R2; ++r) dst[(j + 16 * r) * Hx + kx] = u[r];
+        for (int r = 0; r < R2; ++r) dst[(j + Shape<N>::R1 * r) * Hx + kx] = u[r];
     });
 }
 
@@ -599,23 +711,35 @@ k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, c
 template <typename T, int N>
 __global__ void __launch_bounds__(xy_threads<N>(), xy_ctas<T, N>())
 k_fft_xy_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out, T scale, int has_add, T a0, T a1, T a2,
-             T a3, T a4, T a5, const T *__restrict__ base, const int *__restrict__ skip) {
+             T a3, T a4, T a5, const T *__restrict__ base, const int *__restrict__ skip,
+             InvCtl ic) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    using C = typename CT<T>::type;
     constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, NP = N / 2, R2 = Shape<N>::R2;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw = reinterpret_cast<C *>(smem_raw);
-    C *buf = tw + N;
+    if (ic.ctl != nullptr && blockIdx.x == gridDim.x - 1) {   // an extra CTA prepares the next iteration's tolerance
+        if (threadIdx.x == 0) fp_next_tolerance(ic);
+        return;
+    }
     const C *src = spec + (long)blockIdx.x * N * Hx;
-    load_tw(tw, N);
-    // y: pass 1 reads the columns from HBM
+    const T corr = ic.ctl != nullptr ? (T)(ic.ctl->corr[blockIdx.x / N] * ic.n3) : (T)0;
+    // y: pass 1 reads the columns from HBM, with the macroscopic strain correction added to the zero-frequency term
     col_pass1<N, true, false>(
-        buf, [&](int y, int kx) { return src[y * Hx + kx]; }, [] {}, [&](int y) { return src[y * Hx + N / 2]; });
+        buf,
+        [&](int y, int kx) {
+            C v = src[y * Hx + kx];
+            if (ic.ctl != nullptr && y == 0 && kx == 0) v.x += corr;
+            return v;
+        },
+        [] {}, [&](int y) { return src[y * Hx + N / 2]; });
     col_pass2<N, true>(buf, tw, [](int, int, C *line, const C (&u)[R2]) {
 #pragma unroll
-        for (int r = 0; r < R2; ++r) line[r * 8 * LS] = u[r];
+        for (int r = 0; r < R2; ++r) line[r * (Shape<N>::R1 / 2) * LS] = u[r];
     });
     // x: pass 1 packs rows 2p and 2p+1 as it reads them (Z[k] = A[k] + i B[k], with A[N-k] = conj A[k] past N/2)
     // and writes the lines in place
@@ -641,7 +765,7 @@ k_fft_xy_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
     const T *bsrc = base ? base : out;
     for (int t = threadIdx.x; t < NP * N; t += blockDim.x) {
         const int p = t / N, j = t - p * N;
-        const C z = buf[p * LS + pad16(j)];
+        const C z = buf[p * LS + padn<N>(j)];
         const long o0 = (r0 + 2 * p) * N + j, o1 = o0 + N;
         if (has_add) {
             out[o0] = bsrc[o0] + (z.x * scale + add);
@@ -653,14 +777,84 @@ k_fft_xy_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
     }
 }
 
-// Green operator of the isotropic reference medium applied to one spectral stress (Mandel):
-// eps_kh = (n_h v_k + n_k v_h)/(2 mu0) - c n_k n_h (n.v), v = sigma.n, n = xi/|xi|,
-// c = (lam0+mu0)/(mu0 (lam0+2 mu0)). At frequencies with a Nyquist component the compliance of
-// the reference medium replaces it; the zero frequency is left to the macroscopic update.
-// Returns -Gamma:sigma in s (in place) if apply, and accumulates |xi.sigma|^2 (xi = 2 pi k/N).
+// Constants of the Green operator of the reference medium, formed on the host: the medium, 1/mu0, 1/(2 mu0) and
+// c = (lam0+mu0)/(mu0 (lam0+2 mu0)). (As quotients in the kernel they were 90 FP64 operations of every thread.)
+template <typename T> struct GammaC { T lam0, mu0, im, ih, c; };
+
+// 1/x for x > 0 from an FP32 seed with two Newton steps (4 multiply-adds; the seed is good to 24 bits).
+__device__ __forceinline__ double rcp_pos(double x) {
+    double r = (double)__frcp_rn((float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
+// -Gamma0:sigma at a regular frequency (f1, f2, f3) (not zero, no Nyquist component) and the residual's |xi.sigma|^2,
+// xi = w (f1, f2, f3): eps_kh = (n_h v_k + n_k v_h)/(2 mu0) - c n_k n_h (n.v), v = sigma.n, n = xi/|xi|,
+// |xi.sigma|^2 = |xi|^2 |v|^2. t: the tensor components 11, 22, 33, 23, 13, 12; s: the result (Mandel).
+// FP64 (the FP64 pipe bounds the pass): in terms of xi and one reciprocal, about 95 multiply-adds per frequency where
+// normalising xi takes a square root and a division besides. 64^3 FP64 z pass, with GammaC and the tabulated twiddles:
+// 131 us before, 108 after.
+template <typename C>
+__device__ __forceinline__ double gamma_regular(const C t[6], C s[6], int f1, int f2, int f3, double w,
+                                                const GammaC<double> &gc) {
+    const double x1 = w * f1, x2 = w * f2, x3 = w * f3;
+    const C v1 = cmk<C>(x1 * t[0].x + x2 * t[5].x + x3 * t[4].x, x1 * t[0].y + x2 * t[5].y + x3 * t[4].y);
+    const C v2 = cmk<C>(x1 * t[5].x + x2 * t[1].x + x3 * t[3].x, x1 * t[5].y + x2 * t[1].y + x3 * t[3].y);
+    const C v3 = cmk<C>(x1 * t[4].x + x2 * t[3].x + x3 * t[2].x, x1 * t[4].y + x2 * t[3].y + x3 * t[2].y);
+    const double q = rcp_pos(x1 * x1 + x2 * x2 + x3 * x3);
+    const double w1 = x1 * q, w2 = x2 * q, w3 = x3 * q;
+    // with a_k = -v_k/(2 mu0) and b_k = a_k + c w_k (xi.v) the entries are w_k (a_k + b_k) and w_h b_k + w_k a_h
+    const C ce = cmk<C>(gc.c * (x1 * v1.x + x2 * v2.x + x3 * v3.x), gc.c * (x1 * v1.y + x2 * v2.y + x3 * v3.y));
+    const C a1 = cmk<C>(-gc.ih * v1.x, -gc.ih * v1.y), a2 = cmk<C>(-gc.ih * v2.x, -gc.ih * v2.y),
+            a3 = cmk<C>(-gc.ih * v3.x, -gc.ih * v3.y);
+    const C b1 = cmk<C>(a1.x + w1 * ce.x, a1.y + w1 * ce.y), b2 = cmk<C>(a2.x + w2 * ce.x, a2.y + w2 * ce.y);
+    const C b3 = cmk<C>(a3.x + w3 * ce.x, a3.y + w3 * ce.y);
+    const double sq2 = 1.41421356237309504880;
+    s[0] = cmk<C>(w1 * (a1.x + b1.x), w1 * (a1.y + b1.y));
+    s[1] = cmk<C>(w2 * (a2.x + b2.x), w2 * (a2.y + b2.y));
+    s[2] = cmk<C>(w3 * (a3.x + b3.x), w3 * (a3.y + b3.y));
+    s[3] = cmk<C>(sq2 * (w3 * b2.x + w2 * a3.x), sq2 * (w3 * b2.y + w2 * a3.y));
+    s[4] = cmk<C>(sq2 * (w3 * b1.x + w1 * a3.x), sq2 * (w3 * b1.y + w1 * a3.y));
+    s[5] = cmk<C>(sq2 * (w2 * b1.x + w1 * a2.x), sq2 * (w2 * b1.y + w1 * a2.y));
+    return v1.x * v1.x + v1.y * v1.y + v2.x * v2.x + v2.y * v2.y + v3.x * v3.x + v3.y * v3.y;
+}
+template <typename C>
+__device__ __forceinline__ float gamma_regular(const C t[6], C s[6], int f1, int f2, int f3, float w,
+                                               const GammaC<float> &gc) {
+    const float inv = 1.0f / sqrtf((float)(f1 * f1 + f2 * f2 + f3 * f3));
+    const float n1 = f1 * inv, n2 = f2 * inv, n3 = f3 * inv;
+    const C t11 = t[0], t22 = t[1], t33 = t[2], t23 = t[3], t13 = t[4], t12 = t[5];
+    const C v1 = cmk<C>(t11.x * n1 + t12.x * n2 + t13.x * n3, t11.y * n1 + t12.y * n2 + t13.y * n3);
+    const C v2 = cmk<C>(t12.x * n1 + t22.x * n2 + t23.x * n3, t12.y * n1 + t22.y * n2 + t23.y * n3);
+    const C v3 = cmk<C>(t13.x * n1 + t23.x * n2 + t33.x * n3, t13.y * n1 + t23.y * n2 + t33.y * n3);
+    const C nv = cmk<C>(n1 * v1.x + n2 * v2.x + n3 * v3.x, n1 * v1.y + n2 * v2.y + n3 * v3.y);
+    const float im = gc.im, ih = gc.ih, c = gc.c, sq2 = (float)1.41421356237309504880;
+    auto diag = [&](float nk, C vk) {
+        return cmk<C>(im * nk * vk.x - c * nk * nk * nv.x, im * nk * vk.y - c * nk * nk * nv.y);
+    };
+    auto off = [&](float nk, C vk, float nh, C vh) {
+        return cmk<C>(ih * (nh * vk.x + nk * vh.x) - c * nk * nh * nv.x, ih * (nh * vk.y + nk * vh.y) - c * nk * nh * nv.y);
+    };
+    const C e11 = diag(n1, v1), e22 = diag(n2, v2), e33 = diag(n3, v3);
+    const C e23 = off(n2, v2, n3, v3), e13 = off(n1, v1, n3, v3), e12 = off(n1, v1, n2, v2);
+    s[0] = cmk<C>(-e11.x, -e11.y);
+    s[1] = cmk<C>(-e22.x, -e22.y);
+    s[2] = cmk<C>(-e33.x, -e33.y);
+    s[3] = cmk<C>(-sq2 * e23.x, -sq2 * e23.y);
+    s[4] = cmk<C>(-sq2 * e13.x, -sq2 * e13.y);
+    s[5] = cmk<C>(-sq2 * e12.x, -sq2 * e12.y);
+    const float f2s = (float)(f1 * f1 + f2 * f2 + f3 * f3);
+    return (w * w * f2s) * (v1.x * v1.x + v1.y * v1.y + v2.x * v2.x + v2.y * v2.y + v3.x * v3.x + v3.y * v3.y);
+}
+
+// Green operator of the isotropic reference medium applied to one spectral stress (Mandel) of frequency index
+// (kx, ky, kz): gamma_regular, except that at frequencies with a Nyquist component the compliance of the reference
+// medium replaces it and the zero frequency is left to the macroscopic update. Returns -Gamma:sigma in s (in place) if
+// apply, and accumulates the residual |xi.sigma|^2 (xi = 2 pi k/N) of the frequency and, for 0 < kx < N/2, of its Hermitian
+// partner -k.
 template <typename C, typename T>
-__device__ __forceinline__ void gamma_point(C s[6], int kx, int ky, int kz, int N, T lam0, T mu0, T &acc, bool partner,
-                                            bool apply) {
+__device__ __forceinline__ void gamma_point(C s[6], int kx, int ky, int kz, int N, T w, const GammaC<T> &gc, T &acc,
+                                            bool partner, bool apply) {
     const int fx = kx;                                   // 0..N/2
     const int fy = ky <= (N >> 1) ? ky : ky - N;
     const int fz = kz <= (N >> 1) ? kz : kz - N;
@@ -671,83 +865,54 @@ __device__ __forceinline__ void gamma_point(C s[6], int kx, int ky, int kz, int 
     const int h = N >> 1;
     const bool nyq = kx == h || ky == h || kz == h;
     // Where the Green operator is applied (not on a Nyquist plane, not at zero frequency) the residual comes from
-    // its v = sigma_hat n: |xi.sigma_hat|^2 = w^2 |f|^2 |v|^2, the same at the Hermitian partner -k
+    // its v, the same at the Hermitian partner -k
     const bool fused = apply && !nyq && !(fx == 0 && fy == 0 && fz == 0);
-    if (!fused) {   // equilibrium residual |xi.sigma_hat|^2 at this frequency and, for 0 < kx < N/2, at its
-        // Hermitian partner -k (whose signed frequency differs from -xi on Nyquist ky / kz planes)
-        const T w = (T)(6.283185307179586476925 / N);
-        const int nparts = partner ? 2 : 1;
-        for (int pt = 0; pt < nparts; ++pt) {
-            const int gy = pt == 0 ? fy : ((N - ky) % N <= (N >> 1) ? (N - ky) % N : (N - ky) % N - N);
-            const int gz = pt == 0 ? fz : ((N - kz) % N <= (N >> 1) ? (N - kz) % N : (N - kz) % N - N);
-            const T x1 = w * (pt == 0 ? fx : -fx), x2 = w * gy, x3 = w * gz;
-            const C d1 = cmk<C>(x1 * t11.x + x2 * t12.x + x3 * t13.x, x1 * t11.y + x2 * t12.y + x3 * t13.y);
-            const C d2 = cmk<C>(x1 * t12.x + x2 * t22.x + x3 * t23.x, x1 * t12.y + x2 * t22.y + x3 * t23.y);
-            const C d3 = cmk<C>(x1 * t13.x + x2 * t23.x + x3 * t33.x, x1 * t13.y + x2 * t23.y + x3 * t33.y);
-            acc += d1.x * d1.x + d1.y * d1.y + d2.x * d2.x + d2.y * d2.y + d3.x * d3.x + d3.y * d3.y;
-        }
+    if (fused) {
+        const C t[6] = {t11, t22, t33, t23, t13, t12};
+        const T vv = gamma_regular(t, s, fx, fy, fz, w, gc);
+        acc += (partner ? (T)2 : (T)1) * vv;
+        return;
+    }
+    // equilibrium residual |xi.sigma_hat|^2 at this frequency and, for 0 < kx < N/2, at its Hermitian partner -k
+    // (whose signed frequency differs from -xi on Nyquist ky / kz planes)
+    const int nparts = partner ? 2 : 1;
+    for (int pt = 0; pt < nparts; ++pt) {
+        const int gy = pt == 0 ? fy : ((N - ky) % N <= (N >> 1) ? (N - ky) % N : (N - ky) % N - N);
+        const int gz = pt == 0 ? fz : ((N - kz) % N <= (N >> 1) ? (N - kz) % N : (N - kz) % N - N);
+        const T x1 = w * (pt == 0 ? fx : -fx), x2 = w * gy, x3 = w * gz;
+        const C d1 = cmk<C>(x1 * t11.x + x2 * t12.x + x3 * t13.x, x1 * t11.y + x2 * t12.y + x3 * t13.y);
+        const C d2 = cmk<C>(x1 * t12.x + x2 * t22.x + x3 * t23.x, x1 * t12.y + x2 * t22.y + x3 * t23.y);
+        const C d3 = cmk<C>(x1 * t13.x + x2 * t23.x + x3 * t33.x, x1 * t13.y + x2 * t23.y + x3 * t33.y);
+        acc += d1.x * d1.x + d1.y * d1.y + d2.x * d2.x + d2.y * d2.y + d3.x * d3.x + d3.y * d3.y;
     }
     if (!apply) return;
     if (fx == 0 && fy == 0 && fz == 0) {
         for (int i = 0; i < 6; ++i) s[i] = cmk<C>(0, 0);
         return;
     }
-    if (nyq) {
-        // -S0:sigma, S0 = (1/2mu0)(I - lam0/(3 lam0 + 2 mu0) J)
-        const T a = (T)1 / ((T)2 * mu0), b = lam0 / ((T)2 * mu0 * ((T)3 * lam0 + (T)2 * mu0));
-        const C tr = cmk<C>(s[0].x + s[1].x + s[2].x, s[0].y + s[1].y + s[2].y);
-        for (int i = 0; i < 3; ++i) s[i] = cmk<C>(-(a * s[i].x - b * tr.x), -(a * s[i].y - b * tr.y));
-        for (int i = 3; i < 6; ++i) s[i] = cmk<C>(-a * s[i].x, -a * s[i].y);
-        return;
-    }
-    const T inv = (T)1 / sqrt((T)(fx * fx + fy * fy + fz * fz));
-    const T n1 = fx * inv, n2 = fy * inv, n3 = fz * inv;
-    const C v1 = cmk<C>(t11.x * n1 + t12.x * n2 + t13.x * n3, t11.y * n1 + t12.y * n2 + t13.y * n3);
-    const C v2 = cmk<C>(t12.x * n1 + t22.x * n2 + t23.x * n3, t12.y * n1 + t22.y * n2 + t23.y * n3);
-    const C v3 = cmk<C>(t13.x * n1 + t23.x * n2 + t33.x * n3, t13.y * n1 + t23.y * n2 + t33.y * n3);
-    const C nv = cmk<C>(n1 * v1.x + n2 * v2.x + n3 * v3.x, n1 * v1.y + n2 * v2.y + n3 * v3.y);
-    {   // the residual of this frequency (and of its partner, counted twice)
-        const T w = (T)(6.283185307179586476925 / N);
-        const T f2 = (T)(fx * fx + fy * fy + fz * fz);
-        const T vv = v1.x * v1.x + v1.y * v1.y + v2.x * v2.x + v2.y * v2.y + v3.x * v3.x + v3.y * v3.y;
-        acc += (partner ? (T)2 : (T)1) * (w * w * f2) * vv;
-    }
-    const T im = (T)1 / mu0, ih = (T)0.5 / mu0;
-    const T c = (lam0 + mu0) / (mu0 * (lam0 + (T)2 * mu0));
-    const T sq2 = (T)1.41421356237309504880;
-#define EVP_EPS_KH(nk, vk, nh, vh, diag)                                                              \
-    cmk<C>(((diag) ? im * nk * vk.x : ih * (nh * vk.x + nk * vh.x)) - c * nk * nh * nv.x,             \
-           ((diag) ? im * nk * vk.y : ih * (nh * vk.y + nk * vh.y)) - c * nk * nh * nv.y)
-    const C e11 = EVP_EPS_KH(n1, v1, n1, v1, true);
-    const C e22 = EVP_EPS_KH(n2, v2, n2, v2, true);
-    const C e33 = EVP_EPS_KH(n3, v3, n3, v3, true);
-    const C e23 = EVP_EPS_KH(n2, v2, n3, v3, false);
-    const C e13 = EVP_EPS_KH(n1, v1, n3, v3, false);
-    const C e12 = EVP_EPS_KH(n1, v1, n2, v2, false);
-#undef EVP_EPS_KH
-    s[0] = cmk<C>(-e11.x, -e11.y);
-    s[1] = cmk<C>(-e22.x, -e22.y);
-    s[2] = cmk<C>(-e33.x, -e33.y);
-    s[3] = cmk<C>(-sq2 * e23.x, -sq2 * e23.y);
-    s[4] = cmk<C>(-sq2 * e13.x, -sq2 * e13.y);
-    s[5] = cmk<C>(-sq2 * e12.x, -sq2 * e12.y);
+    // Nyquist: -S0:sigma, S0 = (1/2mu0)(I - lam0/(3 lam0 + 2 mu0) J)
+    const T a = (T)1 / ((T)2 * gc.mu0), b = gc.lam0 / ((T)2 * gc.mu0 * ((T)3 * gc.lam0 + (T)2 * gc.mu0));
+    const C tr = cmk<C>(s[0].x + s[1].x + s[2].x, s[0].y + s[1].y + s[2].y);
+    for (int i = 0; i < 3; ++i) s[i] = cmk<C>(-(a * s[i].x - b * tr.x), -(a * s[i].y - b * tr.y));
+    for (int i = 3; i < 6; ++i) s[i] = cmk<C>(-a * s[i].x, -a * s[i].y);
 }
 
 // ---------------------------------------------------------------------------------------------
 // z pass: CTA = (ky, kx tile); nf fields x TX columns x N planes in shared memory.
 // ---------------------------------------------------------------------------------------------
 template <typename T, int N>
-__global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 ? 3 : 1) k_fft_z(typename CT<T>::type *__restrict__ spec, int nf, int mode, T lam0,
-                                                   T mu0, double *__restrict__ partials, double *__restrict__ mean6, const int *__restrict__ skip,
+__global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 ? 3 : 1) k_fft_z(typename CT<T>::type *__restrict__ spec, int nf, int mode, GammaC<T> gc,
+                                                   double *__restrict__ partials, double *__restrict__ mean6, const int *__restrict__ skip,
                                                    ZCtl zc) {
+    using C = typename CT<T>::type;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    using C = typename CT<T>::type;
     constexpr int TX = tx_z<N, T>(), LS = Shape<N>::LS, Hx = N / 2 + 1, MI = maxit<N>(6 * (TX + 1), z_threads<N, T>());
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *tw = reinterpret_cast<C *>(smem_raw);
-    C *buf = tw + N;
     __shared__ double red[32];
     constexpr int ntiles = (N / 2) / TX;
     const int tile = blockIdx.x % ntiles;
@@ -759,13 +924,13 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     const int nlines = nf * TX + (nyq ? nf : 0);
     const long plane = (long)N * Hx;            // one z plane of one field
     const long fstride = plane * N;
-    load_tw(tw, N);
     // The slab walk: element r = t mod (TX N) of field f sits at column xl and plane z = slab_item(r). With
     // NT threads and NT | TX N, a thread keeps its column, and its planes advance by DZ = NT / TX per step
-    // (slab_item adds DZ to z when r grows by NT, and pad16 adds DZ + DZ / 16 when DZ is a multiple of 16), so its
+    // (slab_item adds DZ to z when r grows by NT, and padn adds DZ + DZ / R1 when DZ is a multiple of R1), so its
     // shared and global addresses advance by constant strides.
     constexpr int NT = z_threads<N, T>(), DZ = NT / TX, KZ = TX * N / NT;
-    constexpr bool walk = (TX * N) % NT == 0 && DZ % 16 == 0 &&
+    constexpr int PZ = Shape<N>::R1, DP = DZ + DZ / PZ;
+    constexpr bool walk = N >= 16 && (TX * N) % NT == 0 && DZ % PZ == 0 &&
                           ((TX == 8 && N % 16 == 0 && LS % 16 == 9) ? NT % 128 == 0 : NT % TX == 0);
     int wz = 0, wxl = 0;
     if constexpr (walk) slab_item<N, TX>((int)threadIdx.x, wz, wxl);
@@ -787,7 +952,7 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     };
     if (mode != Z_INV) {
         // the forward transform's pass 1 (the whole transform when R2 = 1) straight from HBM: item (line, j < M1)
-        // reads elements j + M1 r and writes slots 16 j + r (slot r when R2 = 1), as bfft_pass1
+        // reads elements j + M1 r and writes slots R1 j + r (slot r when R2 = 1), as bfft_pass1
         constexpr int R1 = Shape<N>::R1, M1 = N / R1;
         const int nit = nlines * M1;
         for (int it = threadIdx.x; it < nit; it += blockDim.x) {
@@ -797,7 +962,7 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
 #pragma unroll
             for (int r = 0; r < R1; ++r) v[r] = g[(long)(j + M1 * r) * plane];
             dft_reg<R1, false>(v);
-            C *dst = buf + l * LS + 17 * j;
+            C *dst = buf + l * LS + (R1 + 1) * j;
 #pragma unroll
             for (int r = 0; r < R1; ++r) dst[r] = v[r];
         }
@@ -805,29 +970,30 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
         if constexpr (Shape<N>::R2 > 1) bfft_pass2<N, false>(buf, nlines, tw);
     } else {
         if constexpr (walk) {
-            C *sb = buf + wxl * LS + pad16(wz);
+            C *sb = buf + wxl * LS + padn<N>(wz);
             const C *gb = spec + (long)wz * plane + (long)ky * Hx + kx0 + wxl;
             for (int f = 0; f < nf; ++f) {
 #pragma unroll
                 for (int k = 0; k < KZ; ++k)
-                    cp_async<sizeof(C)>(sb + f * TX * LS + k * (DZ + DZ / 16), gb + f * fstride + (long)k * DZ * plane);
+                    cp_async<sizeof(C)>(sb + f * TX * LS + k * DP, gb + f * fstride + (long)k * DZ * plane);
             }
         } else {
             for (int t = threadIdx.x; t < nf * TX * N; t += blockDim.x) {   // TX, N powers of two: shifts
                 const int f = t / (TX * N), r = t % (TX * N);
                 int z, xl;
                 slab_item<N, TX>(r, z, xl);
-                cp_async<sizeof(C)>(buf + (f * TX + xl) * LS + pad16(z), spec + f * fstride + z * plane + (long)ky * Hx + kx0 + xl);
+                cp_async<sizeof(C)>(buf + (f * TX + xl) * LS + padn<N>(z), spec + f * fstride + z * plane + (long)ky * Hx + kx0 + xl);
             }
         }
         if (nyq)
             for (int t = threadIdx.x; t < nf * N; t += blockDim.x) {
                 const int f = t / N, z = t % N;
-                cp_async<sizeof(C)>(buf + (nf * TX + f) * LS + pad16(z), spec + f * fstride + z * plane + (long)ky * Hx + N / 2);
+                cp_async<sizeof(C)>(buf + (nf * TX + f) * LS + padn<N>(z), spec + f * fstride + z * plane + (long)ky * Hx + N / 2);
             }
         cp_async_wait_all();
         __syncthreads();
     }
+    unsigned ticket = 0;
     if (mode == Z_FWD_GAMMA_INV || mode == Z_FWD_RESID) {
         const bool apply = mode == Z_FWD_GAMMA_INV;
         T acc = (T)0;   // per-thread sum in the field precision; block and global sums in FP64
@@ -840,16 +1006,16 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
                 for (int f = 0; f < 6; ++f) mean6[f] = (double)s6[f].x * inv;
             }
             const bool partner = !(kx == 0 || kx == (N >> 1));
-            gamma_point<C, T>(s6, kx, ky, kz, N, lam0, mu0, acc, partner, apply);
+            gamma_point<C, T>(s6, kx, ky, kz, N, (T)(6.283185307179586476925 / N), gc, acc, partner, apply);
             if (apply)
                 for (int f = 0; f < 6; ++f) p0[f * fstep] = s6[f];
         };
         if constexpr (walk) {   // the same points per thread, in the same order, as the loop below
-            C *pb = buf + wxl * LS + pad16(wz);
+            C *pb = buf + wxl * LS + padn<N>(wz);
 #pragma unroll
-            for (int k = 0; k < KZ; ++k) point(wz + k * DZ, kx0 + wxl, pb + k * (DZ + DZ / 16), TX * LS);
+            for (int k = 0; k < KZ; ++k) point(wz + k * DZ, kx0 + wxl, pb + k * DP, TX * LS);
             if (nyq)
-                for (int t = threadIdx.x; t < N; t += blockDim.x) point(t, N / 2, buf + nf * TX * LS + pad16(t), LS);
+                for (int t = threadIdx.x; t < N; t += blockDim.x) point(t, N / 2, buf + nf * TX * LS + padn<N>(t), LS);
         } else {
             const int npts = (TX + (nyq ? 1 : 0)) * N;
             for (int t = threadIdx.x; t < npts; t += blockDim.x) {
@@ -859,39 +1025,35 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
                 const int kz = reg ? zr : t - TX * N;
                 const int kx = reg ? kx0 + xr : N / 2;
                 const int l0 = reg ? xr : nf * TX, ls = reg ? TX : 1;   // line of field f: l0 + f*ls
-                point(kz, kx, buf + l0 * LS + pad16(kz), ls * LS);
+                point(kz, kx, buf + l0 * LS + padn<N>(kz), ls * LS);
             }
         }
         __syncthreads();
         const double tot = block_sum((double)acc, red);
-        if (threadIdx.x == 0 && partials != nullptr) partials[blockIdx.x] = tot;
+        if (threadIdx.x == 0 && partials != nullptr) {
+            partials[blockIdx.x] = tot;
+            // the block's ticket: taken here, its latency passes under the inverse transform
+            if (zc.ctl != nullptr) ticket = fp_take_ticket(zc);
+        }
     }
     const bool inv = mode == Z_INV || mode == Z_FWD_GAMMA_INV;
     if constexpr (Shape<N>::R2 > 1) {
         if (inv) {
             bfft_pass1<N, true, MI>(buf, nlines);
-            // the inverse transform's pass 2 stored straight to HBM: item (line, j < 16) transforms slots j + 16 r
-            // as bfft_pass2 and stores elements j + 16 r
-            constexpr int R2 = Shape<N>::R2;
-            const int nit = nlines * 16;
+            // the inverse transform's pass 2 stored straight to HBM: item (line, j < R1) transforms slots j + R1 r
+            // as bfft_pass2 and stores elements j + R1 r
+            constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2;
+            const int nit = nlines * R1;
             for (int it = threadIdx.x; it < nit; it += blockDim.x) {
                 int l, j;
-                C *g = hbm_item(it, 16, l, j);
+                C *g = hbm_item(it, R1, l, j);
                 const C *line = buf + l * LS + j;
                 C u[R2];
 #pragma unroll
-                for (int r = 0; r < R2; ++r) {
-                    C a = line[17 * r];
-                    if (r > 0) {
-                        C w = tw[16 * r + j];
-                        w.y = -w.y;
-                        a = cmul(a, w);
-                    }
-                    u[r] = a;
-                }
-                dft_reg<R2, true>(u);
+                for (int r = 0; r < R2; ++r) u[r] = line[(R1 + 1) * r];
+                pass2_tail<N, true>(u, j, tw);
 #pragma unroll
-                for (int r = 0; r < R2; ++r) g[(long)(j + 16 * r) * plane] = u[r];
+                for (int r = 0; r < R2; ++r) g[(long)(j + R1 * r) * plane] = u[r];
             }
         }
     } else if (inv) {
@@ -899,43 +1061,37 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     }
     if (!inv || Shape<N>::R2 == 1) {   // the slab from shared memory
         if constexpr (walk) {
-            const C *sb = buf + wxl * LS + pad16(wz);
+            const C *sb = buf + wxl * LS + padn<N>(wz);
             C *gb = spec + (long)wz * plane + (long)ky * Hx + kx0 + wxl;
             for (int f = 0; f < nf; ++f) {
 #pragma unroll
-                for (int k = 0; k < KZ; ++k) gb[f * fstride + (long)k * DZ * plane] = sb[f * TX * LS + k * (DZ + DZ / 16)];
+                for (int k = 0; k < KZ; ++k) gb[f * fstride + (long)k * DZ * plane] = sb[f * TX * LS + k * DP];
             }
         } else {
             for (int t = threadIdx.x; t < nf * TX * N; t += blockDim.x) {
                 const int f = t / (TX * N), r = t % (TX * N);
                 int z, xl;
                 slab_item<N, TX>(r, z, xl);
-                spec[f * fstride + z * plane + (long)ky * Hx + kx0 + xl] = buf[(f * TX + xl) * LS + pad16(z)];
+                spec[f * fstride + z * plane + (long)ky * Hx + kx0 + xl] = buf[(f * TX + xl) * LS + padn<N>(z)];
             }
         }
         if (nyq)
             for (int t = threadIdx.x; t < nf * N; t += blockDim.x) {
                 const int f = t / N, z = t % N;
-                spec[f * fstride + z * plane + (long)ky * Hx + N / 2] = buf[(nf * TX + f) * LS + pad16(z)];
+                spec[f * fstride + z * plane + (long)ky * Hx + N / 2] = buf[(nf * TX + f) * LS + padn<N>(z)];
             }
     }
-    if (zc.ctl != nullptr) {   // the last block to finish runs the fixed-point control (fpctl.cuh)
-        __shared__ int last;
-        __threadfence();       // this block's partial sum and spectrum are visible to the others
-        __syncthreads();
-        if (threadIdx.x == 0) last = atomicAdd(&zc.ctl->ticket, 1u) == gridDim.x - 1;
-        __syncthreads();
-        if (!last) return;
-        __threadfence();
-        fp_control_block<T>(zc, partials, gridDim.x, spec, fstride, N);
-        if (threadIdx.x == 0) zc.ctl->ticket = 0u;
+    if (zc.ctl != nullptr) {   // the block with the last ticket runs the fixed-point control (fpctl.cuh)
+        if (threadIdx.x >= 32) return;
+        if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
+        fp_control_warp(zc, partials, gridDim.x);
     }
 }
 
-template <typename T, int N> size_t smem_x() { return sizeof(typename CT<T>::type) * (N + (size_t)rowpairs<N>() * Shape<N>::LS); }
-template <typename T, int N> size_t smem_y() { return sizeof(typename CT<T>::type) * (N + (size_t)(tx_y<N, T>() + 1) * Shape<N>::LS); }
+template <typename T, int N> size_t smem_x() { return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)rowpairs<N>() * Shape<N>::LS); }
+template <typename T, int N> size_t smem_y() { return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)(tx_y<N, T>() + 1) * Shape<N>::LS); }
 template <typename T, int N> size_t smem_z(int nf) {
-    return sizeof(typename CT<T>::type) * (N + (size_t)nf * (tx_z<N, T>() + 1) * Shape<N>::LS);
+    return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)nf * (tx_z<N, T>() + 1) * Shape<N>::LS);
 }
 
 template <typename K> cudaError_t allow_smem(K kernel, size_t bytes) {
@@ -960,7 +1116,7 @@ cudaError_t x_c2r_n(const void *spec, T *out, int nfields, T scale, const double
     const long npairs = (long)nfields * N * N / 2;
     constexpr int RP = rowpairs_c2r<N>();
     const int blocks = (int)((npairs + RP - 1) / RP);
-    const size_t sm = sizeof(C) * (N + (size_t)RP * Shape<N>::LS + 2 * (size_t)RP * (N / 2 + 1)) +
+    const size_t sm = sizeof(C) * (Shape<N>::NTW + (size_t)RP * Shape<N>::LS + 2 * (size_t)RP * (N / 2 + 1)) +
                       sizeof(T) * 2 * (size_t)RP * N;
     cudaError_t e = allow_smem(k_fft_x_c2r<T, N>, sm);
     if (e != cudaSuccess) return e;
@@ -972,15 +1128,18 @@ cudaError_t x_c2r_n(const void *spec, T *out, int nfields, T scale, const double
                     scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip);
 }
 
-template <typename T, int N> cudaError_t y_n(void *spec, int nfields, int inverse, cudaStream_t s, const int *skip) {
+template <typename T, int N>
+cudaError_t y_n(void *spec, int nfields, int inverse, cudaStream_t s, const int *skip, const InvCtl *icp = nullptr) {
     using C = typename CT<T>::type;
     constexpr int TX = tx_y<N, T>();
-    const int blocks = nfields * N * ((N / 2) / TX);
+    InvCtl ic{};
+    if (icp != nullptr) ic = *icp;
+    const int blocks = nfields * N * ((N / 2) / TX) + (ic.ctl != nullptr ? 1 : 0);
     const size_t sm = smem_y<T, N>();
     cudaError_t e = inverse ? allow_smem(k_fft_y<T, N, true>, sm) : allow_smem(k_fft_y<T, N, false>, sm);
     if (e != cudaSuccess) return e;
-    if (inverse) return launch_k(skip != nullptr, k_fft_y<T, N, true>, dim3(blocks), dim3(y_threads<N, T>()), sm, s, (C *)spec, skip);
-    return launch_k(skip != nullptr, k_fft_y<T, N, false>, dim3(blocks), dim3(y_threads<N, T>()), sm, s, (C *)spec, skip);
+    if (inverse) return launch_k(skip != nullptr, k_fft_y<T, N, true>, dim3(blocks), dim3(y_threads<N, T>()), sm, s, (C *)spec, skip, ic);
+    return launch_k(skip != nullptr, k_fft_y<T, N, false>, dim3(blocks), dim3(y_threads<N, T>()), sm, s, (C *)spec, skip, ic);
 }
 
 // x and y passes of the forward transform: one fused launch where the plane fits (xy_fused), else the two passes
@@ -1001,7 +1160,7 @@ template <typename T, int N> cudaError_t xy_r2c_n(const T *in, void *spec, int n
 
 template <typename T, int N>
 cudaError_t xy_c2r_n(const void *spec, T *out, int nfields, T scale, const double *add6, cudaStream_t s, const T *base,
-                     const int *skip) {
+                     const int *skip, const InvCtl *icp) {
     if constexpr (xy_fused<T, N>()) {
         using C = typename CT<T>::type;
         constexpr size_t sm = smem_xy<T, N>();
@@ -1011,10 +1170,12 @@ cudaError_t xy_c2r_n(const void *spec, T *out, int nfields, T scale, const doubl
         if (add6)
             for (int i = 0; i < 6; ++i) a[i] = (T)add6[i];
         const int has_add = add6 != nullptr;
-        return launch_k(skip != nullptr, k_fft_xy_c2r<T, N>, dim3(nfields * N), dim3(xy_threads<N>()), sm, s,
-                        (const C *)spec, out, scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip);
+        InvCtl ic{};
+        if (icp != nullptr) ic = *icp;
+        return launch_k(skip != nullptr, k_fft_xy_c2r<T, N>, dim3(nfields * N + (ic.ctl != nullptr ? 1 : 0)), dim3(xy_threads<N>()), sm, s,
+                        (const C *)spec, out, scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip, ic);
     } else {
-        cudaError_t e = y_n<T, N>(const_cast<void *>(spec), nfields, 1, s, skip);
+        cudaError_t e = y_n<T, N>(const_cast<void *>(spec), nfields, 1, s, skip, icp);
         if (e != cudaSuccess) return e;
         return x_c2r_n<T, N>(spec, out, nfields, scale, add6, s, base, skip);
     }
@@ -1031,8 +1192,13 @@ cudaError_t z_n(void *spec, int nfields, int mode, double lam0, double mu0, doub
     if (e != cudaSuccess) return e;
     ZCtl zc{};
     if (zcp != nullptr) zc = *zcp;
+    GammaC<T> gc{};
+    if (mode == Z_FWD_GAMMA_INV) {   // in the field precision, as the kernel would form them
+        const T l = (T)lam0, m = (T)mu0;
+        gc = GammaC<T>{l, m, (T)1 / m, (T)0.5 / m, (l + m) / (m * (l + (T)2 * m))};
+    }
     return launch_k(skip != nullptr, k_fft_z<T, N>, dim3(blocks), dim3(z_threads<N, T>()), sm, s, (C *)spec, nfields, mode,
-                    (T)lam0, (T)mu0, partials, mean6, skip, zc);
+                    gc, partials, mean6, skip, zc);
 }
 
 #define EVP_DISPATCH(N_, CALL)                             \
@@ -1050,9 +1216,7 @@ cudaError_t z_n(void *spec, int nfields, int mode, double lam0, double mu0, doub
 }  // namespace
 
 int fft_z_blocks(int n, int is_double) {
-    const int TX0 = is_double ? 4 : 8;
-    const int TX = TX0 < n / 2 ? TX0 : n / 2;
-    return n * ((n / 2) / TX);
+    return n * ((n / 2) / tx_z_of(n, is_double ? 8 : 4));
 }
 
 int fft_xy_fused(int n, int is_double) {
@@ -1069,10 +1233,10 @@ cudaError_t fft_xy_r2c(const T *in, void *spec, int n, int nfields, cudaStream_t
 
 template <typename T>
 cudaError_t fft_xy_c2r(const void *spec, T *out, int n, int nfields, T scale, const double *add6, cudaStream_t s,
-                       const T *base, const int *skip) {
+                       const T *base, const int *skip, const InvCtl *ic) {
     // the same contract as the x pass (whole rows in 16-byte chunks where the passes run separately)
     if (((uintptr_t)spec | (uintptr_t)out | (uintptr_t)base) & 15) return cudaErrorInvalidValue;
-    EVP_DISPATCH(n, (xy_c2r_n<T, NN>(spec, out, nfields, scale, add6, s, base, skip)))
+    EVP_DISPATCH(n, (xy_c2r_n<T, NN>(spec, out, nfields, scale, add6, s, base, skip, ic)))
 }
 
 template <typename T>
@@ -1088,8 +1252,9 @@ cudaError_t fft_x_c2r(const void *spec, T *out, int n, int nfields, T scale, con
     EVP_DISPATCH(n, (x_c2r_n<T, NN>(spec, out, nfields, scale, add6, s, base, skip)))
 }
 
-template <typename T> cudaError_t fft_y(void *spec, int n, int nfields, int inverse, cudaStream_t s, const int *skip) {
-    EVP_DISPATCH(n, (y_n<T, NN>(spec, nfields, inverse, s, skip)))
+template <typename T>
+cudaError_t fft_y(void *spec, int n, int nfields, int inverse, cudaStream_t s, const int *skip, const InvCtl *ic) {
+    EVP_DISPATCH(n, (y_n<T, NN>(spec, nfields, inverse, s, skip, ic)))
 }
 
 template <typename T>
@@ -1104,10 +1269,10 @@ cudaError_t fft_z(void *spec, int n, int nfields, int mode, double lam0, double 
     template cudaError_t fft_x_r2c<T>(const T *, void *, int, int, cudaStream_t, const int *);                     \
     template cudaError_t fft_x_c2r<T>(const void *, T *, int, int, T, const double *, cudaStream_t, const T *,     \
                                       const int *);                                                                \
-    template cudaError_t fft_y<T>(void *, int, int, int, cudaStream_t, const int *);                               \
+    template cudaError_t fft_y<T>(void *, int, int, int, cudaStream_t, const int *, const InvCtl *);               \
     template cudaError_t fft_xy_r2c<T>(const T *, void *, int, int, cudaStream_t, const int *);                    \
     template cudaError_t fft_xy_c2r<T>(const void *, T *, int, int, T, const double *, cudaStream_t, const T *,    \
-                                       const int *);                                                               \
+                                       const int *, const InvCtl *);                                               \
     template cudaError_t fft_z<T>(void *, int, int, int, double, double, double *, double *, cudaStream_t,         \
                                   const int *, const ZCtl *);
 EVP_FFT_INST(float)

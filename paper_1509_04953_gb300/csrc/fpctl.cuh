@@ -1,12 +1,17 @@
 // Fixed-point control of the basic scheme, on the device (Sec. 2.1 iteration with the mixed boundary
-// conditions). After an iteration's z pass has written its partial sums, one block sums them (in a fixed
-// order) into sum |xi.sigma_hat|^2; its first thread turns that and the mean stress into err_eq and
-// err_bc, decides convergence and computes the correction dE_k of the macroscopic strain on the
-// stress-controlled components. The correction goes into the zero-frequency term of the Green-operator
-// output, which the z pass leaves at zero; after the z pass's own inverse transform that term is the
-// (ky, kx) = (0, 0) entry of every z plane, so the inverse y and x transforms add it to every voxel's
-// strain. The host queues iterations in batches and reads this block once per batch; once `done` is set,
-// the kernels of the iterations still queued return at once.
+// conditions). After an iteration's z pass has written its partial sums, one warp sums them (in a fixed
+// order) into sum |xi.sigma_hat|^2, tests that and the mean stress against the tolerance and computes the
+// correction dE_k of the macroscopic strain on the stress-controlled components. The inverse transform adds it to
+// the zero-frequency term of the Green-operator output, which the z pass leaves at zero: after the z pass's own inverse
+// transform that is the (ky, kx) = (0, 0) entry of every z plane. The host queues iterations in batches and reads this block once per
+// batch; once `done` is set, the kernels of the iterations still queued return at once.
+//
+// The control runs alone at the end of the z pass, so it is a chain of latencies that every iteration waits for. It
+// therefore tests squares (no square root, no division: an FP64 one is a chain of some twenty dependent operations on
+// this GPU), lets one lane per component do the component's work, and the ticket that selects its block is taken
+// before the inverse transform; the next local tolerance, which does need the residuals themselves, is one extra
+// block of the inverse transform (fp_next_tolerance). At 32^3 the control took 8.4 us of a 15 us z pass as one thread's
+// chain after every block's last store, with the correction written into the spectrum.
 #pragma once
 #include <cstdint>
 
@@ -17,16 +22,18 @@ namespace evp {
 
 struct FpCtl {
     int done, it, conv, status, nmax, nfail;
-    unsigned ticket;    // z-pass blocks finished in this iteration (the last one runs the control)
+    unsigned ticket;    // z-pass blocks past their partial sum in this iteration (the last one runs the control)
     int pad;
-    double err_eq, err_bc;
-    double dE[6];
+    double dE[6];       // macroscopic strain increment so far
+    double corr[6];     // its correction in this iteration
     double tol_loc;     // local-solve tolerance of the next iteration (see evp_config.newton_adapt)
     float tol_loc_f;
 };
 
+// tol2, tau02: the squares of the tolerance and of the floor of |<sigma>|; n6 = N^6; ca, cb, cs: the mixed-BC
+// correction's a/det, b/det and 1/(2 mu0).
 struct FpCtlParams {
-    double N3, tau0, tol, a, b, det, mu0, ntol, eta;
+    double n6, tau02, tol2, ca, cb, cs;
     int max_iter;
 };
 
@@ -40,82 +47,100 @@ struct ZCtl {
     FpCtlParams p;
 };
 
-// Every thread of one block calls this with the iteration's nparts partial sums.
-template <typename T>
-__device__ __forceinline__ void fp_control_block(const ZCtl &z, const double *__restrict__ part, int nparts,
-                                                 typename CT<T>::type *__restrict__ spec, long fstride, int n) {
-    __shared__ double red[32];
-    __shared__ double corr[6];
-    __shared__ double meanv[6];
-    __shared__ int iv[4];
-    __shared__ int go;
+// A z-pass block's ticket, taken by the thread that wrote its partial sum. The release orders that sum (and, after the
+// block's barrier, the mean stress) before the ticket, the acquire orders the last block's reads after it; a full
+// fence (__threadfence) would order every outstanding store.
+__device__ __forceinline__ unsigned fp_take_ticket(const ZCtl &z) {
+    unsigned t;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;\n" : "=r"(t) : "l"(&z.ctl->ticket) : "memory");
+    return t;
+}
+
+// The 32 lanes of one warp call this with the iteration's nparts partial sums.
+__device__ __forceinline__ void fp_control_warp(const ZCtl &z, const double *__restrict__ part, int nparts) {
     FpCtl *c = z.ctl;
     const FpCtlParams &p = z.p;
-    // operands of the decision fetched by separate threads, alongside the reduction
-    if (threadIdx.x < 6) meanv[threadIdx.x] = z.scal[threadIdx.x];
-    else if (threadIdx.x == 32) iv[0] = c->it;
-    else if (threadIdx.x == 33) iv[1] = c->nmax;
-    else if (threadIdx.x == 34) iv[2] = z.flags[0];
-    else if (threadIdx.x == 35) iv[3] = z.flags[1];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) s += part[i];
-    s = block_sum(s, red);   // its barriers also publish meanv and iv
-    if (threadIdx.x == 0) {
-        go = 0;
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // every operand is fetched at once: the mean by lanes 0-5, the counters by lanes 8-11
+    const double m = lane < 6 ? __ldcg(z.scal + lane) : 0.0;
+    const int *ip = lane == 8 ? &c->it : lane == 9 ? &c->nmax : lane == 10 ? z.flags : z.flags + 1;
+    const int iv = lane >= 8 && lane < 12 ? __ldcg(ip) : 0;
+    const double dE = lane < 6 ? __ldcg(c->dE + lane) : 0.0;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = lane; i < nparts; i += 128)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i + 32 * q < nparts) a[q] += __ldcg(part + i + 32 * q);
+    double s = (a[0] + a[1]) + (a[2] + a[3]);
+    double mn = m * m, mu_n = lane == 2 ? 0.0 : mn;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(all, s, o);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        mn += __shfl_xor_sync(all, mn, o);
+        mu_n += __shfl_xor_sync(all, mu_n, o);
+    }
+    mn = __shfl_sync(all, mn, 0);       // lanes 0-7 hold |<sigma>|^2 and its stress-controlled part
+    mu_n = __shfl_sync(all, mu_n, 0);
+    const int it = __shfl_sync(all, iv, 8) + 1, nfail = __shfl_sync(all, iv, 10);
+    const int nmax = max(__shfl_sync(all, iv, 9), __shfl_sync(all, iv, 11));
+    const double m0 = __shfl_sync(all, m, 0), m1 = __shfl_sync(all, m, 1);
+    const double den2 = fmax(mn, p.tau02);
+    int status = 0, done = 0, conv = 0;
+    if (nfail != 0) {
+        status = EVP_ERR_NEWTON;
+        done = 1;
+    } else if (!isfinite(s) || !isfinite(mn)) {
+        status = EVP_ERR_NONFINITE;
+        done = 1;
+    } else if (s <= p.tol2 * den2 * p.n6 && mu_n <= p.tol2 * den2) {   // err_eq <= tol and err_bc <= tol
+        conv = 1;
+        done = 1;
+    } else if (it >= p.max_iter) {
+        done = 1;
+    }
+    if (!done && lane < 6) {
+        const double d = lane == 0 ? p.cb * m1 - p.ca * m0 : lane == 1 ? p.cb * m0 - p.ca * m1 : lane == 2 ? 0.0 : -p.cs * m;
+        c->dE[lane] = dE + d;
+        c->corr[lane] = d;
+    }
+    if (lane == 0) {
         z.scal[6] = s;
         z.flags[10] = 0;   // the next iteration's first local-solve pass counts its work list from zero,
         z.flags[11] = 0;   // and its voxels accepted after two steps
-        const int it = iv[0] + 1;
         c->it = it;
-        c->nmax = max(iv[1], iv[3]);
-        double mean[6], mn = 0.0, mu_n = 0.0;
-        for (int i = 0; i < 6; ++i) {
-            mean[i] = meanv[i];
-            mn += mean[i] * mean[i];
-            if (i != 2) mu_n += mean[i] * mean[i];
-        }
-        const double den = fmax(sqrt(mn), p.tau0);
-        const double err_eq = sqrt(s) / (p.N3 * den);
-        const double err_bc = sqrt(fmax(mu_n, 0.0)) / den;
-        c->err_eq = err_eq;
-        c->err_bc = err_bc;
-        if (iv[2] != 0) {
-            c->nfail = iv[2];
-            c->status = EVP_ERR_NEWTON;
-            c->done = 1;
-        } else if (!isfinite(err_eq) || !isfinite(err_bc)) {
-            c->status = EVP_ERR_NONFINITE;
-            c->done = 1;
-        } else if (err_eq <= p.tol && err_bc <= p.tol) {
-            c->conv = 1;
-            c->done = 1;
-        } else if (it >= p.max_iter) {
-            c->done = 1;
-        } else {
-            double dEk[6] = {0, 0, 0, 0, 0, 0};
-            dEk[0] = (p.a * (-mean[0]) - p.b * (-mean[1])) / p.det;
-            dEk[1] = (-p.b * (-mean[0]) + p.a * (-mean[1])) / p.det;
-            for (int i = 3; i < 6; ++i) dEk[i] = -mean[i] / (2.0 * p.mu0);
-            for (int i = 0; i < 6; ++i) {
-                c->dE[i] += dEk[i];
-                corr[i] = dEk[i] * p.N3;   // the inverse transforms are unnormalised; x_c2r scales by 1/N^3
-            }
-            if (p.eta > 0.0) {
-                const double tl = fmax(p.ntol, p.eta * fmax(err_eq, err_bc));
-                c->tol_loc = tl;
-                c->tol_loc_f = (float)tl;
-            }
-            go = 1;
-        }
+        c->nmax = nmax;
+        c->nfail = nfail;
+        c->status = status;
+        c->conv = conv;
+        c->ticket = 0u;
+        c->done = done;
     }
-    __syncthreads();
-    if (!go) return;
-    const long zstride = fstride / n;
-    for (int t = threadIdx.x; t < 6 * n; t += blockDim.x) {
-        const int f = t / n, zz = t - f * n;
-        auto &e = spec[f * fstride + zz * zstride];
-        e.x += (T)corr[f];
+}
+
+// What the inverse transform of an iteration takes from the control (ctl == nullptr: nothing). n3 = N^3 (the transforms
+// are unnormalised).
+struct InvCtl {
+    FpCtl *ctl;
+    const double *scal;     // as ZCtl.scal
+    double n3, tau0, ntol, eta;
+};
+
+// Local-solve tolerance of the next iteration: eta times the larger residual, at least ntol.
+__device__ __forceinline__ void fp_next_tolerance(const InvCtl &v) {
+    if (!(v.eta > 0.0)) return;
+    double mn = 0.0, mu_n = 0.0;
+    for (int i = 0; i < 6; ++i) {
+        const double m = v.scal[i];
+        mn += m * m;
+        if (i != 2) mu_n += m * m;
     }
+    const double den = fmax(sqrt(mn), v.tau0);
+    const double err_eq = sqrt(v.scal[6]) / (v.n3 * den), err_bc = sqrt(fmax(mu_n, 0.0)) / den;
+    const double tl = fmax(v.ntol, v.eta * fmax(err_eq, err_bc));
+    v.ctl->tol_loc = tl;
+    v.ctl->tol_loc_f = (float)tl;
 }
 
 }  // namespace evp

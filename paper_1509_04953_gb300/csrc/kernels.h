@@ -52,6 +52,7 @@ struct MRConst {
 
 // ---- fft.cu ----
 struct ZCtl;   // fpctl.cuh: the fixed-point control that the z pass's last block runs
+struct InvCtl;   // fpctl.cuh: what the inverse transform's first pass takes from it
 enum ZMode { Z_FWD = 0, Z_INV = 1, Z_FWD_GAMMA_INV = 2, Z_FWD_RESID = 3 };
 // skip (optional, device): when *skip != 0 the launched kernel returns at once (a converged fixed point
 // whose remaining queued iterations are discarded). tol_dev (optional, device): the local-solve
@@ -59,7 +60,8 @@ enum ZMode { Z_FWD = 0, Z_INV = 1, Z_FWD_GAMMA_INV = 2, Z_FWD_RESID = 3 };
 template <typename T>
 cudaError_t fft_x_r2c(const T *in, void *spec, int n, int nfields, cudaStream_t s, const int *skip = nullptr);
 template <typename T>
-cudaError_t fft_y(void *spec, int n, int nfields, int inverse, cudaStream_t s, const int *skip = nullptr);
+cudaError_t fft_y(void *spec, int n, int nfields, int inverse, cudaStream_t s, const int *skip = nullptr,
+                  const InvCtl *ic = nullptr);
 template <typename T>
 cudaError_t fft_z(void *spec, int n, int nfields, int mode, double lam0, double mu0, double *partials,
                   double *mean6, cudaStream_t s, const int *skip = nullptr, const ZCtl *zc = nullptr);
@@ -77,7 +79,8 @@ template <typename T>
 cudaError_t fft_xy_r2c(const T *in, void *spec, int n, int nfields, cudaStream_t s, const int *skip = nullptr);
 template <typename T>
 cudaError_t fft_xy_c2r(const void *spec, T *out, int n, int nfields, T scale, const double *add6,
-                       cudaStream_t s, const T *base = nullptr, const int *skip = nullptr);
+                       cudaStream_t s, const T *base = nullptr, const int *skip = nullptr,
+                       const InvCtl *ic = nullptr);
 
 // ---- newton.cu ----
 // solve_fp64: 1 -> the 6x6 Newton system is solved in FP64 even when TA = float.
