@@ -390,7 +390,6 @@ __global__ void __launch_bounds__(kThreads, N >= 64 && N <= 128 ? (sizeof(T) == 
     C *buf = tw + Shape<N>::NTW;
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     constexpr int RP = rowpairs<N>(), LS = Shape<N>::LS, Hx = N / 2 + 1;
     const long p0 = (long)blockIdx.x * RP;
@@ -433,7 +432,6 @@ __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::ty
     C *buf = tw + Shape<N>::NTW;                          // RP packed lines
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     constexpr int RP = rowpairs_c2r<N>(), LS = Shape<N>::LS, Hx = N / 2 + 1;
     C *hs = buf + RP * LS;                    // 2 RP half-spectrum rows, row-major
@@ -505,7 +503,6 @@ k_fft_y(typename CT<T>::type *__restrict__ spec, const int *__restrict__ skip, I
     C *buf = tw + Shape<N>::NTW;
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     constexpr int TX = tx_y<N, T>(), LS = Shape<N>::LS, Hx = N / 2 + 1;
     if (INV && ic.ctl != nullptr && blockIdx.x == gridDim.x - 1) {   // as in k_fft_xy_c2r
@@ -660,7 +657,6 @@ k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, c
     C *buf = tw + Shape<N>::NTW;
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, NP = N / 2, KU = (Hx + 31) / 32, R2 = Shape<N>::R2;
     const T *src = in + (long)blockIdx.x * N * N;   // plane = field * N + z
@@ -719,7 +715,6 @@ k_fft_xy_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
     C *buf = tw + Shape<N>::NTW;
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, NP = N / 2, R2 = Shape<N>::R2;
     if (ic.ctl != nullptr && blockIdx.x == gridDim.x - 1) {   // an extra CTA prepares the next iteration's tolerance
@@ -910,7 +905,6 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     C *buf = tw + Shape<N>::NTW;
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     constexpr int TX = tx_z<N, T>(), LS = Shape<N>::LS, Hx = N / 2 + 1, MI = maxit<N>(6 * (TX + 1), z_threads<N, T>());
     __shared__ double red[32];

@@ -113,7 +113,6 @@ __global__ void __launch_bounds__(kThreads) k_newton(long N3, const TA *__restri
                                                     TA tol, int maxit, TA ls_free, int *__restrict__ flags, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     if (tol_dev != nullptr) tol = *tol_dev;   // local tolerance set on the device for this iteration
     const long v = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -215,7 +214,6 @@ __global__ void __launch_bounds__(kThreads) k_newton_df(long N3, const double *_
                                                        int maxit, int *__restrict__ flags, const int *__restrict__ skip,
     const double *__restrict__ tol_dev) {
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     if (tol_dev != nullptr) tol = *tol_dev;   // local tolerance set on the device for this iteration
     const long v = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -330,7 +328,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_newton_ch
                                                           TA ls_free, int force_refresh, int *__restrict__ flags, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     if (tol_dev != nullptr) tol = *tol_dev;   // local tolerance set on the device for this iteration
     const long v = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -384,7 +381,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? (TWO ? 7 : 8) : 1)
                                                          int32_t *__restrict__ wl, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     if (tol_dev != nullptr) tol = *tol_dev;   // local tolerance set on the device for this iteration
     const long v = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -492,7 +488,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_chord_res
     TA tol, int maxit, TA ls_free, int *__restrict__ flags, const int32_t *__restrict__ wl, const int *__restrict__ skip,
     const TA *__restrict__ tol_dev, MRPtr<TA> mrp) {
     pdl_wait();
-    pdl_trigger();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
     if (tol_dev != nullptr) tol = *tol_dev;   // local tolerance set on the device for this iteration
     const int count = *(volatile const int *)(flags + 10);
