@@ -216,7 +216,7 @@ size_t layout(const evp_config *c, evp_handle *h, char *base) {
     char *rmax = take(rb), *rmax2 = take(rb);
     char *partials = take(sizeof(double) * npart), *scal = take(sizeof(double) * 64);
     char *flags = take(sizeof(int32_t) * 16);
-    char *ctl = take(256);   // FpCtl
+    char *ctl = take(512);   // FpCtl or AlCtl
     char *blk_counts = take(sizeof(int32_t) * nb);
     char *blk_off = take(sizeof(int32_t) * nb + N3);   // offsets, then one mark byte per voxel
     char *count = take(sizeof(int32_t) * 4);
@@ -493,9 +493,10 @@ double vm_strain(const double e[6]) {
 
 // Augmented-Lagrangian iterations of one increment (after the predictor): see k_al_local.
 // Returns a status; fills the iteration count, residuals, mean stress and the macro strain increment.
-static_assert(sizeof(FpCtl) <= 256, "FpCtl must fit its workspace slot");
+static_assert(sizeof(FpCtl) <= 512 && sizeof(AlCtl) <= 512, "FpCtl must fit its workspace slot");
 constexpr int kFpBatch = 16;   // iterations queued between host reads of the control block
 const double kZero6[6] = {0, 0, 0, 0, 0, 0};
+constexpr int kAlBatch = 8;    // the same for the augmented Lagrangian, which takes a quarter of the iterations
 constexpr int kTwoStepIters = 40;   // iterations of an increment whose first local-solve pass takes two chord steps
 
 // The x and y passes of the fixed point's transforms, forward and inverse: one launch each where the (field, z)
@@ -527,7 +528,7 @@ cudaError_t inv_xy(evp_handle *h, T *out, T scale, const double *add6, const T *
         if (e != cudaSuccess) return e;
     }
     PROF(5, 1);
-    return fft_x_c2r<T>(h->spec, out, h->n, 6, scale, add6, h->st, base, skip);
+    return fft_x_c2r<T>(h->spec, out, h->n, 6, scale, add6, h->st, base, skip, ic);
 }
 
 template <typename TA>
@@ -539,71 +540,74 @@ int al_loop(evp_handle *h, MatConst mc, double *dE, int *it_out, int *conv_out, 
     const double mu0 = muV / h->cfg.al_scale, lam0 = (lamV + 2.0 * muV / 3.0) - 2.0 * mu0 / 3.0;
     const double a = lam0 + 2.0 * mu0, b = lam0, det = a * a - b * b;
     const int solve64 = h->prec != EVP_MIXED_FAST;
-    const int nb = al_grid(N3, h->nsm, (int)sizeof(TA));
-    double hs[14];
-    int32_t hf[2];
-    int nmax = 0, conv = 0, it;
-    double ecmp = 0, elam = 0, ebc = 0;
     void *fac = h->cfg.newton_mode == EVP_NEWTON_REUSE ? h->fac : nullptr;
     // local tolerance: newton_tol, or with newton_adapt = eta > 0 loosened to max(newton_tol, eta err) while the
     // iteration is far from converged (err = the larger of the compatibility and multiplier residuals of the
     // previous iteration, 1e-2 before the first), as in the basic scheme
     const double ntol = h->cfg.newton_tol, eta = h->cfg.newton_adapt;
-    double tol_loc = eta > 0.0 ? std::fmax(ntol, eta * 1e-2) : ntol;
+    AlCtl hc{};
+    hc.tol_loc = eta > 0.0 ? std::fmax(ntol, eta * 1e-2) : ntol;
+    hc.tol_loc_f = (float)hc.tol_loc;
+    AlCtlParams p{};
+    p.inv_n3 = 1.0 / (double)N3;
+    p.tau0 = h->p.tau0;
+    p.tol = h->cfg.tol;
+    p.ntol = ntol;
+    p.eta = eta;
+    p.ca = a / det;
+    p.cb = b / det;
+    p.cs = 1.0 / (2.0 * mu0);
+    p.max_iter = h->cfg.max_iter;
+    for (int i = 0; i < 6; ++i) {
+        hc.dE[i] = dE[i];
+        p.E[i] = h->E[i];
+    }
+    AlCtl *dc = (AlCtl *)h->ctl;
+    const int *skip = &dc->done;
+    const TA *tol_dev;
+    if constexpr (sizeof(TA) == 4) tol_dev = &dc->tol_loc_f;
+    else tol_dev = &dc->tol_loc;
+    CK(cudaMemcpyAsync(dc, &hc, sizeof hc, cudaMemcpyHostToDevice, h->st));
     auto local = [&](int init, int refresh) -> int {
+        int nb = 0;
         { PROF(0, 1);
           CK(al_local<TA>(N3, (const TA *)h->epst, (const TA *)h->epse, (const TA *)h->tauc, h->g0, (TA *)h->sigk,
-                          (TA *)h->lam, (TA *)h->pal, local_tab<TA>(h, !init, lam0, mu0), mc,
-                          lam0, mu0, tol_loc, h->cfg.newton_max, solve64, init, h->flags, h->partials, fac,
-                          refresh, h->st, h->nsm, mr_ptr<TA>(h))); }
-        { PROF(6, 1); CK(reduce_partials(h->partials, nb, 14, h->scal + 24, h->st)); }
-        CK(cudaMemcpyAsync(hs, h->scal + 24, sizeof hs, cudaMemcpyDeviceToHost, h->st));
-        CK(cudaMemcpyAsync(hf, h->flags, sizeof hf, cudaMemcpyDeviceToHost, h->st));
-        CK(cudaStreamSynchronize(h->st));
-        if (h->prof) prof_collect(h);
-        nmax = hf[1] > nmax ? hf[1] : nmax;
-        if (hf[0] != 0) return fail(h, EVP_ERR_NEWTON, "local Newton failed in %d voxels", hf[0]);
+                          (TA *)h->lam, (TA *)h->pal, local_tab<TA>(h, !init, lam0, mu0), mc, lam0, mu0, hc.tol_loc,
+                          h->cfg.newton_max, solve64, init, h->flags, h->partials, fac, refresh, h->st, h->nsm,
+                          mr_ptr<TA>(h), skip, tol_dev, &nb)); }
+        { PROF(6, 1); CK(al_control(dc, h->partials, nb, h->flags, p, init, h->st)); }
         return EVP_OK;
     };
+    InvCtl ic{};
+    ic.dadd = dc->dE;
     int rc = local(1, 1);
-    if (rc) { *it_out = 0; *nmax_out = nmax; return rc; }
-    for (it = 1; it <= h->cfg.max_iter; ++it) {
-        // macroscopic strain on the stress-controlled components from <lam>
-        const double m0 = hs[2] / (double)N3, m1 = hs[3] / (double)N3;
-        double dEk[6] = {0, 0, 0, 0, 0, 0};
-        dEk[0] = (a * (-m0) - b * (-m1)) / det;
-        dEk[1] = (-b * (-m0) + a * (-m1)) / det;
-        for (int i = 3; i < 6; ++i) dEk[i] = -(hs[2 + i] / (double)N3) / (2.0 * mu0);
-        for (int i = 0; i < 6; ++i) dE[i] += dEk[i];
-        // compatibility: eps_tr = eps_e^t + dE + Gamma0 * (C0 de - lam)
-        CK(fwd_xy<TA>(h, (const TA *)h->pal));
-        { PROF(3, 1); CK(fft_z<TA>(h->spec, n, 6, Z_FWD_GAMMA_INV, lam0, mu0, nullptr, nullptr, h->st)); }
-        CK(inv_xy<TA>(h, (TA *)h->epst, (TA)(1.0 / (double)N3), dE, (const TA *)h->epse));
-        rc = local(0, it == 1);
-        if (rc) break;
-        double En = 0.0, mn = 0.0, mu_n = 0.0;
-        for (int i = 0; i < 6; ++i) {
-            const double Ei = h->E[i] + dE[i], mi = hs[2 + i] / (double)N3;
-            En += Ei * Ei;
-            mn += mi * mi;
-            if (i != 2) mu_n += mi * mi;
+    if (rc) return rc;
+    for (int queued = 0; queued < h->cfg.max_iter && !hc.done;) {
+        const int nb = std::min(kAlBatch, h->cfg.max_iter - queued);
+        for (int q = 0; q < nb; ++q, ++queued) {
+            // compatibility: eps_tr = eps_e^t + dE + Gamma0 * (C0 de - lam)
+            CK(fwd_xy<TA>(h, (const TA *)h->pal, skip));
+            { PROF(3, 1); CK(fft_z<TA>(h->spec, n, 6, Z_FWD_GAMMA_INV, lam0, mu0, nullptr, nullptr, h->st, skip)); }
+            CK(inv_xy<TA>(h, (TA *)h->epst, (TA)(1.0 / (double)N3), kZero6, (const TA *)h->epse, skip, &ic));
+            rc = local(0, queued == 0);
+            if (rc) return rc;
         }
-        const double den = std::fmax(std::sqrt(mn), h->p.tau0);
-        ecmp = std::sqrt(hs[0] / (double)N3) / std::fmax(std::sqrt(En), 1e-6);
-        elam = std::sqrt(hs[1] / (double)N3) / den;
-        ebc = std::sqrt(mu_n) / den;
-        if (!std::isfinite(ecmp) || !std::isfinite(elam)) { rc = fail(h, EVP_ERR_NONFINITE, "non-finite AL residual"); break; }
-        if (ecmp <= h->cfg.tol && elam <= h->cfg.tol && ebc <= h->cfg.tol && tol_loc <= ntol) { conv = 1; break; }
-        if (eta > 0.0) tol_loc = std::fmax(ntol, eta * std::fmax(ecmp, elam));
+        CK(cudaMemcpyAsync(&hc, dc, sizeof hc, cudaMemcpyDeviceToHost, h->st));
+        CK(cudaStreamSynchronize(h->st));
+        if (h->prof) prof_collect(h);
     }
-    if (it > h->cfg.max_iter) it = h->cfg.max_iter;
-    *it_out = it;
-    *conv_out = conv;
-    *nmax_out = nmax;
-    *err_eq = elam;
-    *err_bc = ebc;
-    for (int i = 0; i < 6; ++i) mean_sig[i] = hs[8 + i] / (double)N3;
-    return rc;
+    *it_out = hc.it;
+    *conv_out = hc.conv;
+    *nmax_out = hc.nmax;
+    *err_eq = hc.elam;
+    *err_bc = hc.ebc;
+    for (int i = 0; i < 6; ++i) {
+        dE[i] = hc.dE[i];
+        mean_sig[i] = hc.mean[i];
+    }
+    if (hc.status == EVP_ERR_NEWTON) return fail(h, EVP_ERR_NEWTON, "local Newton failed in %d voxels", hc.nfail);
+    if (hc.status == EVP_ERR_NONFINITE) return fail(h, EVP_ERR_NONFINITE, "non-finite AL residual");
+    return EVP_OK;
 }
 }  // namespace
 
@@ -912,7 +916,7 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
         zc.p.tol2 = h->cfg.tol * h->cfg.tol;
         zc.p.ca = a / det; zc.p.cb = b / det; zc.p.cs = 1.0 / (2.0 * mu0r);
         zc.p.max_iter = h->cfg.max_iter;
-        const InvCtl ic{dc, h->scal, (double)N3, h->p.tau0, ntol, h->cfg.newton_adapt};
+        const InvCtl ic{dc, h->scal, (double)N3, h->p.tau0, ntol, h->cfg.newton_adapt, nullptr};
         int queued = 0;
         while (true) {
             const int nb = std::min(kFpBatch, h->cfg.max_iter - queued);

@@ -425,7 +425,8 @@ template <int N> __host__ __device__ constexpr int rowpairs_c2r() { return rowpa
 template <typename T, int N>
 __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
                                                        long npairs, T scale, int has_add, T a0, T a1, T a2, T a3, T a4,
-                                                       T a5, const T *__restrict__ base, const int *__restrict__ skip) {
+                                                       T a5, const T *__restrict__ base, const int *__restrict__ skip,
+                                                       const double *__restrict__ dadd) {
     using C = typename CT<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tw = reinterpret_cast<C *>(smem_raw);
@@ -472,10 +473,10 @@ __global__ void __launch_bounds__(kThreads) k_fft_x_c2r(const typename CT<T>::ty
     // with the selection in the loop)
     auto add_of = [&](long row) -> T {
         const int f = (int)(row / ((long)N * N));
-        return f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
+        return dadd ? (T)dadd[f] : f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
     };
     constexpr bool one_field = (N * N) % (2 * RP) == 0;
-    const T add_cta = one_field ? add_of(2 * p0) : (T)0;
+    const T add_cta = one_field && has_add ? add_of(2 * p0) : (T)0;
     for (int t = threadIdx.x; t < np * N; t += blockDim.x) {
         const int pl = t / N, j = t - pl * N;
         const long row0 = 2 * (p0 + pl);
@@ -755,7 +756,7 @@ k_fft_xy_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
     T add = (T)0;
     if (has_add) {
         const int f = (int)(blockIdx.x / N);
-        add = f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
+        add = ic.dadd ? (T)ic.dadd[f] : f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
     }
     const T *bsrc = base ? base : out;
     for (int t = threadIdx.x; t < NP * N; t += blockDim.x) {
@@ -1105,7 +1106,7 @@ template <typename T, int N> cudaError_t x_r2c_n(const T *in, void *spec, int nf
 
 template <typename T, int N>
 cudaError_t x_c2r_n(const void *spec, T *out, int nfields, T scale, const double *add6, cudaStream_t s, const T *base,
-                    const int *skip) {
+                    const int *skip, const InvCtl *ic = nullptr) {
     using C = typename CT<T>::type;
     const long npairs = (long)nfields * N * N / 2;
     constexpr int RP = rowpairs_c2r<N>();
@@ -1119,7 +1120,7 @@ cudaError_t x_c2r_n(const void *spec, T *out, int nfields, T scale, const double
         for (int i = 0; i < 6; ++i) a[i] = (T)add6[i];
     const int has_add = add6 != nullptr;
     return launch_k(skip != nullptr, k_fft_x_c2r<T, N>, dim3(blocks), dim3(kThreads), sm, s, (const C *)spec, out, npairs,
-                    scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip);
+                    scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip, ic != nullptr ? ic->dadd : nullptr);
 }
 
 template <typename T, int N>
@@ -1171,7 +1172,7 @@ cudaError_t xy_c2r_n(const void *spec, T *out, int nfields, T scale, const doubl
     } else {
         cudaError_t e = y_n<T, N>(const_cast<void *>(spec), nfields, 1, s, skip, icp);
         if (e != cudaSuccess) return e;
-        return x_c2r_n<T, N>(spec, out, nfields, scale, add6, s, base, skip);
+        return x_c2r_n<T, N>(spec, out, nfields, scale, add6, s, base, skip, icp);
     }
 }
 
@@ -1240,10 +1241,10 @@ cudaError_t fft_x_r2c(const T *in, void *spec, int n, int nfields, cudaStream_t 
 
 template <typename T>
 cudaError_t fft_x_c2r(const void *spec, T *out, int n, int nfields, T scale, const double *add6, cudaStream_t s,
-                      const T *base, const int *skip) {
+                      const T *base, const int *skip, const InvCtl *ic) {
     // the pass copies whole rows in 16-byte chunks
     if (((uintptr_t)spec | (uintptr_t)out | (uintptr_t)base) & 15) return cudaErrorInvalidValue;
-    EVP_DISPATCH(n, (x_c2r_n<T, NN>(spec, out, nfields, scale, add6, s, base, skip)))
+    EVP_DISPATCH(n, (x_c2r_n<T, NN>(spec, out, nfields, scale, add6, s, base, skip, ic)))
 }
 
 template <typename T>
@@ -1262,7 +1263,7 @@ cudaError_t fft_z(void *spec, int n, int nfields, int mode, double lam0, double 
 #define EVP_FFT_INST(T)                                                                                            \
     template cudaError_t fft_x_r2c<T>(const T *, void *, int, int, cudaStream_t, const int *);                     \
     template cudaError_t fft_x_c2r<T>(const void *, T *, int, int, T, const double *, cudaStream_t, const T *,     \
-                                      const int *);                                                                \
+                                      const int *, const InvCtl *);                                                                \
     template cudaError_t fft_y<T>(void *, int, int, int, cudaStream_t, const int *, const InvCtl *);               \
     template cudaError_t fft_xy_r2c<T>(const T *, void *, int, int, cudaStream_t, const int *);                    \
     template cudaError_t fft_xy_c2r<T>(const void *, T *, int, int, T, const double *, cudaStream_t, const T *,    \

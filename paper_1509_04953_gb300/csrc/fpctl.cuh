@@ -119,12 +119,31 @@ __device__ __forceinline__ void fp_control_warp(const ZCtl &z, const double *__r
     }
 }
 
-// What the inverse transform of an iteration takes from the control (ctl == nullptr: nothing). n3 = N^3 (the transforms
-// are unnormalised).
+// Control block of the augmented-Lagrangian iteration (k_al_control) and its constants: the stopping tolerance, the
+// macroscopic strain at the start of the increment, ca, cb, cs as in FpCtlParams for its reference medium.
+struct AlCtl {
+    int done, it, conv, status, nmax, nfail;
+    double dE[6];           // macroscopic strain increment: of the last iteration that ran, or for the next
+    double mean[6];         // mean stress
+    double ecmp, elam, ebc; // residuals
+    double sum[14];         // the local step's sums (see k_al_local)
+    unsigned ticket;        // blocks of the control that have stored theirs
+    double tol_loc;         // local-solve tolerance of the next iteration
+    float tol_loc_f;
+};
+struct AlCtlParams {
+    double inv_n3, tau0, tol, ntol, eta, ca, cb, cs, E[6];
+    int max_iter;
+};
+
+// What the inverse transform of an iteration takes from the control: with ctl (basic scheme) the correction of the
+// zero-frequency term, n3 = N^3 times FpCtl.corr (the transforms are unnormalised); with dadd (augmented Lagrangian) the six
+// offsets of its last pass in device memory.
 struct InvCtl {
     FpCtl *ctl;
     const double *scal;     // as ZCtl.scal
     double n3, tau0, ntol, eta;
+    const double *dadd;
 };
 
 // Local-solve tolerance of the next iteration: eta times the larger residual, at least ntol.

@@ -66,10 +66,11 @@ template <typename T>
 cudaError_t fft_z(void *spec, int n, int nfields, int mode, double lam0, double mu0, double *partials,
                   double *mean6, cudaStream_t s, const int *skip = nullptr, const ZCtl *zc = nullptr);
 // x-pass complex-to-real. If add6 != nullptr: out[c] = (base ? base[c] : out[c]) + scale * field + add6[c];
-// else out = field.
+// the same with the offsets of ic->dadd if that is set; else out = field.
 template <typename T>
 cudaError_t fft_x_c2r(const void *spec, T *out, int n, int nfields, T scale, const double *add6,
-                      cudaStream_t s, const T *base = nullptr, const int *skip = nullptr);
+                      cudaStream_t s, const T *base = nullptr, const int *skip = nullptr,
+                      const InvCtl *ic = nullptr);
 int fft_z_blocks(int n, int is_double);
 // The x and y passes together: forward = fft_x_r2c then the forward y pass, inverse = the inverse y pass then
 // fft_x_c2r (same contract), with bitwise the same results. Where fft_xy_fused(n, is_double) is 1 each is one
@@ -105,15 +106,19 @@ cudaError_t newton_field_df(long N3, const double *epst, const double *tauc, con
                             LocalTab<double> tab, MatConst mc, double tol, int maxit, int *flags, cudaStream_t s,
                             const int *skip = nullptr,
                             const double *tol_dev = nullptr);
-// Augmented-Lagrangian local step (tab: the compliance S of the crystal with init, S + S0 without), grid-stride over al_grid(N3, nsm, sizeof(TA)) blocks; part: 14 doubles per
-// block. al_blocks(N3) bounds the block count (for sizing).
+// Augmented-Lagrangian local step (tab: the compliance S of the crystal with init, S + S0 without), grid-stride over
+// *nparts blocks (output), part: their 14 sums, [14][*nparts]. al_blocks(N3) bounds the block count (for sizing).
+// skip, tol_dev as in newton_field. al_control: see k_al_control.
+struct AlCtl;
+struct AlCtlParams;
 int al_blocks(long N3);
-int al_grid(long N3, int nsm, int tsize);
 template <typename TA>
 cudaError_t al_local(long N3, const TA *epst, const TA *epse, const TA *tauc, const int32_t *g0, TA *sig, TA *lam, TA *p,
                      LocalTab<TA> tab, MatConst mc, double lam0, double mu0, double tol,
                      int maxit, int solve_fp64, int init, int *flags, double *part, void *fac, int refresh,
-                     cudaStream_t s, int nsm, MRPtr<TA> mrp = MRPtr<TA>{});
+                     cudaStream_t s, int nsm, MRPtr<TA> mrp, const int *skip, const TA *tol_dev, int *nparts);
+cudaError_t al_control(AlCtl *ctl, const double *part, int nparts, const int32_t *flags, const AlCtlParams &p, int first,
+                       cudaStream_t s);
 template <typename TA>
 cudaError_t predictor(long N3, const TA *epse, const TA *deps, const TA *rho, TA *epst, TA *tauc, MatConst mc,
                       double r, const double *dE6, int use_field, cudaStream_t s);

@@ -14,6 +14,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "local.cuh"
+#include "fpctl.cuh"
 
 namespace evp {
 
@@ -569,38 +570,110 @@ template <typename T> __device__ __forceinline__ T iso_apply_c0(T l0, T m0, cons
     return (T)2 * m0 * x[i] + (i < 3 ? l0 * tr : (T)0);
 }
 
-// NV per-thread values summed over the block into part[0..NV): warp sums in the value type (a
-// five-level pairwise tree), then the warp sums in FP64. On the FP32 path this keeps the FP64 pipe
-// out of the per-voxel work; the result stays within a few FP32 roundings of the exact block sum.
-template <int NV, typename T> __device__ __forceinline__ void block_sums(const T (&v)[NV], double *sh, double *part) {
-    T w[NV];
+// Adds the warp's sums of 14 per-thread values to acc: lane l gets value l / 2 (lanes 28 .. 31 nothing). Pairwise trees in
+// the value type, the values split over the lanes as the tree descends (16 exchanges instead of 14 x 5), then one
+// FP64 addition per lane: with the sums in one lane it took 28 FP64-pipe instructions per warp of voxels, 97 us of
+// the FP64 pipe in a 128^3 step.
+template <typename T> __device__ __forceinline__ void warp_accumulate14(const T (&v)[14], double &acc) {
+    const int lane = threadIdx.x & 31;
+    T x[16];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        w[q] = v[q];
+    for (int q = 0; q < 16; ++q) x[q] = q < 14 ? v[q < 14 ? q : 0] : (T)0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) w[q] += __shfl_xor_sync(0xffffffffu, w[q], o);
+    for (int o = 16; o > 1; o >>= 1) {
+        const bool hi = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < o / 2) {   // this lane keeps o / 2 of its o values
+                const T send = hi ? x[i] : x[i + o / 2], keep = hi ? x[i + o / 2] : x[i];
+                x[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if (lane == 0)
+    x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+    acc += (double)x[0];
+}
+
+// What follows a voxel's local solve: sigma stored, the local strain, the multiplier update, the next transform's input
+// and the voxel's terms of the 14 sums. etr is the trial strain eps_tr' of the local problem.
+template <typename TA>
+__device__ __forceinline__ void al_update(long N3, long v, const TA et[6], const TA lm[6], const TA ee[6], const TA etr[6],
+                                          const TA sg[6], TA *__restrict__ sig, TA *__restrict__ lam,
+                                          TA *__restrict__ pout, TA l0, TA m0, TA sa, TA sb, TA sa_lo, TA sb_lo,
+                                          double sad, double sbd, int init, TA (&sums)[14]) {
+    // local strain e_tr = eps_tr' - S0 sigma and the gap d = eps_tr - e_tr to about twice the field
+    // precision: near convergence eps_tr and e_tr agree to many digits, and forming them in plain FP32
+    // leaves rounding noise in d (hence in the multiplier update) that keeps the iteration from
+    // settling. FP64 does it on the FP64 path; the FP32 path uses error-free transformations on the
+    // FP32 pipe (the FP64 pipe issues 1/64 as fast).
+    TA el[6], d[6], de[6];
+    if constexpr (sizeof(TA) == 4) {
+        float t1, e1, th, e2;
+        two_sum_f(sg[0], sg[1], t1, e1);
+        two_sum_f(t1, sg[2], th, e2);
+        const float tl = __fadd_rn(e1, e2);   // tr(sigma) = th + tl
 #pragma unroll
-        for (int q = 0; q < NV; ++q) sh[wid * NV + q] = (double)w[q];
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double t = 0.0;
-        for (int k = 0; k < nw; ++k) t += sh[k * NV + threadIdx.x];
-        part[threadIdx.x] = t;
+        for (int c = 0; c < 6; ++c) {
+            sig[c * N3 + v] = sg[c];
+            if (init) {
+                el[c] = et[c];
+                d[c] = 0.f;
+            } else {
+                float p, pe;
+                two_prod_f(sa, sg[c], p, pe);
+                pe = fmaf(sa_lo, sg[c], pe);   // S0 sigma (shear part) = p + pe
+                float sh = p, sl = pe;
+                if (c < 3) {
+                    float q, qe, se;
+                    two_prod_f(sb, th, q, qe);
+                    qe = fmaf(sb, tl, fmaf(sb_lo, th, qe));   // sb tr = q + qe
+                    two_sum_f(p, -q, sh, se);
+                    sl = __fadd_rn(se, __fsub_rn(pe, qe));
+                }
+                float u, ue, w, we;
+                two_sum_f(etr[c], -sh, u, ue);            // e_tr = u + ul
+                const float ul = __fsub_rn(ue, sl);
+                two_sum_f(et[c], -u, w, we);              // d = eps_tr - e_tr
+                d[c] = __fadd_rn(w, __fsub_rn(we, ul));
+                el[c] = __fadd_rn(u, ul);
+            }
+            de[c] = el[c] - ee[c];
+        }
+    } else {
+        double s6[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) s6[c] = (double)sg[c];
+        const double str = s6[0] + s6[1] + s6[2];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            sig[c * N3 + v] = sg[c];
+            const double eld = init ? (double)et[c] : (double)etr[c] - (sad * s6[c] - (c < 3 ? sbd * str : 0.0));
+            d[c] = (TA)((double)et[c] - eld);
+            el[c] = (TA)eld;
+            de[c] = el[c] - ee[c];
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const TA dl = iso_apply_c0(l0, m0, d, c);
+        const TA nl = init ? sg[c] : lm[c] + dl;
+        lam[c * N3 + v] = nl;
+        pout[c * N3 + v] = nl - iso_apply_c0(l0, m0, de, c);
+        sums[0] += d[c] * d[c];
+        sums[1] += dl * dl;
+        sums[2 + c] = nl;
+        sums[8 + c] = sg[c];
     }
 }
 
-// The warp's sums of NV per-thread values (a five-level pairwise tree in the value type), added in FP64 by
-// lane 0 to row[0..NV) (one row per warp: no other warp touches it, so no barrier).
-template <int NV, typename T> __device__ __forceinline__ void warp_accumulate(const T (&v)[NV], double *row) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        T w = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-        if ((threadIdx.x & 31) == 0) row[q] += (double)w;
+// The block's 14 sums from its lanes' (warp_accumulate14), one column per block in part. rows: 14 doubles per warp.
+__device__ __forceinline__ void al_store_sums(double acc, double *rows, double *__restrict__ part) {
+    const int lane = threadIdx.x & 31;
+    if ((lane & 1) == 0 && lane < 28) rows[(threadIdx.x >> 5) * 14 + (lane >> 1)] = acc;
+    __syncthreads();
+    if (threadIdx.x < 14) {
+        double t = 0.0;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += rows[k * 14 + threadIdx.x];
+        part[(long)threadIdx.x * gridDim.x + blockIdx.x] = t;
     }
 }
 
@@ -612,14 +685,16 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
                                                       TA sb, TA sa_lo, TA sb_lo, double sad, double sbd, TA tol,
                                                       int maxit, TA ls_free, int init,
                                                       int *__restrict__ flags, double *__restrict__ part,
-                                                      TS *__restrict__ fac, int refresh, MRPtr<TA> mrp) {
+                                                      TS *__restrict__ fac, int refresh, MRPtr<TA> mrp,
+                                                      const int *__restrict__ skip, const TA *__restrict__ tol_dev) {
+    pdl_wait();
+    if (skip != nullptr && *skip) return;   // the increment's iteration has ended
+    if (tol_dev != nullptr) tol = *tol_dev;
     constexpr int NV = 14;
     // grid-stride over tiles of blockDim voxels (block-uniform trip count): the block's warps run their tiles
-    // without waiting for one another; each warp sums its tile's values and lane 0 adds them, in FP64, to the
-    // warp's row of acc; the rows are summed once, at the end
-    __shared__ double acc[(kThreads / 32) * NV];
-    for (int i = threadIdx.x; i < (kThreads / 32) * NV; i += blockDim.x) acc[i] = 0.0;
-    __syncthreads();
+    // without waiting for one another, each adding its tile's sums to its lanes' FP64 accumulators
+    __shared__ double rows[(kThreads / 32) * NV];
+    double acc = 0.0;
     int t_fail = 0, t_mx = 0, t_it = 0, t_ev = 0;
     const long stride = (long)gridDim.x * blockDim.x;
     for (long v0 = (long)blockIdx.x * blockDim.x; v0 < N3; v0 += stride) {
@@ -671,69 +746,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
                 r = newton_voxel<TA, TF>(pb, el6, tauc[v], sg, mc, tol, maxit, ls_free, nev);
         }
         pb.leave(sg);
-        // local strain e_tr = eps_tr' - S0 sigma and the gap d = eps_tr - e_tr to about twice the field
-        // precision: near convergence eps_tr and e_tr agree to many digits, and forming them in plain FP32
-        // leaves rounding noise in d (hence in the multiplier update) that keeps the iteration from
-        // settling. FP64 does it on the FP64 path; the FP32 path uses error-free transformations on the
-        // FP32 pipe (the FP64 pipe issues 1/64 as fast).
-        TA el[6], d[6], de[6];
-        if constexpr (sizeof(TA) == 4) {
-            float t1, e1, th, e2;
-            two_sum_f(sg[0], sg[1], t1, e1);
-            two_sum_f(t1, sg[2], th, e2);
-            const float tl = __fadd_rn(e1, e2);   // tr(sigma) = th + tl
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                sig[c * N3 + v] = sg[c];
-                if (init) {
-                    el[c] = et[c];
-                    d[c] = 0.f;
-                } else {
-                    float p, pe;
-                    two_prod_f(sa, sg[c], p, pe);
-                    pe = fmaf(sa_lo, sg[c], pe);   // S0 sigma (shear part) = p + pe
-                    float sh = p, sl = pe;
-                    if (c < 3) {
-                        float q, qe, se;
-                        two_prod_f(sb, th, q, qe);
-                        qe = fmaf(sb, tl, fmaf(sb_lo, th, qe));   // sb tr = q + qe
-                        two_sum_f(p, -q, sh, se);
-                        sl = __fadd_rn(se, __fsub_rn(pe, qe));
-                    }
-                    float u, ue, w, we;
-                    two_sum_f(etr[c], -sh, u, ue);            // e_tr = u + ul
-                    const float ul = __fsub_rn(ue, sl);
-                    two_sum_f(et[c], -u, w, we);              // d = eps_tr - e_tr
-                    d[c] = __fadd_rn(w, __fsub_rn(we, ul));
-                    el[c] = __fadd_rn(u, ul);
-                }
-                de[c] = el[c] - ee[c];
-            }
-        } else {
-            double s6[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) s6[c] = (double)sg[c];
-            const double str = s6[0] + s6[1] + s6[2];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                sig[c * N3 + v] = sg[c];
-                const double eld = init ? (double)et[c] : (double)etr[c] - (sad * s6[c] - (c < 3 ? sbd * str : 0.0));
-                d[c] = (TA)((double)et[c] - eld);
-                el[c] = (TA)eld;
-                de[c] = el[c] - ee[c];
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const TA dl = iso_apply_c0(l0, m0, d, c);
-            const TA nl = init ? sg[c] : lm[c] + dl;
-            lam[c * N3 + v] = nl;
-            pout[c * N3 + v] = nl - iso_apply_c0(l0, m0, de, c);
-            sums[0] += d[c] * d[c];
-            sums[1] += dl * dl;
-            sums[2 + c] = nl;
-            sums[8 + c] = sg[c];
-        }
+        al_update<TA>(N3, v, et, lm, ee, etr, sg, sig, lam, pout, l0, m0, sa, sb, sa_lo, sb_lo, sad, sbd, init, sums);
     }
     if (valid) {
         const int its = r < 0 ? -r : r;
@@ -742,15 +755,265 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
         t_it += its;
         t_ev += nev;
     }
-    warp_accumulate<NV>(sums, acc + (threadIdx.x >> 5) * NV);
+    warp_accumulate14(sums, acc);
     }
     // flags as in k_newton
-    // (its barrier follows every warp's last acc update, so acc is complete after it)
     block_solve_stats(t_fail, t_mx, t_it, t_ev, 0, flags);
-    if (threadIdx.x < NV) {
-        double t = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += acc[k * NV + threadIdx.x];
-        part[NV * (long)blockIdx.x + threadIdx.x] = t;
+    al_store_sums(acc, rows, part);
+}
+
+// The augmented-Lagrangian step of the FP32 path with stored factors. A full solver in the loop takes 168 registers, so
+// 12 warps per SM: its loads (47 words a voxel, 71 with the Ma-Roters law) wait mostly uncovered. Here the loop holds
+// the chord iteration's common path only (full steps with the stored factors, as many as it takes, with
+// chord_voxel's operations in its order); a voxel that leaves it (a refresh or a backtracking step) is solved from
+// the start by al_solve_rest, out of line. Crystal tables and factors are read again at each step, from L1 and shared
+// memory, and the operands of the update after the solve, so 72 registers carry 28 warps per SM (local step per
+// increment at 4 / 5 / 6 / 7 / 8 CTAs of 128 threads: 7.25 / 6.7 / 6.43 / 6.38 / 6.48 ms at 128^3, and 3.79 / 3.49 / 3.53 /
+// 3.35 / 3.36 ms with the Ma-Roters law at 64^3). At 128^3 the step takes 122 us, 545 MB at 4.5 TB/s, where the full solver
+// took 270 (97 of them on the FP64 pipe for the sums, see warp_accumulate14); with Ma-Roters at 64^3 57 us, 83 before.
+constexpr int kAlCtas = 7;
+struct AlArgs {
+    long N3;
+    const float *epst, *epse, *tauc;
+    const int32_t *g0;
+    float *sig, *lam, *p;
+    LocalTab<float> tab;
+    MatConst mc;
+    float l0, m0, sa, sb, sa_lo, sb_lo, tol, ls_free;
+    double sad, sbd;
+    int maxit;
+    float *fac;
+    MRPtr<float> mrp;
+};
+__device__ __forceinline__ float ld_again(const float *p) {   // a load that is not merged with an earlier one
+    float x;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
+    return x;
+}
+template <bool MR, typename F> __device__ __forceinline__ auto with_law(const AlArgs &a, long v, float tc, F f) {
+    if constexpr (MR) return f(FlowMR<float>{a.mrp.tpi, a.N3, v, tc});
+    else return f(tc);
+}
+template <typename TF, bool MR>
+__device__ __noinline__ int al_solve_rest(const AlArgs &a, float tol, long v, const float etr[6], float sg[6], int &nev) {
+    Problem<float> pb;
+    pb.init(a.tab, a.g0[v]);
+    float F[21];
+    load_factors((const float *)a.fac, a.N3, v, F);
+    for (int c = 0; c < 6; ++c) sg[c] = a.sig[c * a.N3 + v];
+    int nref = 0;
+    const int r = with_law<MR>(a, v, a.tauc[v], [&](const auto &hf) {
+        return chord_voxel<float, float, TF>(pb, etr, hf, sg, a.mc, tol, a.maxit, a.ls_free, F, false, nev, nref);
+    });
+    if (nref) store_factors(a.fac, a.N3, v, F);
+    return r;
+}
+
+template <typename TF, bool MR>
+__global__ void __launch_bounds__(kThreads, kAlCtas) k_al_chord(const __grid_constant__ AlArgs a, int *__restrict__ flags,
+                                                          double *__restrict__ part, const int *__restrict__ skip,
+                                                          const float *__restrict__ tol_dev) {
+    pdl_wait();
+    if (skip != nullptr && *skip) return;   // the increment's iteration has ended
+    const float tol = tol_dev != nullptr ? *tol_dev : a.tol;
+    constexpr int NV = 14;
+    __shared__ double rows[(kThreads / 32) * NV];
+    __shared__ __align__(16) float fsh[21 * kThreads];
+    double acc = 0.0;
+    const long N3 = a.N3, stride = (long)gridDim.x * blockDim.x;
+    int t_fail = 0, t_mx = 0, t_it = 0, t_ev = 0;
+    for (long v0 = (long)blockIdx.x * blockDim.x; v0 < N3; v0 += stride) {
+        const long v = v0 + threadIdx.x;
+        const bool valid = v < N3;
+        float sums[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) sums[q] = 0.f;
+        if (valid) {
+            prefetch_factors((const float *)a.fac, N3, v, fsh);
+            int g = a.g0[v];
+            const float tc = a.tauc[v];
+            float etr[6], sg[6];
+            auto trial = [&](const float et[6], const float lm[6]) {
+                const float ltr = lm[0] + lm[1] + lm[2];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) etr[c] = et[c] + a.sa * lm[c] - (c < 3 ? a.sb * ltr : 0.f);
+            };
+            {
+                float et[6], lm[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    et[c] = a.epst[c * N3 + v];
+                    lm[c] = a.lam[c * N3 + v];
+                    sg[c] = a.sig[c * N3 + v];
+                }
+                trial(et, lm);
+            }
+            EvalR<float> e;
+            auto residual = [&](const float s[6]) {
+                asm volatile("" : "+r"(g));   // the tables are read again: nothing of them is held between steps
+                Problem<float> pb;
+                pb.init(a.tab, g);
+                with_law<MR>(a, v, tc, [&](const auto &hf) { evaluate_r(pb, etr, hf, drcp(tc), s, a.mc, e); });
+            };
+            residual(sg);
+            int r = 0, nev = 1;
+            float prev = -1.f;
+            for (int it = 1; r == 0; ++it) {
+                float d[6];
+                {
+                    float F[21];
+                    prefetched_factors(fsh, F);
+                    ldl_apply<float, float>(F, e.r, d);
+                }
+                float rd = 0.f, dn = 0.f, sn = 0.f;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    rd += e.r[i] * d[i];
+                    dn += d[i] * d[i];
+                    sn += sg[i] * sg[i];
+                }
+                dn = dsqrt(dn);
+                const float scale = dsqrt(sn) + tc;
+                if (dn <= tol * scale && rd >= 0.f) {
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) sg[i] -= d[i];
+                    r = it;
+                    break;
+                }
+                if (it >= a.maxit || rd <= 0.f || (prev > 0.f && dn > 0.25f * prev)) break;
+                const float phi0 = e.phi;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) sg[i] -= d[i];
+                residual(sg);
+                ++nev;
+                if (!(e.phi <= phi0 - 1e-4f * rd || dn <= a.ls_free * scale)) break;
+                if (dn <= tol * scale) r = it;
+                prev = dn;
+            }
+            if (r == 0) {   // off the common path
+                float s6[6], t6[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) t6[c] = etr[c];
+                r = al_solve_rest<TF, MR>(a, tol, v, t6, s6, nev);
+#pragma unroll
+                for (int c = 0; c < 6; ++c) sg[c] = s6[c];
+            }
+            {
+                float et[6], lm[6], ee[6];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    et[c] = ld_again(a.epst + c * N3 + v);
+                    lm[c] = ld_again(a.lam + c * N3 + v);
+                    ee[c] = a.epse[c * N3 + v];
+                }
+                trial(et, lm);
+                al_update<float>(N3, v, et, lm, ee, etr, sg, a.sig, a.lam, a.p, a.l0, a.m0, a.sa, a.sb, a.sa_lo, a.sb_lo,
+                                 a.sad, a.sbd, 0, sums);
+            }
+            const int its = r < 0 ? -r : r;
+            t_fail += r < 0;
+            t_mx = max(t_mx, its);
+            t_it += its;
+            t_ev += nev;
+        }
+        warp_accumulate14(sums, acc);
+    }
+    block_solve_stats(t_fail, t_mx, t_it, t_ev, 0, flags);
+    al_store_sums(acc, rows, part);
+}
+
+// Control of the augmented-Lagrangian iteration after each local step: block q adds up sum q of the step's blocks, in a
+// fixed order, and the last block to finish runs the stopping tests and, where the iteration goes on, forms the
+// macroscopic strain correction on the stress-controlled components from <lam> and the next local tolerance. The host
+// queues iterations in batches and reads the control block once per batch (a read after every iteration cost about 25 us
+// of a 145 us iteration at 64^3). One block per sum: 1000 partial sums of each are 900 FP64-pipe cycles of an SM.
+__global__ void __launch_bounds__(256) k_al_control(AlCtl *c, const double *__restrict__ part, int nparts,
+                                                    const int32_t *__restrict__ flags, AlCtlParams p, int first) {
+    pdl_wait();
+    __shared__ double red[32];
+    const int lane = threadIdx.x & 31;
+    // every operand is fetched at once: the partial sums, and by warp 0 the control block
+    const bool ended = c->done != 0;
+    double dEl = 0.0, tol_loc = 0.0;
+    int it = 0, nmax = 0, nfail = 0, mx = 0;
+    if (threadIdx.x < 32) {
+        dEl = lane < 6 ? c->dE[lane] : 0.0;
+        tol_loc = c->tol_loc;
+        it = c->it + (first ? 0 : 1);
+        nmax = c->nmax;
+        nfail = flags[0];
+        mx = flags[1];
+    }
+    double s = 0.0;
+    for (int i = threadIdx.x; i < nparts; i += 1024) {
+        double x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = i + 256 * q < nparts ? part[(long)blockIdx.x * nparts + i + 256 * q] : 0.0;
+        s += (x[0] + x[1]) + (x[2] + x[3]);
+    }
+    if (ended) return;
+    s = block_sum(s, red);
+    if (threadIdx.x >= 32) return;
+    unsigned ticket = 0;
+    if (lane == 0) {
+        c->sum[blockIdx.x] = s;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;\n" : "=r"(ticket) : "l"(&c->ticket) : "memory");
+    }
+    if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
+    const double hl = lane < 14 ? __ldcg(c->sum + lane) * p.inv_n3 : 0.0;   // the means
+    const unsigned all = 0xffffffffu;
+    // lanes 0-5: component i of |E|^2, |<lam>|^2 and its stress-controlled part, summed over lanes 0-7
+    const double mi = __shfl_sync(all, hl, 2 + (lane & 7)), sig = __shfl_sync(all, hl, 8 + (lane & 7));
+    const double Ei = lane < 6 ? p.E[lane] + dEl : 0.0, ml = lane < 6 ? mi : 0.0;
+    double En = Ei * Ei, mn = ml * ml, mu_n = lane == 2 ? 0.0 : mn;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        En += __shfl_xor_sync(all, En, o);
+        mn += __shfl_xor_sync(all, mn, o);
+        mu_n += __shfl_xor_sync(all, mu_n, o);
+    }
+    // lane 0: |<lam>|, 1: |E|, 2 and 3: the RMS gaps, 4: the stress-controlled |<lam>|; then lanes 0-2 their quotients
+    const double g0 = __shfl_sync(all, hl, 0), g1 = __shfl_sync(all, hl, 1);
+    const double root = sqrt(lane == 0 ? mn : lane == 1 ? En : lane == 2 ? g0 : lane == 3 ? g1 : mu_n);
+    const double den = fmax(__shfl_sync(all, root, 0), p.tau0), nE = fmax(__shfl_sync(all, root, 1), 1e-6);
+    const double q = __shfl_sync(all, root, 2 + (lane < 3 ? lane : 2)) / (lane == 0 ? nE : den);
+    const double ecmp = __shfl_sync(all, q, 0), elam = __shfl_sync(all, q, 1), ebc = __shfl_sync(all, q, 2);
+    const double m0 = __shfl_sync(all, mi, 0), m1 = __shfl_sync(all, mi, 1);
+    int status = 0, done = 0, conv = 0;
+    if (nfail != 0) {
+        status = EVP_ERR_NEWTON;
+        done = 1;
+    } else if (!first) {
+        if (!isfinite(ecmp) || !isfinite(elam)) {
+            status = EVP_ERR_NONFINITE;
+            done = 1;
+        } else if (ecmp <= p.tol && elam <= p.tol && ebc <= p.tol && tol_loc <= p.ntol) {
+            conv = 1;
+            done = 1;
+        } else if (it >= p.max_iter) {
+            done = 1;
+        }
+    }
+    if (lane < 6) {
+        c->mean[lane] = sig;
+        const double d = lane == 0 ? p.cb * m1 - p.ca * m0 : lane == 1 ? p.cb * m0 - p.ca * m1 : lane == 2 ? 0.0 : -p.cs * mi;
+        if (!done) c->dE[lane] = dEl + d;
+    }
+    if (lane == 0) {
+        c->it = it;
+        c->nmax = max(nmax, mx);
+        c->nfail = nfail;
+        c->status = status;
+        c->conv = conv;
+        c->ecmp = ecmp;
+        c->elam = elam;
+        c->ebc = ebc;
+        if (!done && !first && p.eta > 0.0) {
+            c->tol_loc = fmax(p.ntol, p.eta * fmax(ecmp, elam));
+            c->tol_loc_f = (float)c->tol_loc;
+        }
+        c->ticket = 0u;
+        c->done = done;
     }
 }
 
@@ -962,7 +1225,9 @@ cudaError_t newton_chord_field(long N3, const TA *epst, const TA *tauc, const in
 }
 
 int al_blocks(long N3) { return (int)((N3 + kThreads - 1) / kThreads); }
-int al_grid(long N3, int nsm, int tsize) { return std::min(al_blocks(N3), std::max(nsm, 1) * (tsize == 4 ? 3 : 2)); }
+int al_grid(long N3, int nsm, int tsize, int chord) {
+    return std::min(al_blocks(N3), std::max(nsm, 1) * (chord ? kAlCtas : tsize == 4 ? 3 : 2));
+}
 
 cudaError_t newton_field_df(long N3, const double *epst, const double *tauc, const int32_t *g0, double *sig,
                             LocalTab<double> tab, MatConst mc, double tol, int maxit, int *flags, cudaStream_t s, const int *skip,
@@ -973,29 +1238,46 @@ cudaError_t newton_field_df(long N3, const double *epst, const double *tauc, con
     return cudaGetLastError();
 }
 
+int al_chord(size_t tsize, const void *fac, int refresh) { return tsize == 4 && fac != nullptr && !refresh; }
+
+cudaError_t al_control(AlCtl *ctl, const double *part, int nparts, const int32_t *flags, const AlCtlParams &p, int first,
+                       cudaStream_t s) {
+    return launch_k(true, k_al_control, dim3(14), dim3(256), 0, s, ctl, part, nparts, flags, p, first);
+}
+
 template <typename TA>
 cudaError_t al_local(long N3, const TA *epst, const TA *epse, const TA *tauc, const int32_t *g0, TA *sig, TA *lam, TA *p,
                      LocalTab<TA> tab, MatConst mc, double lam0, double mu0, double tol,
                      int maxit, int solve_fp64, int init, int *flags, double *part, void *fac, int refresh,
-                     cudaStream_t s, int nsm, MRPtr<TA> mrp) {
-    const int blocks = al_grid(N3, nsm, (int)sizeof(TA));
+                     cudaStream_t s, int nsm, MRPtr<TA> mrp, const int *skip, const TA *tol_dev, int *nparts) {
+    const int chord = al_chord(sizeof(TA), fac, refresh);
+    const int blocks = *nparts = al_grid(N3, nsm, (int)sizeof(TA), chord);
     const double sad = 1.0 / (2.0 * mu0), sbd = lam0 / (2.0 * mu0 * (3.0 * lam0 + 2.0 * mu0));
     const TA sa = (TA)sad, sb = (TA)sbd;
     const TA sa_lo = (TA)(sad - (double)sa), sb_lo = (TA)(sbd - (double)sb);   // S0 = (sa + sa_lo) I - (sb + sb_lo) J
-    return by_law(mrp, [&](auto law) {
+    cudaError_t err = cudaSuccess;
+    by_law(mrp, [&](auto law) {
         constexpr bool MR = decltype(law)::value;
-        if (solve_fp64)
-            k_al_local<TA, TA, double, MR><<<blocks, kThreads, 0, s>>>(N3, epst, epse, tauc, g0, sig, lam, p, tab,
-                                                                       mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo,
-                                                                       sb_lo, sad, sbd, (TA)tol, maxit,
-                                                                       ls_free_of<TA>(), init, flags, part, (TA *)fac,
-                                                                       refresh, mrp);
-        else
-            k_al_local<TA, TA, TA, MR><<<blocks, kThreads, 0, s>>>(N3, epst, epse, tauc, g0, sig, lam, p, tab,
-                                                                   mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo, sb_lo,
-                                                                   sad, sbd, (TA)tol, maxit, ls_free_of<TA>(), init,
-                                                                   flags, part, (TA *)fac, refresh, mrp);
+        if constexpr (sizeof(TA) == 4) {
+            if (chord) {
+                const AlArgs a{N3, epst, epse, tauc, g0, sig, lam, p, tab, mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo, sb_lo,
+                               (TA)tol, ls_free_of<TA>(), sad, sbd, maxit, (TA *)fac, mrp};
+                err = solve_fp64 ? launch_k(true, k_al_chord<double, MR>, dim3(blocks), dim3(kThreads), 0, s, a, flags,
+                                            part, skip, tol_dev)
+                                 : launch_k(true, k_al_chord<float, MR>, dim3(blocks), dim3(kThreads), 0, s, a, flags,
+                                            part, skip, tol_dev);
+                return;
+            }
+        }
+        auto go = [&](auto kernel) {
+            err = launch_k(true, kernel, dim3(blocks), dim3(kThreads), 0, s, N3, epst, epse, tauc, g0, sig, lam, p, tab,
+                           mc, (TA)lam0, (TA)mu0, sa, sb, sa_lo, sb_lo, sad, sbd, (TA)tol, maxit, ls_free_of<TA>(), init,
+                           flags, part, (TA *)fac, refresh, mrp, skip, tol_dev);
+        };
+        if (solve_fp64) go(k_al_local<TA, TA, double, MR>);
+        else go(k_al_local<TA, TA, TA, MR>);
     });
+    return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 template <typename TA>
@@ -1031,7 +1313,8 @@ template <typename TA> cudaError_t total_strain(long N3, const TA *epse, const T
                                                 int32_t *, int, cudaStream_t, const int *, const TA *, MRPtr<TA>, int); \
     template cudaError_t al_local<TA>(long, const TA *, const TA *, const TA *, const int32_t *, TA *, TA *, TA *, \
                                       LocalTab<TA>, MatConst, double, double, double, int, int, \
-                                      int, int *, double *, void *, int, cudaStream_t, int, MRPtr<TA>);           \
+                                      int, int *, double *, void *, int, cudaStream_t, int, MRPtr<TA>, const int *, \
+                                      const TA *, int *);                                                        \
     template cudaError_t predictor<TA>(long, const TA *, const TA *, const TA *, TA *, TA *, MatConst, double,    \
                                        const double *, int, cudaStream_t);                                        \
     template cudaError_t state_update<TA>(long, const TA *, const TA *, const int32_t *, const TA *, TA *, TA *,  \
