@@ -1123,27 +1123,24 @@ int pf_step(evp_handle *h, int nsteps, pf_stats *out) {
     if (h->r == 2) { PROF(11, 1); CK(pf_interp(h->n, h->k, h->kpf, h->st)); }   // softened densities
     int32_t ovf = 0;
     if (out) {
-        const int nb = pf_stat_blocks(h->N3pf);
         // every id in use is below next_id: only those words of the id bitmap are cleared and counted
         const int words = std::min(h->bitmap_words, (h->next_id + 31) / 32);
         { PROF(12, 3);
         if (h->dbl)
             CK(pf_stats_launch<double>(h->npf, h->ids, (double *)h->eta, h->gpf, h->kpf, h->pc, h->bitmap, words,
-                                       h->partials, h->st));
+                                       h->rmax_bytes ? h->rmax : nullptr, h->partials, h->scal + 8, h->scal + 10, h->st));
         else
             CK(pf_stats_launch<float>(h->npf, h->ids, (float *)h->eta, h->gpf, h->kpf, h->pc, h->bitmap, words,
-                                      h->partials, h->st));
-        CK(reduce_partials(h->partials, nb, 2, h->scal + 8, h->st));
+                                      h->rmax_bytes ? h->rmax : nullptr, h->partials, h->scal + 8, h->scal + 10, h->st));
         }
-        double hs[2], ng = 0;
+        double hs[3];
         CK(cudaMemcpyAsync(hs, h->scal + 8, sizeof hs, cudaMemcpyDeviceToHost, h->st));
-        CK(cudaMemcpyAsync(&ng, h->partials + 2 * (long)nb, sizeof ng, cudaMemcpyDeviceToHost, h->st));
         CK(cudaMemcpyAsync(&ovf, h->flags + 2, sizeof ovf, cudaMemcpyDeviceToHost, h->st));
         CK(cudaStreamSynchronize(h->st));
         if (h->prof) prof_collect(h);
         out->F_tot = hs[0];
         out->X_rex = hs[1] / (double)h->N3pf;
-        out->n_grains = (int)ng;
+        out->n_grains = (int)hs[2];
         out->overflow = ovf;
     } else {
         CK(cudaMemcpyAsync(&ovf, h->flags + 2, sizeof ovf, cudaMemcpyDeviceToHost, h->st));

@@ -202,9 +202,12 @@ template <typename T>
 cudaError_t pf_restrict(int n, int K, const int32_t *ids, const T *eta, int32_t *g, cudaStream_t s);
 cudaError_t pf_init(int n, int r, int K, const int32_t *g0, int32_t *ids, void *eta, int32_t *ids2, void *eta2,
                     int eta_double, int32_t *gpf, cudaStream_t s);
+// Statistics of the active sets: out2 = (free energy, recrystallised points), ngrains = distinct grain ids. rcur: the row
+// bounds of (ids, eta), may be null. partials: 2 pf_stat_blocks(n^3) doubles of scratch.
 template <typename T>
 cudaError_t pf_stats_launch(int n, const int32_t *ids, const T *eta, const int32_t *g, const double *k, PFConst pc,
-                     uint32_t *bitmap, int bitmap_words, double *partials, cudaStream_t s);
+                     uint32_t *bitmap, int bitmap_words, const uint8_t *rcur, double *partials, double *out2, double *ngrains,
+                     cudaStream_t s);
 cudaError_t reduce_partials(const double *partials, int nparts, int nvals, double *out, cudaStream_t s,
                             const int *skip = nullptr);
 
