@@ -6,6 +6,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "powtab.cuh"
 
 namespace evp {
 
@@ -34,7 +35,7 @@ template <typename T> __device__ __forceinline__ T pow_nm1(T ax, const MatConst 
         }
         return r;
     }
-    return ax > (T)0 ? (T)pow((double)ax, mc.n - 1.0) : (T)0;
+    return ax > (T)0 ? (T)pow_tab((double)ax, mc.n - 1.0) : (T)0;
 }
 
 // Flow-rule constants in the arithmetic precision.

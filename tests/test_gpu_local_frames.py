@@ -19,7 +19,7 @@ def rel(a, b):
     return np.abs(np.asarray(a) - np.asarray(b)).max() / max(np.abs(np.asarray(b)).max(), 1e-300)
 
 
-@pytest.mark.parametrize("exponent", [10.0, 7.0, 4.5])
+@pytest.mark.parametrize("exponent", [10.0, 7.0, 10.37, 4.5])
 @pytest.mark.parametrize("newton,scheme", [("f32_tangent", "basic"), ("exact", "basic"), ("reuse", "basic"),
                                            ("reuse", "al"), ("exact", "al")])
 def test_fp64_local_solves_at_other_exponents_match_the_oracle(newton, scheme, exponent):
