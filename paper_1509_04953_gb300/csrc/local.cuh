@@ -668,16 +668,15 @@ __device__ __forceinline__ void evaluate_crystal(const Cubic<TA> &cu, const TA e
         }
     }
     const TA fn = gs * q6, fs = gs * q12, st = cu.s12 * (sg[0] + sg[1] + sg[2]);
-    const TA ep[6] = {fn * (gD[1] + gD[2]), fn * (gD[0] - gD[2]), -fn * (gD[0] + gD[1]),
-                      fs * (gB[1] + gB[2]), fs * (gB[0] + gA[2]), fs * (gA[0] + gA[1])};
+    const TA ep[6] = {gD[1] + gD[2], gD[0] - gD[2], -(gD[0] + gD[1]), gB[1] + gB[2], gB[0] + gA[2], gA[0] + gA[1]};
     TA el = (TA)0;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        const TA acc = i < 3 ? cu.d * sg[i] + st : cu.s44 * sg[i];
-        r[i] = (acc - etr[i]) + ep[i];
-        if constexpr (WP) el += sg[i] * ((TA)0.5 * acc - etr[i]);
+        const TA u = (i < 3 ? cu.d : cu.s44) * sg[i] + (i < 3 ? st - etr[i] : -etr[i]);   // S sigma - eps_tr
+        r[i] = (i < 3 ? fn : fs) * ep[i] + u;
+        if constexpr (WP) el += sg[i] * (u - etr[i]);
     }
-    if constexpr (WP) phi = el + ps * pot;
+    if constexpr (WP) phi = (TA)0.5 * el + ps * pot;
     if constexpr (WK) {
         const TK ksk = (TK)ks, kn = ksk * (TK)(1.0 / 6.0), kx = ksk * (TK)0.11785113019775792073, kt = ksk * (TK)(1.0 / 12.0);
         const Cubic<TK> ck = cu.template as<TK>();
