@@ -190,7 +190,7 @@ size_t layout(const evp_config *c, evp_handle *h, char *base) {
     const int nb = nucleate_blocks(N3);
     const int r = c->pf_refine == 2 ? 2 : 1;
     const long M3 = (long)r * n * r * n * r * n;   // phase-field points
-    const int npart = std::max(std::max(fft_z_blocks((int)n, T == 8), 2 * pf_stat_blocks(M3) + 1), 14 * al_blocks(N3));
+    const int npart = std::max(std::max(fft_z_blocks((int)n, T == 8, Z_FWD_GAMMA_INV), 2 * pf_stat_blocks(M3) + 1), 14 * al_blocks(N3));
     size_t off = 0;
     auto take = [&](size_t bytes) -> char * {
         off = (off + 255) & ~(size_t)255;
@@ -884,7 +884,7 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
     const double ntol = h->cfg.newton_tol;
     int status = EVP_OK, it = 0, conv = 0, nmax = 0;
     double err_eq = 0, err_bc = 0, mean[6] = {0, 0, 0, 0, 0, 0};
-    const int zb = fft_z_blocks(n, h->dbl);
+    const int zb = fft_z_blocks(n, h->dbl, Z_FWD_GAMMA_INV);
     double hs[8];
     int64_t hcount[3] = {0, 0, 0};
     const int reuse = h->cfg.newton_mode == EVP_NEWTON_REUSE;
@@ -1360,7 +1360,7 @@ int adjoint_sweep(evp_handle *h, const AdjLayout &L, const double *gbar, double 
     const int nseg = (T + ck - 1) / ck;
     const double lam0 = h->mc.lam0, mu0 = h->mc.mu0;
     const double aa_ = lam0 + 2.0 * mu0, bb_ = lam0, det = aa_ * aa_ - bb_ * bb_;
-    const int zb = fft_z_blocks(n, h->dbl);
+    const int zb = fft_z_blocks(n, h->dbl, Z_FWD_GAMMA_INV);
     double gk1 = 0, gk2 = 0, gt0 = 0, gn = 0;
     int rc = save_slot(h, base + L.slot + (size_t)nseg * slot_b, nseg);
     if (rc) return rc;
@@ -1511,7 +1511,7 @@ int evp_adjoint_end(evp_handle *h, const double *gbar, double *grad, double tol,
 extern "C" {
 int evp_residual_scratch_bytes(int n, int precision, size_t *bytes) {
     if (!pow2(n) || !bytes || precision < EVP_FP64 || precision > EVP_MIXED_FAST) return EVP_ERR_ARG;
-    *bytes = sizeof(double) * (size_t)fft_z_blocks(n, precision == EVP_FP64);
+    *bytes = sizeof(double) * (size_t)fft_z_blocks(n, precision == EVP_FP64, Z_FWD_RESID);
     return EVP_OK;
 }
 
@@ -1530,7 +1530,7 @@ int evp_stress_residual(int n, int precision, const void *sig_dev, void *spec_de
         e = fft_xy_r2c<float>((const float *)sig_dev, spec_dev, n, 6, s);
         if (e == cudaSuccess) e = fft_z<float>(spec_dev, n, 6, Z_FWD_RESID, 0, 0, part, out_dev, s);
     }
-    if (e == cudaSuccess) e = reduce_partials(part, fft_z_blocks(n, dbl), 1, out_dev + 6, s);
+    if (e == cudaSuccess) e = reduce_partials(part, fft_z_blocks(n, dbl, Z_FWD_RESID), 1, out_dev + 6, s);
     return e == cudaSuccess ? EVP_OK : EVP_ERR_CUDA;
 }
 

@@ -417,8 +417,16 @@ template <int N> __host__ __device__ constexpr int tile_threads(int lines, int e
                : ((((lines + extra) * (N / Shape<N>::R1) + maxit<N>(lines) - 1) / maxit<N>(lines) + 31) / 32) * 32;
 }
 template <int N, typename T> __host__ __device__ constexpr int y_threads() { return tile_threads<N>(tx_y<N, T>(), 1); }
-template <int N, typename T> __host__ __device__ constexpr int z_threads() {
-    return N == 16 || N == 32 ? 128 : tile_threads<N>(6 * tx_z<N, T>(), 6);
+// z pass of 256^3 in FP32: the Nyquist column in CTAs of its own (TX rows ky each) instead of on tile 0. Its six lines
+// more are what keeps a second CTA off the SM (118 KB of shared memory instead of 106 KB): 432 us a pass with one CTA of
+// 288 threads, 387 us with two of 256 (390 us with 384 threads, 419 us with 512). At 128^3 three CTAs fit either way
+// (46.4 us, 44.8 us apart), and the residual's sums, which go tile by tile, keep their order there and in Z_FWD_RESID.
+__host__ __device__ constexpr bool z_split_of(int n, int tsize) { return n >= 256 && tsize == 4; }
+template <int N, typename T, bool SPLIT> __host__ __device__ constexpr int z_threads() {
+    return SPLIT ? kThreads : N == 16 || N == 32 ? 128 : tile_threads<N>(6 * tx_z<N, T>(), 6);
+}
+template <int N, typename T, bool SPLIT> __host__ __device__ constexpr int z_ctas() {
+    return SPLIT ? 2 : sizeof(T) == 4 && N <= 128 ? 3 : 1;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -937,12 +945,13 @@ __device__ __forceinline__ void gamma_point(C s[6], int kx, int ky, int kz, int 
 }
 
 // ---------------------------------------------------------------------------------------------
-// z pass: CTA = (ky, kx tile); nf fields x TX columns x N planes in shared memory.
+// z pass: CTA = (ky, kx tile); nf fields x TX columns x N planes in shared memory. SPLIT: the first N / TX CTAs take the
+// Nyquist column instead, TX rows ky each.
 // ---------------------------------------------------------------------------------------------
-template <typename T, int N>
-__global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 ? 3 : 1) k_fft_z(typename CT<T>::type *__restrict__ spec, int nf, int mode, GammaC<T> gc,
-                                                   double *__restrict__ partials, double *__restrict__ mean6, const int *__restrict__ skip,
-                                                   ZCtl zc) {
+template <typename T, int N, bool SPLIT>
+__global__ void __launch_bounds__(z_threads<N, T, SPLIT>(), z_ctas<N, T, SPLIT>())
+k_fft_z(typename CT<T>::type *__restrict__ spec, int nf, int mode, GammaC<T> gc, double *__restrict__ partials,
+        double *__restrict__ mean6, const int *__restrict__ skip, ZCtl zc) {
     using C = typename CT<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tw = reinterpret_cast<C *>(smem_raw);
@@ -950,23 +959,29 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    constexpr int TX = tx_z<N, T>(), LS = Shape<N>::LS, Hx = N / 2 + 1, MI = maxit<N>(6 * (TX + 1), z_threads<N, T>());
+    constexpr int TX = tx_z<N, T>(), LS = Shape<N>::LS, Hx = N / 2 + 1, NT = z_threads<N, T, SPLIT>(),
+                  MI = maxit<N>(6 * (SPLIT ? TX : TX + 1), NT);
     __shared__ double red[32];
     constexpr int ntiles = (N / 2) / TX;
-    const int tile = blockIdx.x % ntiles;
-    const int ky = blockIdx.x / ntiles;
-    // lines: f*TX + xl for the TX regular columns of field f, then (tile 0 only) nf*TX + f for the
+    constexpr int NQ = SPLIT ? N / TX : 0;
+    const bool column = SPLIT && (int)blockIdx.x < NQ;   // TX rows ky of the Nyquist column
+    const int b = (int)blockIdx.x - NQ;
+    const int tile = column ? 0 : b % ntiles;
+    const int ky0 = column ? (int)blockIdx.x * TX : b / ntiles;
+    // lines: f*TX + xl for the TX columns of field f, then (tile 0 without SPLIT) nf*TX + f for the
     // Nyquist column kx = N/2 of field f
-    const bool nyq = tile == 0;
-    const int kx0 = tile * TX;
+    const bool nyq = !SPLIT && tile == 0;
+    const int kx0 = column ? N / 2 : tile * TX;
     const int nlines = nf * TX + (nyq ? nf : 0);
+    const long col0 = (long)ky0 * Hx + kx0;     // first column of the tile in a plane, and the step to the next
+    const int cstep = column ? Hx : 1;
     const long plane = (long)N * Hx;            // one z plane of one field
     const long fstride = plane * N;
     // The slab walk: element r = t mod (TX N) of field f sits at column xl and plane z = slab_item(r). With
     // NT threads and NT | TX N, a thread keeps its column, and its planes advance by DZ = NT / TX per step
     // (slab_item adds DZ to z when r grows by NT, and padn adds DZ + DZ / R1 when DZ is a multiple of R1), so its
     // shared and global addresses advance by constant strides.
-    constexpr int NT = z_threads<N, T>(), DZ = NT / TX, KZ = TX * N / NT;
+    constexpr int DZ = NT / TX, KZ = TX * N / NT;
     constexpr int PZ = Shape<N>::R1, DP = DZ + DZ / PZ;
     constexpr bool walk = N >= 16 && (TX * N) % NT == 0 && DZ % PZ == 0 &&
                           ((TX == 8 && N % 16 == 0 && LS % 16 == 9) ? NT % 128 == 0 : NT % TX == 0);
@@ -981,12 +996,12 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
             const int xl = it % TX, f = it / (TX * L);
             i = (it / TX) % L;
             l = f * TX + xl;
-            return spec + f * fstride + (long)ky * Hx + kx0 + xl;
+            return spec + f * fstride + col0 + xl * cstep;
         }
         const int q = it - nreg, f = q / L;
         i = q - f * L;
         l = nf * TX + f;
-        return spec + f * fstride + (long)ky * Hx + N / 2;
+        return spec + f * fstride + (long)ky0 * Hx + N / 2;
     };
     if (mode != Z_INV) {
         // the forward transform's pass 1 (the whole transform when R2 = 1) straight from HBM: item (line, j < M1)
@@ -1009,7 +1024,7 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     } else {
         if constexpr (walk) {
             C *sb = buf + wxl * LS + padn<N>(wz);
-            const C *gb = spec + (long)wz * plane + (long)ky * Hx + kx0 + wxl;
+            const C *gb = spec + (long)wz * plane + col0 + wxl * cstep;
             for (int f = 0; f < nf; ++f) {
 #pragma unroll
                 for (int k = 0; k < KZ; ++k)
@@ -1020,13 +1035,13 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
                 const int f = t / (TX * N), r = t % (TX * N);
                 int z, xl;
                 slab_item<N, TX>(r, z, xl);
-                cp_async<sizeof(C)>(buf + (f * TX + xl) * LS + padn<N>(z), spec + f * fstride + z * plane + (long)ky * Hx + kx0 + xl);
+                cp_async<sizeof(C)>(buf + (f * TX + xl) * LS + padn<N>(z), spec + f * fstride + z * plane + col0 + xl * cstep);
             }
         }
         if (nyq)
             for (int t = threadIdx.x; t < nf * N; t += blockDim.x) {
                 const int f = t / N, z = t % N;
-                cp_async<sizeof(C)>(buf + (nf * TX + f) * LS + padn<N>(z), spec + f * fstride + z * plane + (long)ky * Hx + N / 2);
+                cp_async<sizeof(C)>(buf + (nf * TX + f) * LS + padn<N>(z), spec + f * fstride + z * plane + (long)ky0 * Hx + N / 2);
             }
         cp_async_wait_all();
         __syncthreads();
@@ -1036,7 +1051,7 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
         const bool apply = mode == Z_FWD_GAMMA_INV;
         T acc = (T)0;   // per-thread sum in the field precision; block and global sums in FP64
         // one frequency: its six field values at p0 + f * fstep in the slab
-        auto point = [&](int kz, int kx, C *p0, int fstep) {
+        auto point = [&](int kz, int kx, int ky, C *p0, int fstep) {
             C s6[6];
             for (int f = 0; f < 6; ++f) s6[f] = p0[f * fstep];
             if (kx == 0 && ky == 0 && kz == 0 && mean6 != nullptr) {
@@ -1050,10 +1065,11 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
         };
         if constexpr (walk) {   // the same points per thread, in the same order, as the loop below
             C *pb = buf + wxl * LS + padn<N>(wz);
+            const int kxw = column ? N / 2 : kx0 + wxl, kyw = column ? ky0 + wxl : ky0;
 #pragma unroll
-            for (int k = 0; k < KZ; ++k) point(wz + k * DZ, kx0 + wxl, pb + k * DP, TX * LS);
+            for (int k = 0; k < KZ; ++k) point(wz + k * DZ, kxw, kyw, pb + k * DP, TX * LS);
             if (nyq)
-                for (int t = threadIdx.x; t < N; t += blockDim.x) point(t, N / 2, buf + nf * TX * LS + padn<N>(t), LS);
+                for (int t = threadIdx.x; t < N; t += blockDim.x) point(t, N / 2, ky0, buf + nf * TX * LS + padn<N>(t), LS);
         } else {
             const int npts = (TX + (nyq ? 1 : 0)) * N;
             for (int t = threadIdx.x; t < npts; t += blockDim.x) {
@@ -1061,9 +1077,9 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
                 int zr = 0, xr = 0;
                 if (reg) slab_item<N, TX>(t, zr, xr);
                 const int kz = reg ? zr : t - TX * N;
-                const int kx = reg ? kx0 + xr : N / 2;
+                const int kx = reg && !column ? kx0 + xr : N / 2, ky = column ? ky0 + xr : ky0;
                 const int l0 = reg ? xr : nf * TX, ls = reg ? TX : 1;   // line of field f: l0 + f*ls
-                point(kz, kx, buf + l0 * LS + padn<N>(kz), ls * LS);
+                point(kz, kx, ky, buf + l0 * LS + padn<N>(kz), ls * LS);
             }
         }
         __syncthreads();
@@ -1100,7 +1116,7 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
     if (!inv || Shape<N>::R2 == 1) {   // the slab from shared memory
         if constexpr (walk) {
             const C *sb = buf + wxl * LS + padn<N>(wz);
-            C *gb = spec + (long)wz * plane + (long)ky * Hx + kx0 + wxl;
+            C *gb = spec + (long)wz * plane + col0 + wxl * cstep;
             for (int f = 0; f < nf; ++f) {
 #pragma unroll
                 for (int k = 0; k < KZ; ++k) gb[f * fstride + (long)k * DZ * plane] = sb[f * TX * LS + k * DP];
@@ -1110,13 +1126,13 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
                 const int f = t / (TX * N), r = t % (TX * N);
                 int z, xl;
                 slab_item<N, TX>(r, z, xl);
-                spec[f * fstride + z * plane + (long)ky * Hx + kx0 + xl] = buf[(f * TX + xl) * LS + padn<N>(z)];
+                spec[f * fstride + z * plane + col0 + xl * cstep] = buf[(f * TX + xl) * LS + padn<N>(z)];
             }
         }
         if (nyq)
             for (int t = threadIdx.x; t < nf * N; t += blockDim.x) {
                 const int f = t / N, z = t % N;
-                spec[f * fstride + z * plane + (long)ky * Hx + N / 2] = buf[(nf * TX + f) * LS + padn<N>(z)];
+                spec[f * fstride + z * plane + (long)ky0 * Hx + N / 2] = buf[(nf * TX + f) * LS + padn<N>(z)];
             }
     }
     if (zc.ctl != nullptr) {   // the block with the last ticket runs the fixed-point control (fpctl.cuh)
@@ -1128,8 +1144,8 @@ __global__ void __launch_bounds__(z_threads<N, T>(), sizeof(T) == 4 && N <= 128 
 
 template <typename T, int N> size_t smem_x() { return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)rowpairs<N>() * Shape<N>::LS); }
 template <typename T, int N> size_t smem_y() { return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)(tx_y<N, T>() + 1) * Shape<N>::LS); }
-template <typename T, int N> size_t smem_z(int nf) {
-    return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)nf * (tx_z<N, T>() + 1) * Shape<N>::LS);
+template <typename T, int N> size_t smem_z(int nf, bool split) {
+    return sizeof(typename CT<T>::type) * (Shape<N>::NTW + (size_t)nf * (tx_z<N, T>() + (split ? 0 : 1)) * Shape<N>::LS);
 }
 
 template <typename K> cudaError_t allow_smem(K kernel, size_t bytes) {
@@ -1219,14 +1235,14 @@ cudaError_t xy_c2r_n(const void *spec, T *out, int nfields, T scale, const doubl
     }
 }
 
-template <typename T, int N>
-cudaError_t z_n(void *spec, int nfields, int mode, double lam0, double mu0, double *partials, double *mean6,
+template <typename T, int N, bool SPLIT>
+cudaError_t z_launch(void *spec, int nfields, int mode, double lam0, double mu0, double *partials, double *mean6,
                 cudaStream_t s, const int *skip, const ZCtl *zcp) {
     using C = typename CT<T>::type;
     constexpr int TX = tx_z<N, T>();
-    const int blocks = N * ((N / 2) / TX);
-    const size_t sm = smem_z<T, N>(nfields);
-    cudaError_t e = allow_smem(k_fft_z<T, N>, smem_z<T, N>(6));
+    const int blocks = N * ((N / 2) / TX) + (SPLIT ? N / TX : 0);
+    const size_t sm = smem_z<T, N>(nfields, SPLIT);
+    cudaError_t e = allow_smem(k_fft_z<T, N, SPLIT>, smem_z<T, N>(6, SPLIT));
     if (e != cudaSuccess) return e;
     ZCtl zc{};
     if (zcp != nullptr) zc = *zcp;
@@ -1235,8 +1251,16 @@ cudaError_t z_n(void *spec, int nfields, int mode, double lam0, double mu0, doub
         const T l = (T)lam0, m = (T)mu0;
         gc = GammaC<T>{l, m, (T)1 / m, (T)0.5 / m, (l + m) / (m * (l + (T)2 * m))};
     }
-    return launch_k(skip != nullptr, k_fft_z<T, N>, dim3(blocks), dim3(z_threads<N, T>()), sm, s, (C *)spec, nfields, mode,
+    return launch_k(skip != nullptr, k_fft_z<T, N, SPLIT>, dim3(blocks), dim3(z_threads<N, T, SPLIT>()), sm, s, (C *)spec, nfields, mode,
                     gc, partials, mean6, skip, zc);
+}
+
+template <typename T, int N>
+cudaError_t z_n(void *spec, int nfields, int mode, double lam0, double mu0, double *partials, double *mean6,
+                cudaStream_t s, const int *skip, const ZCtl *zcp) {
+    if constexpr (z_split_of(N, sizeof(T)))
+        if (mode != Z_FWD_RESID) return z_launch<T, N, true>(spec, nfields, mode, lam0, mu0, partials, mean6, s, skip, zcp);
+    return z_launch<T, N, false>(spec, nfields, mode, lam0, mu0, partials, mean6, s, skip, zcp);
 }
 
 #define EVP_DISPATCH(N_, CALL)                             \
@@ -1253,8 +1277,9 @@ cudaError_t z_n(void *spec, int nfields, int mode, double lam0, double mu0, doub
 
 }  // namespace
 
-int fft_z_blocks(int n, int is_double) {
-    return n * ((n / 2) / tx_z_of(n, is_double ? 8 : 4));
+int fft_z_blocks(int n, int is_double, int mode) {
+    const int t = is_double ? 8 : 4, tx = tx_z_of(n, t);
+    return n * ((n / 2) / tx) + (mode != Z_FWD_RESID && z_split_of(n, t) ? n / tx : 0);
 }
 
 int fft_xy_fused(int n, int is_double) {

@@ -71,7 +71,7 @@ template <typename T>
 cudaError_t fft_x_c2r(const void *spec, T *out, int n, int nfields, T scale, const double *add6,
                       cudaStream_t s, const T *base = nullptr, const int *skip = nullptr,
                       const InvCtl *ic = nullptr);
-int fft_z_blocks(int n, int is_double);
+int fft_z_blocks(int n, int is_double, int mode);
 // The x and y passes together: forward = fft_x_r2c then the forward y pass, inverse = the inverse y pass then
 // fft_x_c2r (same contract), with bitwise the same results. Where fft_xy_fused(n, is_double) is 1 each is one
 // launch over (field, z) planes held in shared memory; otherwise the two passes are launched.

@@ -84,7 +84,7 @@ extern "C" int evp_stress_residual_noalloc(int n, int precision, const void *sig
     if (!pow2 || !sig_dev || !spec_dev || !out_dev) return EVP_ERR_ARG;
     if (precision < EVP_FP64 || precision > EVP_MIXED_FAST) return EVP_ERR_ARG;
     const int dbl = precision == EVP_FP64;
-    const int nparts = evp::fft_z_blocks(n, dbl);
+    const int nparts = evp::fft_z_blocks(n, dbl, evp::Z_FWD_RESID);
     if (nparts > kMaxPartials) return EVP_ERR_ARG;   // larger than the fixed scratch array
     double *part = nullptr;
     const int rc = partials_for_current_device(&part);
