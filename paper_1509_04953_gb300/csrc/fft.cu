@@ -8,13 +8,16 @@
 //   y pass : inverse
 //   x pass : half spectrum -> real, fused with the strain update eps += field/N^3 + dE
 // Where a (field, z) plane fits in shared memory next to two others, the x and y passes run as one launch
-// per direction over whole planes (k_fft_xy_r2c, k_fft_xy_c2r), so an iteration crosses HBM three times.
+// per direction over whole planes (k_fft_xy_r2c, k_fft_xy_c2r), so an iteration crosses HBM three times; at 256^3 in FP32
+// a cluster of CTAs holds the plane (k_fft_xy_r2c_cl, k_fft_xy_c2r_cl).
 // Spectra are [field][z|kz][ky][kx] with kx = 0..N/2 (row length N/2+1).
 //
 // Line transforms: Stockham auto-sort with register butterflies. N = R1 * R2 with R1 = 16 (8 for N <= 32, see Shape)
 // and R2 = N / R1 <= 16: a radix-R1 pass (no twiddles) and a radix-R2 pass (twiddles W_N^{r j}),
 // natural order in and out. Shared-memory lines are padded (one slot per R1) so that the strided
 // pass-1 writes hit distinct banks.
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -22,6 +25,8 @@
 #include "common.cuh"
 #include "fpctl.cuh"
 #include "kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace evp {
 
@@ -700,6 +705,38 @@ template <int N, bool INV, typename C, typename St> __device__ void col_pass2(C 
     __syncthreads();
 }
 
+// The two half-spectrum rows of each packed line, in place (row 2p at slots 0..N/2, row 2p+1 at N/2+1..N+1): one line per
+// warp, which reads the line's values before it writes.
+template <int N, typename C> __device__ __forceinline__ void unpack_rows(C *buf, int nlines) {
+    constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, KU = (Hx + 31) / 32;
+            const int lane = threadIdx.x & 31;
+            const auto h = (decltype(buf->x))0.5;
+            for (int p = threadIdx.x >> 5; p < nlines; p += blockDim.x >> 5) {
+                C *line = buf + p * LS;
+                C a[KU], b[KU];
+    #pragma unroll
+                for (int u = 0; u < KU; ++u) {
+                    const int k = lane + 32 * u;
+                    if (k < Hx) {
+                        const C zk = line[padn<N>(k & (N - 1))];
+                        const C zc = cconj(line[padn<N>((N - k) & (N - 1))]);
+                        a[u] = cmk<C>(h * (zk.x + zc.x), h * (zk.y + zc.y));
+                        b[u] = cmk<C>(h * (zk.y - zc.y), -h * (zk.x - zc.x));   // (zk - zc) / 2i
+                    }
+                }
+                __syncwarp();
+    #pragma unroll
+                for (int u = 0; u < KU; ++u) {
+                    const int k = lane + 32 * u;
+                    if (k < Hx) {
+                        line[k] = a[u];
+                        line[Hx + k] = b[u];
+                    }
+                }
+                __syncwarp();
+            }
+}
+
 template <typename T, int N>
 __global__ void __launch_bounds__(xy_threads<N>(), xy_ctas<T, N>())
 k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, const int *__restrict__ skip) {
@@ -710,40 +747,13 @@ k_fft_xy_r2c(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, c
     load_tw<N>(tw);   // constants: under the preceding kernel's tail
     pdl_wait();
     if (skip != nullptr && *skip) return;   // the fixed point has converged
-    constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, NP = N / 2, KU = (Hx + 31) / 32, R2 = Shape<N>::R2;
+    constexpr int Hx = N / 2 + 1, NP = N / 2, R2 = Shape<N>::R2;
     const T *src = in + (long)blockIdx.x * N * N;   // plane = field * N + z
     C *dst = out + (long)blockIdx.x * N * Hx;
     // x: line p packs rows 2p and 2p+1 as one complex row; pass 1 reads them from HBM
     x_pass1_ld<N, false, false>(buf, NP, [&](int p, int e) { return cmk<C>(src[(2 * p) * N + e], src[(2 * p + 1) * N + e]); });
     bfft_pass2<N, false>(buf, NP, tw);
-    {   // unpack one line per warp: read the line's values, then write its two half-spectrum rows in place
-        const int lane = threadIdx.x & 31;
-        const T h = (T)0.5;
-        for (int p = threadIdx.x >> 5; p < NP; p += blockDim.x >> 5) {
-            C *line = buf + p * LS;
-            C a[KU], b[KU];
-#pragma unroll
-            for (int u = 0; u < KU; ++u) {
-                const int k = lane + 32 * u;
-                if (k < Hx) {
-                    const C zk = line[padn<N>(k & (N - 1))];
-                    const C zc = cconj(line[padn<N>((N - k) & (N - 1))]);
-                    a[u] = cmk<C>(h * (zk.x + zc.x), h * (zk.y + zc.y));
-                    b[u] = cmk<C>(h * (zk.y - zc.y), -h * (zk.x - zc.x));   // (zk - zc) / 2i
-                }
-            }
-            __syncwarp();
-#pragma unroll
-            for (int u = 0; u < KU; ++u) {
-                const int k = lane + 32 * u;
-                if (k < Hx) {
-                    line[k] = a[u];
-                    line[Hx + k] = b[u];
-                }
-            }
-            __syncwarp();
-        }
-    }
+    unpack_rows<N>(buf, NP);
     __syncthreads();
     // y: down the columns of the row-major plane; pass 2 stores rows j + R1 r to HBM
     col_pass1<N, false, true>(
@@ -814,6 +824,182 @@ k_fft_xy_c2r(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out,
         const int p = t / N, j = t - p * N;
         const C z = buf[p * LS + padn<N>(j)];
         const long o0 = (r0 + 2 * p) * N + j, o1 = o0 + N;
+        if (has_add) {
+            out[o0] = bsrc[o0] + (z.x * scale + add);
+            out[o1] = bsrc[o1] + (z.y * scale + add);
+        } else {
+            out[o0] = z.x;
+            out[o1] = z.y;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The same for planes larger than one SM holds: a cluster of CL CTAs holds the plane. CTA k has the rows
+// [2 LB k, 2 LB (k + 1)) as LB packed lines for the x transform and the columns [LB k, LB (k + 1)) for the y transform
+// (the last CTA the Nyquist column too); between the two a thread reads the elements of its next item from the CTAs
+// that hold them (distributed shared memory), and writes its own CTA's buffer when the whole cluster has read. The
+// items, operands and order of operations are those of the separate passes, so the spectra are the same bit by bit.
+// Used at 256^3 in FP32 (a plane is 280 KB), where the separate passes cross HBM four times more per iteration and each
+// runs near the memory's rate. Forward: 352 us as two passes, 290 us with clusters of 4 (512 threads, 76 KB, two CTAs
+// per SM; 342 us with clusters of 2 and one CTA per SM, 306 us with 8). Inverse: 433 us as two passes, 389 us (an
+// L2 prefetch of the strain rows ahead of the transforms made it 440 us). At 128^3 in FP64, which the FP64 pipe
+// bounds, the same kernels were slower than the separate passes (transform pair 1640-1690 us, 1605 us).
+// ---------------------------------------------------------------------------------------------
+template <typename T, int N> constexpr int xy_cluster() { return sizeof(T) == 4 && N == 256 ? 4 : 0; }
+template <int N, int CL> struct XyPart {
+    static constexpr int LB = N / 2 / CL, RB = 2 * LB, P = LB + 1, M1 = N / Shape<N>::R1, NT = LB * M1;
+    static constexpr int slots = LB * Shape<N>::LS > N * P ? LB * Shape<N>::LS : N * P;
+    template <typename T> static constexpr size_t smem() {
+        return sizeof(typename CT<T>::type) * (Shape<N>::NTW + slots + N);
+    }
+};
+
+template <typename T, int N, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(XyPart<N, CL>::NT, 2)
+k_fft_xy_r2c_cl(const T *__restrict__ in, typename CT<T>::type *__restrict__ out, const int *__restrict__ skip) {
+    using C = typename CT<T>::type;
+    using X = XyPart<N, CL>;
+    constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2, Hx = N / 2 + 1, M1 = X::M1, LB = X::LB, RB = X::RB, P = X::P;
+    static_assert(R1 == 16 && RB % M1 == 0 && N % M1 == 0, "pass-1 rows of one CTA");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW, *nyq = buf + X::slots;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = blockIdx.x % CL, t = threadIdx.x;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
+    pdl_wait();
+    if (skip != nullptr && *skip) return;   // the fixed point has converged
+    const long plane = blockIdx.x / CL;
+    const T *src = in + (plane * N + rank * RB) * N;
+    C *dst = out + plane * N * Hx;
+    x_pass1_ld<N, false, false>(buf, LB, [&](int p, int e) { return cmk<C>(src[(2 * p) * N + e], src[(2 * p + 1) * N + e]); });
+    bfft_pass2<N, false>(buf, LB, tw);
+    unpack_rows<N>(buf, LB);
+    cl.sync();
+    const int kxl = t % LB, j1 = t / LB, kx = rank * LB + kxl;
+    const bool last = rank == CL - 1;
+    C v[R1];
+#pragma unroll
+    for (int r = 0; r < R1; ++r) v[r] = cl.map_shared_rank(buf, M1 * r / RB)[xy_at<N>(j1 + M1 * r % RB, kx)];
+    if (last)
+        for (int y = t; y < N; y += X::NT) nyq[y] = cl.map_shared_rank(buf, y / RB)[xy_at<N>(y % RB, N / 2)];
+    cl.sync();
+    auto pass1 = [&](int j, int c) {
+        dft_reg<R1, false>(v);
+#pragma unroll
+        for (int r = 0; r < R1; ++r) buf[(R1 * j + r) * P + c] = v[r];
+    };
+    pass1(j1, kxl);
+    if (last && t < M1) {
+#pragma unroll
+        for (int r = 0; r < R1; ++r) v[r] = nyq[t + M1 * r];
+        pass1(t, LB);
+    }
+    __syncthreads();
+    auto pass2 = [&](int j, int c) {
+        C u[R2];
+#pragma unroll
+        for (int r = 0; r < R2; ++r) u[r] = buf[(j + R1 * r) * P + c];
+        pass2_tail<N, false>(u, j, tw);
+#pragma unroll
+        for (int r = 0; r < R2; ++r) dst[(j + R1 * r) * Hx + rank * LB + c] = u[r];
+    };
+    for (int i = t; i < LB * R1; i += X::NT) pass2(i / LB, i % LB);
+    if (last && t < R1) pass2(t, LB);
+}
+
+template <typename T, int N, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(XyPart<N, CL>::NT, 2)
+k_fft_xy_c2r_cl(const typename CT<T>::type *__restrict__ spec, T *__restrict__ out, T scale, int has_add, T a0, T a1, T a2,
+                T a3, T a4, T a5, const T *__restrict__ base, const int *__restrict__ skip, InvCtl ic) {
+    using C = typename CT<T>::type;
+    using X = XyPart<N, CL>;
+    constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2, Hx = N / 2 + 1, M1 = X::M1, LB = X::LB, RB = X::RB, P = X::P;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C *tw = reinterpret_cast<C *>(smem_raw);
+    C *buf = tw + Shape<N>::NTW;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = blockIdx.x % CL, t = threadIdx.x;
+    load_tw<N>(tw);   // constants: under the preceding kernel's tail
+    pdl_wait();
+    if (skip != nullptr && *skip) return;   // the fixed point has converged
+    if (ic.ctl != nullptr && blockIdx.x >= gridDim.x - CL) {   // an extra cluster prepares the next iteration's tolerance
+        if (rank == 0 && t == 0) fp_next_tolerance(ic);
+        return;
+    }
+    const long plane = blockIdx.x / CL;
+    const int f = (int)(plane / N);
+    const C *src = spec + plane * N * Hx;
+    const bool last = rank == CL - 1;
+    const T *bsrc = base ? base : out;
+    const long r0 = plane * N + rank * RB;
+    // y: pass 1 from HBM, the macroscopic strain correction added to the zero-frequency term
+    auto pass1 = [&](int j, int c) {
+        C v[R1];
+#pragma unroll
+        for (int r = 0; r < R1; ++r) v[r] = src[(j + M1 * r) * Hx + rank * LB + c];
+        if (ic.ctl != nullptr && rank == 0 && j == 0 && c == 0) v[0].x += (T)(ic.ctl->corr[f] * ic.n3);
+        dft_reg<R1, true>(v);
+#pragma unroll
+        for (int r = 0; r < R1; ++r) buf[(R1 * j + r) * P + c] = v[r];
+    };
+    pass1(t / LB, t % LB);
+    if (last && t < M1) pass1(t, LB);
+    __syncthreads();
+    auto pass2 = [&](int j, int c) {   // in place: item (j, c) reads and writes rows j + R1 r
+        C u[R2];
+#pragma unroll
+        for (int r = 0; r < R2; ++r) u[r] = buf[(j + R1 * r) * P + c];
+        pass2_tail<N, true>(u, j, tw);
+#pragma unroll
+        for (int r = 0; r < R2; ++r) buf[(j + R1 * r) * P + c] = u[r];
+    };
+    for (int i = t; i < LB * R1; i += X::NT) pass2(i / LB, i % LB);
+    if (last && t < R1) pass2(t, LB);
+    cl.sync();
+    // x: pass 1 packs rows 2p and 2p+1 (Z[k] = A[k] + i B[k], with A[N-k] = conj A[k] past N/2); column k is in CTA k / LB
+    // Read one by one the folded elements made the pass 472 us. The partner N - k of item j's element r is element R1 - 1 - r of item M1 - j (element R1 - r of itself for j = 0),
+    // so each half-spectrum value is read once and the folded half comes by shuffle.
+    static_assert(M1 == 16 && R1 == 16, "a line's items fill a half-warp");
+    const int p = t / M1, j = t % M1, row = (rank * RB + 2 * p) * P, mate = (t & 16) | ((M1 - j) & 15);
+    C v[R1], w[R1 / 2];
+#pragma unroll
+    for (int r = 0; r < R1 / 2; ++r) {
+        const C *line = cl.map_shared_rank(buf, M1 * r / LB) + row + j + M1 * r % LB;
+        const C A = line[0], B = line[P];
+        v[r] = cmk<C>(A.x - B.y, A.y + B.x);
+        w[r] = cmk<C>(A.x + B.y, B.x - A.y);
+    }
+#pragma unroll
+    for (int r = R1 / 2; r < R1; ++r) {
+        v[r].x = __shfl_sync(0xffffffffu, w[R1 - 1 - r].x, mate);
+        v[r].y = __shfl_sync(0xffffffffu, w[R1 - 1 - r].y, mate);
+        if (j == 0) {
+            if (r > R1 / 2) v[r] = w[(R1 - r) % (R1 / 2)];
+            else {
+                const C *line = cl.map_shared_rank(buf, CL - 1) + row + LB;
+                v[r] = cmk<C>(line[0].x - line[P].y, line[0].y + line[P].x);
+            }
+        }
+    }
+    cl.sync();
+    dft_reg<R1, true>(v);
+    {
+        C *d = buf + p * Shape<N>::LS + (R1 + 1) * j;
+#pragma unroll
+        for (int r = 0; r < R1; ++r) d[r] = v[r];
+    }
+    __syncthreads();
+    bfft_pass2<N, true>(buf, LB, tw);
+    T add = (T)0;
+    if (has_add)
+        add = ic.dadd ? (T)ic.dadd[f] : f == 0 ? a0 : f == 1 ? a1 : f == 2 ? a2 : f == 3 ? a3 : f == 4 ? a4 : a5;
+#pragma unroll 4
+    for (int i = t; i < LB * N; i += X::NT) {
+        const int q = i / N, e = i % N;
+        const C z = buf[q * Shape<N>::LS + padn<N>(e)];
+        const long o0 = (r0 + 2 * q) * N + e, o1 = o0 + N;
         if (has_add) {
             out[o0] = bsrc[o0] + (z.x * scale + add);
             out[o1] = bsrc[o1] + (z.y * scale + add);
@@ -1205,6 +1391,15 @@ template <typename T, int N> cudaError_t xy_r2c_n(const T *in, void *spec, int n
         if (e != cudaSuccess) return e;
         return launch_k(skip != nullptr, k_fft_xy_r2c<T, N>, dim3(nfields * N), dim3(xy_threads<N>()), sm, s, in,
                         (C *)spec, skip);
+    } else if constexpr (xy_cluster<T, N>() > 0) {
+        using C = typename CT<T>::type;
+        constexpr int CL = xy_cluster<T, N>();
+        using X = XyPart<N, CL>;
+        constexpr size_t sm = X::template smem<T>();
+        cudaError_t e = allow_smem(k_fft_xy_r2c_cl<T, N, CL>, sm);
+        if (e != cudaSuccess) return e;
+        return launch_k(skip != nullptr, k_fft_xy_r2c_cl<T, N, CL>, dim3(nfields * N * CL), dim3(X::NT), sm, s, in,
+                        (C *)spec, skip);
     } else {
         cudaError_t e = x_r2c_n<T, N>(in, spec, nfields, s, skip);
         if (e != cudaSuccess) return e;
@@ -1215,19 +1410,30 @@ template <typename T, int N> cudaError_t xy_r2c_n(const T *in, void *spec, int n
 template <typename T, int N>
 cudaError_t xy_c2r_n(const void *spec, T *out, int nfields, T scale, const double *add6, cudaStream_t s, const T *base,
                      const int *skip, const InvCtl *icp) {
-    if constexpr (xy_fused<T, N>()) {
+    if constexpr (xy_fused<T, N>() || xy_cluster<T, N>() > 0) {
         using C = typename CT<T>::type;
-        constexpr size_t sm = smem_xy<T, N>();
-        cudaError_t e = allow_smem(k_fft_xy_c2r<T, N>, sm);
-        if (e != cudaSuccess) return e;
         T a[6] = {0, 0, 0, 0, 0, 0};   // rounded to the field precision here, as in the x pass
         if (add6)
             for (int i = 0; i < 6; ++i) a[i] = (T)add6[i];
         const int has_add = add6 != nullptr;
         InvCtl ic{};
         if (icp != nullptr) ic = *icp;
-        return launch_k(skip != nullptr, k_fft_xy_c2r<T, N>, dim3(nfields * N + (ic.ctl != nullptr ? 1 : 0)), dim3(xy_threads<N>()), sm, s,
-                        (const C *)spec, out, scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip, ic);
+        if constexpr (!xy_fused<T, N>()) {
+            constexpr int CL = xy_cluster<T, N>();
+            using X = XyPart<N, CL>;
+            constexpr size_t sm = X::template smem<T>();
+            cudaError_t e = allow_smem(k_fft_xy_c2r_cl<T, N, CL>, sm);
+            if (e != cudaSuccess) return e;
+            return launch_k(skip != nullptr, k_fft_xy_c2r_cl<T, N, CL>, dim3((nfields * N + (ic.ctl != nullptr ? 1 : 0)) * CL),
+                            dim3(X::NT), sm, s, (const C *)spec, out, scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5],
+                            base, skip, ic);
+        } else {
+            constexpr size_t sm = smem_xy<T, N>();
+            cudaError_t e = allow_smem(k_fft_xy_c2r<T, N>, sm);
+            if (e != cudaSuccess) return e;
+            return launch_k(skip != nullptr, k_fft_xy_c2r<T, N>, dim3(nfields * N + (ic.ctl != nullptr ? 1 : 0)), dim3(xy_threads<N>()), sm, s,
+                            (const C *)spec, out, scale, has_add, a[0], a[1], a[2], a[3], a[4], a[5], base, skip, ic);
+        }
     } else {
         cudaError_t e = y_n<T, N>(const_cast<void *>(spec), nfields, 1, s, skip, icp);
         if (e != cudaSuccess) return e;
@@ -1284,9 +1490,9 @@ int fft_z_blocks(int n, int is_double, int mode) {
 
 int fft_xy_fused(int n, int is_double) {
     if (is_double) {
-        EVP_DISPATCH(n, (int)(xy_fused<double, NN>()))
+        EVP_DISPATCH(n, (int)(xy_fused<double, NN>() || xy_cluster<double, NN>() > 0))
     }
-    EVP_DISPATCH(n, (int)(xy_fused<float, NN>()))
+    EVP_DISPATCH(n, (int)(xy_fused<float, NN>() || xy_cluster<float, NN>() > 0))
 }
 
 template <typename T>
