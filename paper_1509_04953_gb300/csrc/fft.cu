@@ -1026,7 +1026,7 @@ __device__ __forceinline__ double rcp_pos(double x) {
 // |xi.sigma|^2 = |xi|^2 |v|^2. t: the tensor components 11, 22, 33, 23, 13, 12; s: the result (Mandel).
 // FP64 (the FP64 pipe bounds the pass): in terms of xi and one reciprocal, about 95 multiply-adds per frequency where
 // normalising xi takes a square root and a division besides. 64^3 FP64 z pass, with GammaC and the tabulated twiddles:
-// 131 us before, 108 after.
+// 131 us before, 102 after.
 template <typename C>
 __device__ __forceinline__ double gamma_regular(const C t[6], C s[6], int f1, int f2, int f3, double w,
                                                 const GammaC<double> &gc) {
@@ -1382,7 +1382,7 @@ cudaError_t y_n(void *spec, int nfields, int inverse, cudaStream_t s, const int 
     return launch_k(skip != nullptr, k_fft_y<T, N, false>, dim3(blocks), dim3(y_threads<N, T>()), sm, s, (C *)spec, skip, ic);
 }
 
-// x and y passes of the forward transform: one fused launch where the plane fits (xy_fused), else the two passes
+// x and y passes of the forward transform: one launch where the plane fits one CTA (xy_fused) or a cluster, else two
 template <typename T, int N> cudaError_t xy_r2c_n(const T *in, void *spec, int nfields, cudaStream_t s, const int *skip) {
     if constexpr (xy_fused<T, N>()) {
         using C = typename CT<T>::type;
