@@ -122,9 +122,16 @@ def load():
 
 def _torch():
     import torch
-    if not torch.cuda.is_available():
+    # a live CUDA context answers without counting the devices
+    if not torch.cuda.is_initialized() and not torch.cuda.is_available():
         raise EVPError("no CUDA device: libevp_gb300 runs on the GPU only")
     return torch
+
+
+def _stream(torch):
+    """Handle of the current stream, without the Python stream object (0.3 us instead of 2.9 us of a small transform's
+    14 us on the host)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 NEWTON_MODES = {"exact": 0, "reuse": 1, "f32_tangent": 2}
@@ -392,7 +399,7 @@ def rfft3d(x):
     cd = torch.complex128 if prec == 0 else torch.complex64
     out = torch.empty((nf, n, n, n // 2 + 1), dtype=cd, device="cuda")
     rc = load().evp_rfft3d(n, prec, nf, x.contiguous().data_ptr(), out.data_ptr(),
-                           torch.cuda.current_stream().cuda_stream)
+                           _stream(torch))
     if rc != 0:
         raise EVPError(f"evp_rfft3d: {EVP_ERR.get(rc, rc)}")
     return out
@@ -405,7 +412,7 @@ def irfft3d(spec):
     prec = 0 if spec.dtype == torch.complex128 else 1
     rd = torch.float64 if prec == 0 else torch.float32
     out = torch.empty((nf, n, n, n), dtype=rd, device="cuda")
-    rc = load().evp_irfft3d(n, prec, nf, spec.data_ptr(), out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    rc = load().evp_irfft3d(n, prec, nf, spec.data_ptr(), out.data_ptr(), _stream(torch))
     if rc != 0:
         raise EVPError(f"evp_irfft3d: {EVP_ERR.get(rc, rc)}")
     return out
@@ -442,7 +449,7 @@ def stress_residual(sig):
     spec = torch.empty((6, n, n, n // 2 + 1), dtype=cd, device="cuda")
     out = torch.empty(7, dtype=torch.float64, device="cuda")
     rc = L.evp_stress_residual(n, prec, sig.contiguous().data_ptr(), spec.data_ptr(), scratch.data_ptr(),
-                               out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+                               out.data_ptr(), _stream(torch))
     if rc != 0:
         raise EVPError(f"evp_stress_residual: {EVP_ERR.get(rc, rc)}")
     return spec, out

@@ -40,3 +40,21 @@ def test_residual_keeps_the_spectrum():
     gen = torch.Generator(device="cuda").manual_seed(3)
     x = torch.randn((6, 256, 256, 256), generator=gen, device="cuda")
     assert torch.equal(evp.stress_residual(x)[0], evp.rfft3d(x))
+
+
+def test_transform_runs_on_the_current_stream():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1509_04953_gb300 import build
+    build.build()
+    from paper_1509_04953_gb300 import evp
+    assert evp._stream(torch) == torch.cuda.current_stream().cuda_stream
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        assert evp._stream(torch) == s.cuda_stream
+        x = torch.randn((1, 8, 8, 8), device="cuda")
+        spec = evp.rfft3d(x)
+    s.synchronize()
+    want = torch.fft.rfftn(x[0].double())
+    assert ((spec[0] - want).abs().max() / want.abs().max()).item() < 2e-6
