@@ -152,7 +152,8 @@ typedef struct evp_handle evp_handle;
 #define EVP_F_GRAIN (1u << 8)   /* current grain id (argmax order parameter), 1 x int32 */
 #define EVP_F_G0    (1u << 9)   /* initial grain id (orientation index), 1 x int32 (get only) */
 #define EVP_F_DRAWS (1u << 10)  /* kappa draws so far, 1 x int32 */
-#define EVP_F_IDS   (1u << 11)  /* active-set ids, kmax x int32 per PF point (slot-major, ascending ids, -1 = empty
+#define EVP_F_IDS   (1u << 11)  /* active-set ids, kmax x int32 per PF point (slot-major, ascending ids; a negative
+                                   id, -1 as written by the library, ends a list: empty
                                    slots last) */
 #define EVP_F_ETA   (1u << 12)  /* active-set order parameters, kmax x T per PF point */
 #define EVP_F_GRAIN_PF (1u << 13)  /* argmax id per PF point, 1 x int32 per PF point (get only; the same as

@@ -203,8 +203,8 @@ __global__ void __launch_bounds__(kPF) k_pf(int n, const int32_t *__restrict__ i
 // The same update as k_pf, voxel by voxel and in the same arithmetic order (so FP64 results are bitwise the
 // same), organised for the SM. A CTA owns a 32 x 8 column tile and marches through kZC planes of z. The active
 // sets of the planes z-1, z, z+1 (interior) and the x/y halo of plane z are staged in shared memory by cp.async,
-// as (id, eta) entries with a -1 id after each list's last staged slot: as an unsigned head that is the largest id, so the
-// seven-list merge reads one entry per step and needs no slot-count checks and no test for an ended list. Which slots to stage comes from a per-row bound: rmax[s] >= the number of
+// as (id, eta) entries with a -1 id after each list's last staged slot: as an unsigned head a negative id lies above every
+// grain id, so the seven-list merge reads one entry per step and needs no slot-count checks and no test for an ended list. Which slots to stage comes from a per-row bound: rmax[s] >= the number of
 // entries of every point of the 32-point row segment s = (z n + y) (n / 32) + x / 32, so every staged load is
 // independent of the others. Each step writes the exact bound of the rows it produced and clears, in the
 // destination, the slots between a point's new count and the destination's previous bound, which keeps every
@@ -375,7 +375,7 @@ k_pf_tile(int n, const int32_t *__restrict__ ids, const T *__restrict__ eta, int
             else pl.R += e * e;
         }
         pl.close();
-        uint32_t head[7];   // a list's current id; an ended list's -1 is the largest
+        uint32_t head[7];   // a list's current id; an ended list's negative one is above every id
         T cur[7];
 #pragma unroll
         for (int q = 0; q < 7; ++q) tb.en.get(at[q], head[q], cur[q]);
@@ -394,8 +394,8 @@ k_pf_tile(int n, const int32_t *__restrict__ ids, const T *__restrict__ eta, int
             uint32_t uid = head[0];
 #pragma unroll
             for (int q = 1; q < 7; ++q) uid = min(uid, head[q]);
-            if (uid == 0xffffffffu) break;
             const int cid = (int)uid;
+            if (cid < 0) break;   // any negative id ends a list, and as unsigned heads they lie above every id
             T e0 = (T)0, nb = (T)0;
 #pragma unroll
             for (int q = 0; q < 7; ++q)
@@ -546,8 +546,8 @@ __global__ void __launch_bounds__(256) k_pf_stats(int n, const int32_t *__restri
 
 // The same on grids of 32 points per edge and more: a warp takes a 32-point row segment. It copies the segment's lists
 // and those of its y+ and z+ neighbours into shared memory, with the rows' slot bounds (rcur, see k_pf_tile), so every load
-// is independent of the others, coalesced and warp-uniform, and merges pairs of lists there (an ended list's -1 is the
-// largest id); the x+ neighbour's list is the next lane's. The pair energy accumulates as
+// is independent of the others, coalesced and warp-uniform, and merges pairs of lists there (an ended list's negative id
+// lies above every grain id as an unsigned number); the x+ neighbour's list is the next lane's. The pair energy accumulates as
 // sum_j e_j^2 (e_0^2 + .. + e_(j-1)^2). A warp walks kStatRows rows before its block adds up (the FP64 block sum is 10
 // FP64-pipe instructions a warp). 128^3: 142 us FP32 and 523 us FP64, where one thread per point with dependent global
 // loads took 226 and 706, and matching the lists pairwise in registers 249 and 706.
@@ -572,7 +572,7 @@ template <typename T> __device__ __forceinline__ T pf_diff2(const PFRow<T> &a, i
     T g = (T)0;
     int pa = 0, pb = 0;
     uint32_t ia = (uint32_t)a.id[0][la], ib = (uint32_t)b.id[0][lb];
-    while ((ia & ib) != 0xffffffffu) {
+    while ((int32_t)(ia & ib) >= 0) {   // until both lists have ended (any negative id)
         T ea = (T)0, eb = (T)0;
         const bool ta = ia <= ib, tb = ib <= ia;
         if (ta) {
