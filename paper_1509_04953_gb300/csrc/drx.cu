@@ -89,11 +89,18 @@ __global__ void k_drx_init(long N3, const int32_t *__restrict__ g0, T *__restric
 
 // Sum of the 12 densities. FP32: as three floats, two error-free sums per term (Knuth), added in FP64 at the end: at
 // least as close to the exact sum as an FP64 running sum, with 5 FP64-pipe operations instead of 24 (128^3: 94 us with
-// those, bound by the FP64 pipe; the 117 MB take 18).
+// those, bound by the FP64 pipe; the 117 MB take 18). Where the FP32 running sum leaves its range, or a density is not finite,
+// the error-free sums are not (infinity less infinity): those points take the FP64 running sum.
 __device__ __forceinline__ void two_sum_r(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
     const float bb = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+template <typename T> __device__ __forceinline__ double plain_sum12(const T r[12]) {
+    double kk = 0.0;
+#pragma unroll
+    for (int a = 0; a < 12; ++a) kk += (double)r[a];
+    return kk;
 }
 __device__ __forceinline__ double sum12(const float r[12]) {
     float hi = r[0], lo = 0.f, lo2 = 0.f;
@@ -104,14 +111,10 @@ __device__ __forceinline__ double sum12(const float r[12]) {
         two_sum_r(lo, e, lo, e2);
         lo2 = __fadd_rn(lo2, e2);
     }
+    if (!isfinite(hi)) return plain_sum12(r);
     return (double)hi + ((double)lo + (double)lo2);
 }
-__device__ __forceinline__ double sum12(const double r[12]) {
-    double kk = 0.0;
-#pragma unroll
-    for (int a = 0; a < 12; ++a) kk += r[a];
-    return kk;
-}
+__device__ __forceinline__ double sum12(const double r[12]) { return plain_sum12(r); }
 template <typename T>
 __global__ void k_refresh_k(long N3, const T *__restrict__ rho, double *__restrict__ k) {
     const long v = (long)blockIdx.x * blockDim.x + threadIdx.x;
