@@ -157,34 +157,16 @@ __device__ int newton_voxel_df(const Problem<double> &pb, const double etr[6], d
 #pragma unroll
         for (int i = 0; i < 6; ++i) rf[i] = (float)e.r[i];
         if (!ldl_solve<float, float>(e.K, rf, df)) return -it;
-        double d[6], sn = 0.0;
-        float dn2 = 0.f, rdf = 0.f;
+        double d[6], rd = 0.0, dn = 0.0, sn = 0.0;
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
             d[i] = (double)df[i];
-            rdf += rf[i] * df[i];
-            dn2 += df[i] * df[i];
+            rd += e.r[i] * d[i];
+            dn += d[i] * d[i];
             sn += sg[i] * sg[i];
         }
-        // the norms and r.d steer the stopping and line-search tests only: in FP32 (the step and the residual it was
-        // solved for are FP32 vectors), in FP64 where a value leaves the range of FP32
-        const float snf = (float)sn;
-        const bool in_range = dn2 > 1e-30f && dn2 < 1e30f && snf < 1e30f && fabsf(rdf) > 1e-35f && fabsf(rdf) < 1e30f;
-        double dn, scale, rd;
-        if (in_range) {
-            dn = (double)sqrtf(dn2);
-            scale = (double)sqrtf(snf) + tauc;
-            rd = (double)rdf;
-        } else {
-            dn = rd = 0.0;
-#pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                dn += d[i] * d[i];
-                rd += e.r[i] * d[i];
-            }
-            dn = dsqrt(dn);
-            scale = dsqrt(sn) + tauc;
-        }
+        dn = dsqrt(dn);
+        const double scale = dsqrt(sn) + tauc;
         if (dn <= tol * scale && rd >= 0.0) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) sg[i] -= d[i];
