@@ -567,25 +567,21 @@ template <typename T> __device__ __forceinline__ void fam_stress(int f, const T 
 }
 
 // Rates of one family. Power law: t = tau / tau_c, gam = |t|^n sign(t), slope = |t|^(n-1), pot += |t|^(n+1), to be
-// scaled by the caller. Ma-Roters: t = tau, gam, slope and pot as in Eq. FlowRule. WK: slopes wanted, in TK; tk holds
-// the resolved stresses in TK (for an FP32 tangent they are formed in FP32: six conversions instead of twelve).
+// scaled by the caller. Ma-Roters: t = tau, gam, slope and pot as in Eq. FlowRule. WK: slopes wanted, in TK, each
+// rounded once from TA: as ninth powers of FP32 stress differences they put the FP32 tangent of the FP64 residual off by up
+// to 26 units of 2^-24 instead of 5.
 template <bool WK, bool WP, typename TK, typename TA>
-__device__ __forceinline__ void fam_rates(TA, int, const TA t[4], const TK tk[4], const MatConst &mc, TA gam[4],
-                                          TK slope[4], TA &pot) {
+__device__ __forceinline__ void fam_rates(TA, int, const TA t[4], const MatConst &mc, TA gam[4], TK slope[4], TA &pot) {
     if (mc.n_int == 10) {
         // the workloads' exponent: |t|^9 = |t| ((t^2)^2)^2, the very products pow_nm1's bit loop forms
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const TA b2 = t[q] * t[q], b4 = b2 * b2, b8 = b4 * b4, ax = fabs(t[q]);
-            if constexpr (WK && sizeof(TK) == sizeof(TA)) {
-                const TA p9 = ax * b8;
-                slope[q] = p9;
+            const TA b2 = t[q] * t[q], b4 = b2 * b2, b8 = b4 * b4;
+            if constexpr (WK) {
+                const TA p9 = fabs(t[q]) * b8;
+                slope[q] = (TK)p9;
                 gam[q] = p9 * t[q];
             } else {
-                if constexpr (WK) {   // FP32 tangent of the FP64 residual
-                    const TK x = fabs(tk[q]), c2 = x * x, c4 = c2 * c2;
-                    slope[q] = x * (c4 * c4);
-                }
                 gam[q] = copysign(b8 * b2, t[q]);
             }
             if constexpr (WP) pot += gam[q] * t[q];
@@ -601,8 +597,8 @@ __device__ __forceinline__ void fam_rates(TA, int, const TA t[4], const TK tk[4]
     }
 }
 template <bool WK, bool WP, typename TK, typename TA>
-__device__ __forceinline__ void fam_rates(const FlowMR<TA> &hf, int f, const TA t[4], const TK *, const MatConst &mc,
-                                          TA gam[4], TK slope[4], TA &pot) {
+__device__ __forceinline__ void fam_rates(const FlowMR<TA> &hf, int f, const TA t[4], const MatConst &mc, TA gam[4],
+                                          TK slope[4], TA &pot) {
     const TA ga = mr_ga<TA>(mc);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -643,18 +639,14 @@ __device__ __forceinline__ void evaluate_crystal(const Cubic<TA> &cu, const TA e
     TA h[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) h[i] = (i < 3 ? an : as) * sg[i];
-    TK hk[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) hk[i] = (TK)h[i];
     TA gD[3], gA[3], gB[3], pot = (TA)0;
     TK W[3], kA[3], kB[3], kX[3];
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
         TA t[4], g[4];
-        TK w[4], tk[4];
+        TK w[4];
         fam_stress(f, h, t);
-        fam_stress(f, hk, tk);
-        fam_rates<WK, WP, TK>(hf, f, t, tk, mc, g, w, pot);
+        fam_rates<WK, WP, TK>(hf, f, t, mc, g, w, pot);
         const TA gu = g[0] - g[1], gw = g[2] - g[3];
         gD[f] = (g[0] + g[1]) + (g[2] + g[3]);
         gA[f] = gu + gw;

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kThreads) k_newton(long N3, const TA *__restri
 }
 
 // FP64 path: Newton on the FP64 residual with an FP32 tangent and FP32 6x6 solve. Each step is a
-// slightly inexact Newton step (relative tangent error ~1e-7), so the iteration contracts at least
+// slightly inexact Newton step (tangent rounded to FP32: a few 1e-7 relative), so the iteration contracts at least
 // ~1e-6 per step near the solution and stops on the same step-size test; Armijo backtracking on
 // the FP64 potential keeps it globally convergent.
 __device__ int newton_voxel_df(const Problem<double> &pb, const double etr[6], double tauc, double sg[6],
