@@ -1339,6 +1339,7 @@ k_fft_z(typename CT<T>::type *__restrict__ spec, int nf, int mode, GammaC<T> gc,
     if (zc.ctl != nullptr) {   // the block with the last ticket runs the fixed-point control (fpctl.cuh)
         if (threadIdx.x >= 32) return;
         if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
+        __syncwarp();   // as in k_al_control; the inverse transform's barriers do the same
         fp_control_warp(zc, partials, gridDim.x);
     }
 }

@@ -56,7 +56,8 @@ __device__ __forceinline__ unsigned fp_take_ticket(const ZCtl &z) {
     return t;
 }
 
-// The 32 lanes of one warp call this with the iteration's nparts partial sums.
+// The 32 lanes of one warp call this with the iteration's nparts partial sums. Between fp_take_ticket and this call lies
+// a barrier of the block (those of the inverse transform) or of the warp, which passes the acquire on to the other lanes.
 __device__ __forceinline__ void fp_control_warp(const ZCtl &z, const double *__restrict__ part, int nparts) {
     FpCtl *c = z.ctl;
     const FpCtlParams &p = z.p;

@@ -946,6 +946,7 @@ __global__ void __launch_bounds__(256) k_al_control(AlCtl *c, const double *__re
         asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;\n" : "=r"(ticket) : "l"(&c->ticket) : "memory");
     }
     if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
+    __syncwarp();   // lane 0's acquire orders the other lanes' reads of the sums (a shuffle orders no memory)
     const double hl = lane < 14 ? __ldcg(c->sum + lane) * p.inv_n3 : 0.0;   // the means
     const unsigned all = 0xffffffffu;
     // lanes 0-5: component i of |E|^2, |<lam>|^2 and its stress-controlled part, summed over lanes 0-7
