@@ -51,25 +51,16 @@ template <typename TA> __device__ __forceinline__ void flow_consts(const MatCons
 __host__ __device__ constexpr int pk(int i, int j) { return i * (i + 1) / 2 + j; }
 
 // Per-grain tables: compliance rows (36 words) and Schmid vectors (12 x 6 words) per grain, each grain
-// starting on a 16-byte boundary (144 g / 288 g bytes in FP32, twice that in FP64). They are read with
+// starting on a 16-byte boundary (144 g / 288 g bytes), for the FP32 local problems. They are read with
 // 16-byte vector loads; the load instructions, not the bytes (the tables sit in L1), are what a
 // per-voxel kernel issuing one load per word runs short of.
-template <typename TA> __device__ __forceinline__ void load_compliance(const TA *__restrict__ S, TA Sp[21]) {
-    TA full[36];
-    if constexpr (sizeof(TA) == 4) {
-        const float4 *S4 = reinterpret_cast<const float4 *>(S);
+__device__ __forceinline__ void load_compliance(const float *__restrict__ S, float Sp[21]) {
+    float full[36];
+    const float4 *S4 = reinterpret_cast<const float4 *>(S);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const float4 t = __ldg(S4 + k);
-            full[4 * k] = t.x; full[4 * k + 1] = t.y; full[4 * k + 2] = t.z; full[4 * k + 3] = t.w;
-        }
-    } else {
-        const double2 *S2 = reinterpret_cast<const double2 *>(S);
-#pragma unroll
-        for (int k = 0; k < 18; ++k) {
-            const double2 t = __ldg(S2 + k);
-            full[2 * k] = t.x; full[2 * k + 1] = t.y;
-        }
+    for (int k = 0; k < 9; ++k) {
+        const float4 t = __ldg(S4 + k);
+        full[4 * k] = t.x; full[4 * k + 1] = t.y; full[4 * k + 2] = t.z; full[4 * k + 3] = t.w;
     }
 #pragma unroll
     for (int i = 0; i < 6; ++i)
@@ -77,21 +68,12 @@ template <typename TA> __device__ __forceinline__ void load_compliance(const TA 
         for (int j = 0; j <= i; ++j) Sp[i * (i + 1) / 2 + j] = full[6 * i + j];
 }
 // Schmid vectors of slip systems 2p and 2p+1 (12 consecutive words, 16-byte aligned).
-template <typename TA> __device__ __forceinline__ void load_slip_pair(const TA *__restrict__ M, int p, TA m[12]) {
-    if constexpr (sizeof(TA) == 4) {
-        const float4 *M4 = reinterpret_cast<const float4 *>(M + 12 * p);
+__device__ __forceinline__ void load_slip_pair(const float *__restrict__ M, int p, float m[12]) {
+    const float4 *M4 = reinterpret_cast<const float4 *>(M + 12 * p);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float4 t = __ldg(M4 + k);
-            m[4 * k] = t.x; m[4 * k + 1] = t.y; m[4 * k + 2] = t.z; m[4 * k + 3] = t.w;
-        }
-    } else {
-        const double2 *M2 = reinterpret_cast<const double2 *>(M + 12 * p);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const double2 t = __ldg(M2 + k);
-            m[2 * k] = t.x; m[2 * k + 1] = t.y;
-        }
+    for (int k = 0; k < 3; ++k) {
+        const float4 t = __ldg(M4 + k);
+        m[4 * k] = t.x; m[4 * k + 1] = t.y; m[4 * k + 2] = t.z; m[4 * k + 3] = t.w;
     }
 }
 
@@ -105,22 +87,17 @@ template <typename TA> __device__ __forceinline__ void load_slip_pair(const TA *
 // stress out. k_newton_df at 64^3: 319 us per fixed-point iteration, 501 with the sample-frame vectors.
 // The FP32 problems stay in the sample frame: rotating the stress in FP32 adds a rounding of the stress itself, and
 // the equilibrium residual of the converged FP32 field rose from 5.0e-7 to 7.5e-7 of its tolerance's 1e-6.
-// The grain table holds kFrameWords words per grain: R (crystal -> sample, row-major) and 3 words of padding.
-template <typename T> __device__ __forceinline__ void load_frame(const T *__restrict__ R, T r[9]) {
-    if constexpr (sizeof(T) == 4) {
-        const float4 *R4 = reinterpret_cast<const float4 *>(R);
-        const float4 a = __ldg(R4), b = __ldg(R4 + 1);
-        r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y; r[6] = b.z; r[7] = b.w;
-        r[8] = __ldg(R + 8);
-    } else {
-        const double2 *R2 = reinterpret_cast<const double2 *>(R);
+// The grain table holds kFrameWords words per grain: R (crystal -> sample, row-major) and a word of padding, which keeps
+// each grain's words on a 16-byte boundary.
+static_assert(kFrameWords % 2 == 0 && kFrameWords >= 9, "frames are read in 16-byte pairs");
+__device__ __forceinline__ void load_frame(const double *__restrict__ R, double r[9]) {
+    const double2 *R2 = reinterpret_cast<const double2 *>(R);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const double2 t = __ldg(R2 + k);
-            r[2 * k] = t.x; r[2 * k + 1] = t.y;
-        }
-        r[8] = __ldg(R + 8);
+    for (int k = 0; k < 4; ++k) {
+        const double2 t = __ldg(R2 + k);
+        r[2 * k] = t.x; r[2 * k + 1] = t.y;
     }
+    r[8] = __ldg(R + 8);
 }
 // out = Mandel(A^T X A) with X the symmetric tensor of Mandel vector x and A given by its entries a(i, j).
 template <typename T, typename F> __device__ __forceinline__ void rotate_mandel(const T x[6], F a, T out[6]) {
@@ -267,41 +244,40 @@ template <typename TA, typename TK = TA> struct Eval {
     TA phi;
 };
 
-template <typename TA>
-__device__ __forceinline__ void evaluate(const TA Sp[21], const TA *__restrict__ M, const TA etr[6], TA tauc, TA inv_tc,
-                                         const TA sg[6], const MatConst &mc, Eval<TA> &e) {
-    TA dt, g0, nn;
+__device__ __forceinline__ void evaluate(const float Sp[21], const float *__restrict__ M, const float etr[6], float tauc,
+                                         float inv_tc, const float sg[6], const MatConst &mc, Eval<float> &e) {
+    float dt, g0, nn;
     flow_consts(mc, dt, g0, nn);
-    TA phi = (TA)0;
+    float phi = 0.f;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        TA acc = (TA)0;
+        float acc = 0.f;
 #pragma unroll
         for (int j = 0; j < 6; ++j) acc += Sp[i >= j ? pk(i, j) : pk(j, i)] * sg[j];
         e.r[i] = acc - etr[i];
-        phi += sg[i] * ((TA)0.5 * acc - etr[i]);
+        phi += sg[i] * (0.5f * acc - etr[i]);
     }
 #pragma unroll
     for (int q = 0; q < 21; ++q) e.K[q] = Sp[q];
-    const TA cphi = dt * g0 * tauc / (nn + (TA)1);
-    const TA cslope = dt * nn * g0 * inv_tc;
+    const float cphi = dt * g0 * tauc / (nn + 1.f);
+    const float cslope = dt * nn * g0 * inv_tc;
 #pragma unroll 1
     for (int p = 0; p < 6; ++p) {
-      TA mm[12];
+      float mm[12];
       load_slip_pair(M, p, mm);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const TA *m = mm + 6 * h;
-        TA tau = (TA)0;
+        const float *m = mm + 6 * h;
+        float tau = 0.f;
 #pragma unroll
         for (int i = 0; i < 6; ++i) tau += m[i] * sg[i];
-        const TA x = tau * inv_tc;
-        const TA ax = fabs(x);
-        const TA p9 = pow_nm1(ax, mc);       // |x|^(n-1)
-        const TA p10 = p9 * ax;              // |x|^n
-        const TA gd = x < (TA)0 ? -g0 * p10 : g0 * p10;
-        const TA slope = cslope * p9;
-        TA sm[6];
+        const float x = tau * inv_tc;
+        const float ax = fabs(x);
+        const float p9 = pow_nm1(ax, mc);       // |x|^(n-1)
+        const float p10 = p9 * ax;              // |x|^n
+        const float gd = x < 0.f ? -g0 * p10 : g0 * p10;
+        const float slope = cslope * p9;
+        float sm[6];
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
             e.r[i] += dt * gd * m[i];
@@ -362,37 +338,36 @@ template <typename TA> __device__ __forceinline__ void mr_sys(const FlowMR<TA> &
     }
 }
 
-template <typename TA>
-__device__ __forceinline__ void evaluate(const TA Sp[21], const TA *__restrict__ M, const TA etr[6], const FlowMR<TA> &f,
-                                         TA, const TA sg[6], const MatConst &mc, Eval<TA> &e) {
-    TA dt, g0, nn;
+__device__ __forceinline__ void evaluate(const float Sp[21], const float *__restrict__ M, const float etr[6],
+                                         const FlowMR<float> &f, float, const float sg[6], const MatConst &mc, Eval<float> &e) {
+    float dt, g0, nn;
     flow_consts(mc, dt, g0, nn);
-    const TA ga = mr_ga<TA>(mc);
-    TA phi = (TA)0;
+    const float ga = mr_ga<float>(mc);
+    float phi = 0.f;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        TA acc = (TA)0;
+        float acc = 0.f;
 #pragma unroll
         for (int j = 0; j < 6; ++j) acc += Sp[i >= j ? pk(i, j) : pk(j, i)] * sg[j];
         e.r[i] = acc - etr[i];
-        phi += sg[i] * ((TA)0.5 * acc - etr[i]);
+        phi += sg[i] * (0.5f * acc - etr[i]);
     }
 #pragma unroll
     for (int q = 0; q < 21; ++q) e.K[q] = Sp[q];
 #pragma unroll 1
     for (int p = 0; p < 6; ++p) {
-      TA mm[12];
+      float mm[12];
       load_slip_pair(M, p, mm);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const TA *m = mm + 6 * h;
-        TA tau = (TA)0;
+        const float *m = mm + 6 * h;
+        float tau = 0.f;
 #pragma unroll
         for (int i = 0; i < 6; ++i) tau += m[i] * sg[i];
-        TA tp, itc, gd, slope, psi;
+        float tp, itc, gd, slope, psi;
         mr_sys(f, 2 * p + h, tp, itc);
         mr_flow(tau, tp, itc, ga, gd, slope, psi);
-        TA sm[6];
+        float sm[6];
 #pragma unroll
         for (int i = 0; i < 6; ++i) {
             e.r[i] += dt * gd * m[i];
@@ -472,35 +447,35 @@ template <typename TA> struct EvalR {
 };
 // UNROLL: slip-system pairs unrolled per loop trip (6 = fully, letting the table loads run ahead of
 // the arithmetic where registers allow).
-template <typename TA, int UNROLL = 1>
-__device__ __forceinline__ void evaluate_r(const TA Sp[21], const TA *__restrict__ M, const TA etr[6], TA tauc, TA inv_tc,
-                                           const TA sg[6], const MatConst &mc, EvalR<TA> &e) {
-    TA dt, g0, nn;
+template <int UNROLL = 1>
+__device__ __forceinline__ void evaluate_r(const float Sp[21], const float *__restrict__ M, const float etr[6], float tauc,
+                                           float inv_tc, const float sg[6], const MatConst &mc, EvalR<float> &e) {
+    float dt, g0, nn;
     flow_consts(mc, dt, g0, nn);
-    TA phi = (TA)0;
+    float phi = 0.f;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        TA acc = (TA)0;
+        float acc = 0.f;
 #pragma unroll
         for (int j = 0; j < 6; ++j) acc += Sp[i >= j ? pk(i, j) : pk(j, i)] * sg[j];
         e.r[i] = acc - etr[i];
-        phi += sg[i] * ((TA)0.5 * acc - etr[i]);
+        phi += sg[i] * (0.5f * acc - etr[i]);
     }
-    const TA cphi = dt * g0 * tauc / (nn + (TA)1);
+    const float cphi = dt * g0 * tauc / (nn + 1.f);
 #pragma unroll UNROLL
     for (int p = 0; p < 6; ++p) {
-        TA mm[12];
+        float mm[12];
         load_slip_pair(M, p, mm);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const TA *m = mm + 6 * h;
-            TA tau = (TA)0;
+            const float *m = mm + 6 * h;
+            float tau = 0.f;
 #pragma unroll
             for (int i = 0; i < 6; ++i) tau += m[i] * sg[i];
-            const TA x = tau * inv_tc, ax = fabs(x);
-            const TA p10 = pow_nm1(ax, mc) * ax;
-            const TA gd = x < (TA)0 ? -g0 * p10 : g0 * p10;
-            const TA dg = dt * gd;
+            const float x = tau * inv_tc, ax = fabs(x);
+            const float p10 = pow_nm1(ax, mc) * ax;
+            const float gd = x < 0.f ? -g0 * p10 : g0 * p10;
+            const float dg = dt * gd;
 #pragma unroll
             for (int i = 0; i < 6; ++i) e.r[i] += dg * m[i];
             phi += cphi * p10 * ax;
@@ -510,35 +485,35 @@ __device__ __forceinline__ void evaluate_r(const TA Sp[21], const TA *__restrict
 }
 
 
-template <typename TA, int UNROLL = 1>
-__device__ __forceinline__ void evaluate_r(const TA Sp[21], const TA *__restrict__ M, const TA etr[6],
-                                           const FlowMR<TA> &f, TA, const TA sg[6], const MatConst &mc, EvalR<TA> &e) {
-    TA dt, g0, nn;
+template <int UNROLL = 1>
+__device__ __forceinline__ void evaluate_r(const float Sp[21], const float *__restrict__ M, const float etr[6],
+                                           const FlowMR<float> &f, float, const float sg[6], const MatConst &mc, EvalR<float> &e) {
+    float dt, g0, nn;
     flow_consts(mc, dt, g0, nn);
-    const TA ga = mr_ga<TA>(mc);
-    TA phi = (TA)0;
+    const float ga = mr_ga<float>(mc);
+    float phi = 0.f;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        TA acc = (TA)0;
+        float acc = 0.f;
 #pragma unroll
         for (int j = 0; j < 6; ++j) acc += Sp[i >= j ? pk(i, j) : pk(j, i)] * sg[j];
         e.r[i] = acc - etr[i];
-        phi += sg[i] * ((TA)0.5 * acc - etr[i]);
+        phi += sg[i] * (0.5f * acc - etr[i]);
     }
 #pragma unroll UNROLL
     for (int p = 0; p < 6; ++p) {
-        TA mm[12];
+        float mm[12];
         load_slip_pair(M, p, mm);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const TA *m = mm + 6 * h;
-            TA tau = (TA)0;
+            const float *m = mm + 6 * h;
+            float tau = 0.f;
 #pragma unroll
             for (int i = 0; i < 6; ++i) tau += m[i] * sg[i];
-            TA tp, itc, gd, slope, psi;
+            float tp, itc, gd, slope, psi;
             mr_sys(f, 2 * p + h, tp, itc);
             mr_flow(tau, tp, itc, ga, gd, slope, psi);
-            const TA dg = dt * gd;
+            const float dg = dt * gd;
 #pragma unroll
             for (int i = 0; i < 6; ++i) e.r[i] += dg * m[i];
             phi += dt * psi;
@@ -773,7 +748,7 @@ __device__ __forceinline__ void evaluate_r(const Problem<double> &p, const doubl
 template <int UNROLL = 1, typename H>
 __device__ __forceinline__ void evaluate_r(const Problem<float> &p, const float etr[6], const H &hf, float inv_tc,
                                            const float sg[6], const MatConst &mc, EvalR<float> &e) {
-    evaluate_r<float, UNROLL>(p.Sp, p.M, etr, hf, inv_tc, sg, mc, e);
+    evaluate_r<UNROLL>(p.Sp, p.M, etr, hf, inv_tc, sg, mc, e);
 }
 
 }  // namespace evp
