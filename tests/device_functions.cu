@@ -2,6 +2,14 @@
 #include "local.cuh"
 
 namespace {
+__global__ void k_pow(long n, const double *__restrict__ x, const double *__restrict__ y, double *__restrict__ table,
+                      double *__restrict__ cuda) {
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    table[i] = evp::pow_tab(x[i], y[i]);
+    cuda[i] = pow(x[i], y[i]);
+}
+
 // sg: 6 x n stresses in the crystal frame; k32, k64: 21 x n tangents (packed lower)
 __global__ void k_tangent(long n, const double *__restrict__ sg, evp::Cubic<double> cub, double tauc, evp::MatConst mc,
                           float *__restrict__ k32, double *__restrict__ k64) {
@@ -24,6 +32,10 @@ __global__ void k_tangent(long n, const double *__restrict__ sg, evp::Cubic<doub
 }
 }  // namespace
 
+extern "C" int dev_pow(long n, const double *x, const double *y, double *table, double *cuda, void *stream) {
+    k_pow<<<(unsigned)((n + 127) / 128), 128, 0, (cudaStream_t)stream>>>(n, x, y, table, cuda);
+    return (int)cudaGetLastError();
+}
 extern "C" int dev_tangent(long n, const double *sg, double d, double s12, double s44, double tauc, double gdot0,
                            double dt, double exponent, int n_int, float *k32, double *k64, void *stream) {
     evp::MatConst mc{};

@@ -19,5 +19,6 @@ def load(tmp):
     assert r.returncode == 0, r.stderr
     lib = C.CDLL(so)
     vp, i, d, n = C.c_void_p, C.c_int, C.c_double, C.c_long
+    lib.dev_pow.argtypes = [n, vp, vp, vp, vp, vp]
     lib.dev_tangent.argtypes = [n, vp, d, d, d, d, d, d, d, i, vp, vp, vp]
     return torch, lib
