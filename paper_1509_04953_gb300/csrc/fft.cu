@@ -47,8 +47,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Radices and padded line stride. N = 16 and 32 take R1 = 8: a plane or a slab of such a grid is small, its transform is
 // bound by the latency of each thread's chain and by the threads it occupies, and radix-8 items are twice as many and
 // half as long as radix-16 ones (32^3 FP32 plane of 16 packed lines: 64 items instead of 32). Their second pass starts
-// with the last stage of the radix-16 network (pass2_tail), so the arithmetic is that of the radix-16 split,
-// operation by operation. The line strides keep both ways a warp walks a tile (along lines, across lines) at most
+// with the last stage of the radix-16 network (pass2_tail), so the butterflies are those of the radix-16 split. The line strides keep both ways a warp walks a tile (along lines, across lines) at most
 // two-way bank-conflicted. NTW: slots of the twiddle table (load_tw).
 template <int N> struct Shape {
     static constexpr int R1 = N < 16 ? N : N <= 32 ? 8 : 16;
@@ -256,7 +255,9 @@ template <bool FY> __device__ __forceinline__ double2 cmul_r(double2 a, double2 
 // tw[R1 r + j], then a radix-R2 DFT. N <= 32: values r and r + R2/2 are the even and odd halves of a radix-16 DFT, so
 // its last stage (W16^j, at tw[N + j]) gives its outputs j and j + 8, which then take the twiddles and the radix-R2/2
 // DFT of the 16 x R2/2 split; slot j + 8 q holds its output q.
-// FY (cmul_r): chosen so that FP32 transforms of 16 and 32 points give the bits of the radix-16 form.
+// FP32: which product of each sum is fused (FY of cmul_r, and the selects below) follows the compiler's choices in the
+// radix-16 form, so that a transform of 16 or 32 points rounded as it did before the split (compared bit by bit when
+// this form came in). Either choice rounds the same number of times; nothing depends on it.
 template <int N, bool INV, bool FY = true, typename C> __device__ __forceinline__ void pass2_tail(C (&u)[Shape<N>::R2], int j, const C *tw) {
     constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2;
     auto tw_at = [&](int i) {
