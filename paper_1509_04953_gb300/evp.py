@@ -130,8 +130,9 @@ def _torch():
 
 def _stream(torch):
     """Handle of the current stream, without the Python stream object (0.3 us instead of 2.9 us of a small transform's
-    14 us on the host)."""
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    14 us on the host) where this PyTorch has the call for it, which is not part of its public interface."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
 
 
 NEWTON_MODES = {"exact": 0, "reuse": 1, "f32_tangent": 2}
