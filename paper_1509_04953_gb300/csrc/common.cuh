@@ -31,6 +31,13 @@ __device__ __forceinline__ double block_sum(double v, double *sh /* >= 32 double
     return v;
 }
 
+// Error-free sum of two floats (Knuth): s is the rounded sum and s + e equals a + b exactly, while s is finite.
+__device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
 // Programmatic dependent launch (sm_90+). The kernels of one fixed-point iteration are queued back to back; each is
 // launched with programmatic stream serialization, so its launch overlaps the exit of its predecessor's last CTAs.
 // pdl_wait() blocks until the preceding kernel has completed and its memory is visible (a no-op for a kernel

@@ -91,11 +91,6 @@ __global__ void k_drx_init(long N3, const int32_t *__restrict__ g0, T *__restric
 // least as close to the exact sum as an FP64 running sum, with 5 FP64-pipe operations instead of 24 (128^3: 94 us with
 // those, bound by the FP64 pipe; the 117 MB take 18). Where the FP32 running sum leaves its range, or a density is not finite,
 // the error-free sums are not (infinity less infinity): those points take the FP64 running sum.
-__device__ __forceinline__ void two_sum_r(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
 template <typename T> __device__ __forceinline__ double plain_sum12(const T r[12]) {
     double kk = 0.0;
 #pragma unroll
@@ -107,8 +102,8 @@ __device__ __forceinline__ double sum12(const float r[12]) {
 #pragma unroll
     for (int a = 1; a < 12; ++a) {
         float e, e2;
-        two_sum_r(hi, r[a], hi, e);
-        two_sum_r(lo, e, lo, e2);
+        two_sum_f(hi, r[a], hi, e);
+        two_sum_f(lo, e, lo, e2);
         lo2 = __fadd_rn(lo2, e2);
     }
     if (!isfinite(hi)) return plain_sum12(r);

@@ -493,7 +493,7 @@ double vm_strain(const double e[6]) {
 
 // Augmented-Lagrangian iterations of one increment (after the predictor): see k_al_local.
 // Returns a status; fills the iteration count, residuals, mean stress and the macro strain increment.
-static_assert(sizeof(FpCtl) <= 512 && sizeof(AlCtl) <= 512, "FpCtl must fit its workspace slot");
+static_assert(sizeof(FpCtl) <= 512 && sizeof(AlCtl) <= 512, "FpCtl and AlCtl share one workspace slot");
 constexpr int kFpBatch = 16;   // iterations queued between host reads of the control block
 const double kZero6[6] = {0, 0, 0, 0, 0, 0};
 constexpr int kAlBatch = 8;    // the same for the augmented Lagrangian, which takes a quarter of the iterations

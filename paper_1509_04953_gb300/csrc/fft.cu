@@ -350,7 +350,8 @@ template <int N, bool INV, typename C> __device__ void bfft_pass2(C *buf, int nl
     __syncthreads();
 }
 
-// In-place transform of nlines padded lines (line l at buf + l*LS). tw: see load_tw. Starts after and ends with a barrier. MAXIT >= ceil(nlines * (N/R1) / blockDim).
+// In-place transform of nlines padded lines (line l at buf + l*LS). tw: see load_tw. Starts after and ends with a
+// barrier. MAXIT >= ceil(nlines * (N/R1) / blockDim).
 template <int N, bool INV, int MAXIT, typename C> __device__ void block_fft(C *buf, int nlines, const C *tw) {
     constexpr int R1 = Shape<N>::R1, R2 = Shape<N>::R2, LS = Shape<N>::LS;
     if constexpr (R2 == 1) {   // a single radix-N pass; every line is owned by one thread
@@ -725,32 +726,32 @@ template <int N, bool INV, typename C, typename St> __device__ void col_pass2(C 
 // warp, which reads the line's values before it writes.
 template <int N, typename C> __device__ __forceinline__ void unpack_rows(C *buf, int nlines) {
     constexpr int LS = Shape<N>::LS, Hx = N / 2 + 1, KU = (Hx + 31) / 32;
-            const int lane = threadIdx.x & 31;
-            const auto h = (decltype(buf->x))0.5;
-            for (int p = threadIdx.x >> 5; p < nlines; p += blockDim.x >> 5) {
-                C *line = buf + p * LS;
-                C a[KU], b[KU];
-    #pragma unroll
-                for (int u = 0; u < KU; ++u) {
-                    const int k = lane + 32 * u;
-                    if (k < Hx) {
-                        const C zk = line[padn<N>(k & (N - 1))];
-                        const C zc = cconj(line[padn<N>((N - k) & (N - 1))]);
-                        a[u] = cmk<C>(h * (zk.x + zc.x), h * (zk.y + zc.y));
-                        b[u] = cmk<C>(h * (zk.y - zc.y), -h * (zk.x - zc.x));   // (zk - zc) / 2i
-                    }
-                }
-                __syncwarp();
-    #pragma unroll
-                for (int u = 0; u < KU; ++u) {
-                    const int k = lane + 32 * u;
-                    if (k < Hx) {
-                        line[k] = a[u];
-                        line[Hx + k] = b[u];
-                    }
-                }
-                __syncwarp();
+    const int lane = threadIdx.x & 31;
+    const auto h = (decltype(buf->x))0.5;
+    for (int p = threadIdx.x >> 5; p < nlines; p += blockDim.x >> 5) {
+        C *line = buf + p * LS;
+        C a[KU], b[KU];
+#pragma unroll
+        for (int u = 0; u < KU; ++u) {
+            const int k = lane + 32 * u;
+            if (k < Hx) {
+                const C zk = line[padn<N>(k & (N - 1))];
+                const C zc = cconj(line[padn<N>((N - k) & (N - 1))]);
+                a[u] = cmk<C>(h * (zk.x + zc.x), h * (zk.y + zc.y));
+                b[u] = cmk<C>(h * (zk.y - zc.y), -h * (zk.x - zc.x));   // (zk - zc) / 2i
             }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < KU; ++u) {
+            const int k = lane + 32 * u;
+            if (k < Hx) {
+                line[k] = a[u];
+                line[Hx + k] = b[u];
+            }
+        }
+        __syncwarp();
+    }
 }
 
 template <typename T, int N>
@@ -974,9 +975,10 @@ k_fft_xy_c2r_cl(const typename CT<T>::type *__restrict__ spec, T *__restrict__ o
     for (int i = t; i < LB * R1; i += X::NT) pass2(i / LB, i % LB);
     if (last && t < R1) pass2(t, LB);
     cl.sync();
-    // x: pass 1 packs rows 2p and 2p+1 (Z[k] = A[k] + i B[k], with A[N-k] = conj A[k] past N/2); column k is in CTA k / LB
-    // Read one by one the folded elements made the pass 472 us. The partner N - k of item j's element r is element R1 - 1 - r of item M1 - j (element R1 - r of itself for j = 0),
-    // so each half-spectrum value is read once and the folded half comes by shuffle.
+    // x: pass 1 packs rows 2p and 2p+1 (Z[k] = A[k] + i B[k], with A[N-k] = conj A[k] past N/2); column k is in CTA
+    // k / LB. The partner N - k of item j's element r is element R1 - 1 - r of item M1 - j (element R1 - r of itself for
+    // j = 0), so each half-spectrum value is read once and the folded half comes by shuffle: 389 us a pass, 472 us with
+    // every folded element read from the CTA that holds it.
     static_assert(M1 == 16 && R1 == 16, "a line's items fill a half-warp");
     const int p = t / M1, j = t % M1, row = (rank * RB + 2 * p) * P, mate = (t & 16) | ((M1 - j) & 15);
     C v[R1], w[R1 / 2];

@@ -538,13 +538,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_chord_res
 // init = 1 is the start of an increment: sigma from the plain implicit update at eps_tr (S instead of
 // Sal, no lam term), then lam = sigma and e_tr = eps_tr. Partial sums per block: |eps_tr - e_tr|^2,
 // |C0 (eps_tr - e_tr)|^2, the six components of lam and the six of sigma.
-// Error-free transformations on FP32 (Knuth's two-sum; the rounding error of a product by fma): an
-// FP32 result plus the float that it rounded away, exactly.
-__device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
+// The error-free product beside two_sum_f: p + e equals a b exactly.
 __device__ __forceinline__ void two_prod_f(float a, float b, float &p, float &e) {
     p = __fmul_rn(a, b);
     e = fmaf(a, b, -p);
@@ -1031,13 +1025,6 @@ __global__ void __launch_bounds__(256) k_predictor(long N3, const TA *__restrict
     for (int c = 0; c < 6; ++c) epst[c * N3 + v] = ee[c] + (use_field ? r * dd[c] : dE[c]);
 }
 
-// Error-free sum of two floats (Knuth's two-sum): s + e equals a + b exactly.
-__device__ __forceinline__ void two_sum_k(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
 // k = sum of the 12 densities as a double. FP64 fields: summed in FP64. FP32 fields: summed as an unevaluated
 // float pair (two-sum per term, the rounding errors added in float) and converted once: the result is within a few
 // units of 2^-48 of the exact sum of the FP32 densities (the FP64 running sum is exact for them too, or nearly),
@@ -1053,7 +1040,7 @@ __device__ __forceinline__ double density_total(const float r[12]) {
 #pragma unroll
     for (int a = 1; a < 12; ++a) {
         float s, e;
-        two_sum_k(hi, r[a], s, e);
+        two_sum_f(hi, r[a], s, e);
         hi = s;
         lo = __fadd_rn(lo, e);
     }
