@@ -152,9 +152,8 @@ typedef struct evp_handle evp_handle;
 #define EVP_F_GRAIN (1u << 8)   /* current grain id (argmax order parameter), 1 x int32 */
 #define EVP_F_G0    (1u << 9)   /* initial grain id (orientation index), 1 x int32 (get only) */
 #define EVP_F_DRAWS (1u << 10)  /* kappa draws so far, 1 x int32 */
-#define EVP_F_IDS   (1u << 11)  /* active-set ids, kmax x int32 per PF point (slot-major, ascending ids; a negative
-                                   id, -1 as written by the library, ends a list: empty
-                                   slots last) */
+#define EVP_F_IDS   (1u << 11)  /* active-set ids, kmax x int32 per PF point (slot-major, ascending ids, -1 = empty
+                                   slots last; in set_fields any negative id ends a list) */
 #define EVP_F_ETA   (1u << 12)  /* active-set order parameters, kmax x T per PF point */
 #define EVP_F_GRAIN_PF (1u << 13)  /* argmax id per PF point, 1 x int32 per PF point (get only; the same as
                                       EVP_F_GRAIN when pf_refine <= 1) */
@@ -250,8 +249,8 @@ int evp_adjoint_end(evp_handle *h, const double *gbar, double *grad, double tol,
  * time is accumulated per kernel class. Classes: 0 newton, 1 fft_xy_r2c, 2 fft_y_fwd,
  * 3 fft_z_gamma, 4 fft_y_inv, 5 fft_xy_c2r_update, 6 reduce, 7 predictor, 8 state_update,
  * 9 nucleate, 10 pf_step, 11 pf_soften, 12 pf_stats. Classes 1 and 5 are the x passes of the forward and
- * inverse transforms; where a (field, z) plane fits one SM's shared memory (FP32 up to n = 128, FP64 up to
- * n = 64, n >= 32) the y pass runs inside them and classes 2 and 4 stay empty. ms and launches hold
+ * inverse transforms; where a (field, z) plane fits one SM's shared memory (n >= 16, FP32 up to n = 128, FP64 up to
+ * n = 64) or a cluster's (FP32 at n = 256) the y pass runs inside them and classes 2 and 4 stay empty. ms and launches hold
  * EVP_NCLASS entries. */
 #define EVP_NCLASS 13
 int evp_set_profiling(evp_handle *h, int on);

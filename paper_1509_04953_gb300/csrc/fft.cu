@@ -1043,8 +1043,8 @@ __device__ __forceinline__ double rcp_pos(double x) {
 // xi = w (f1, f2, f3): eps_kh = (n_h v_k + n_k v_h)/(2 mu0) - c n_k n_h (n.v), v = sigma.n, n = xi/|xi|,
 // |xi.sigma|^2 = |xi|^2 |v|^2. t: the tensor components 11, 22, 33, 23, 13, 12; s: the result (Mandel).
 // FP64 (the FP64 pipe bounds the pass): in terms of xi and one reciprocal, about 95 multiply-adds per frequency where
-// normalising xi takes a square root and a division besides. 64^3 FP64 z pass, with GammaC and the tabulated twiddles:
-// 131 us before, 102 after.
+// normalising xi takes a square root and a division besides. 64^3 FP64 z pass, with GammaC, the tabulated twiddles and
+// the butterflies above: 107 us, 133 without them.
 template <typename C>
 __device__ __forceinline__ double gamma_regular(const C t[6], C s[6], int f1, int f2, int f3, double w,
                                                 const GammaC<double> &gc) {

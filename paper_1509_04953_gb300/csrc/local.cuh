@@ -86,7 +86,7 @@ __device__ __forceinline__ void load_slip_pair(const float *__restrict__ M, int 
 // components and +-1/sqrt12 on two shears (Mandel), so the 12 resolved stresses take 21 additions, the plastic strain
 // another 28 and the tangent 24 before its scaling, where the sample-frame Schmid vectors take 72, 72 and 252
 // multiply-adds. A solve adds three rotations of a symmetric tensor (51 operations each): trial strain and stress in,
-// stress out. k_newton_df at 64^3: 319 us per fixed-point iteration, 501 with the sample-frame vectors.
+// stress out. k_newton_df at 64^3: 373 us per fixed-point iteration, 512 with the sample-frame vectors.
 // The FP32 problems stay in the sample frame: rotating the stress in FP32 adds a rounding of the stress itself, and
 // the equilibrium residual of the converged FP32 field rose from 5.0e-7 to 7.5e-7 of its tolerance's 1e-6.
 // The grain table holds kFrameWords words per grain: R (crystal -> sample, row-major) and a word of padding, which keeps

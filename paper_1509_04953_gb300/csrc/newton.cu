@@ -749,8 +749,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(TA) == 4 ? 3 : 2) k_al_local(
 // the start by al_solve_rest, out of line. Crystal tables and factors are read again at each step, from L1 and shared
 // memory, and the operands of the update after the solve, so 72 registers carry 28 warps per SM (local step per
 // increment at 4 / 5 / 6 / 7 / 8 CTAs of 128 threads: 7.25 / 6.7 / 6.43 / 6.38 / 6.48 ms at 128^3, and 3.79 / 3.49 / 3.53 /
-// 3.35 / 3.36 ms with the Ma-Roters law at 64^3). At 128^3 the step takes 122 us, 545 MB at 4.5 TB/s, where the full solver
-// took 270 (97 of them on the FP64 pipe for the sums, see warp_accumulate14); with Ma-Roters at 64^3 57 us, 83 before.
+// 3.35 / 3.36 ms with the Ma-Roters law at 64^3). Per step after the first, averaged over
+// an increment's iterations (first three, last quarter): 128^3 148 us (182, 128), 545 MB at 3.7 TB/s, where the full
+// solver took 251 (270, 228; 97 of them on the FP64 pipe for the sums, see warp_accumulate14); with Ma-Roters at 64^3
+// 59 us (83, 40), 73 (83, 65) before.
 constexpr int kAlCtas = 7;
 struct AlArgs {
     long N3;
