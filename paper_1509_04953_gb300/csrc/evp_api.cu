@@ -601,10 +601,9 @@ int al_loop(evp_handle *h, MatConst mc, double *dE, int *it_out, int *conv_out, 
     *nmax_out = hc.nmax;
     *err_eq = hc.elam;
     *err_bc = hc.ebc;
-    for (int i = 0; i < 6; ++i) {
-        dE[i] = hc.dE[i];
-        mean_sig[i] = hc.mean[i];
-    }
+    for (int i = 0; i < 6; ++i) dE[i] = hc.dE[i];
+    if (hc.status != EVP_ERR_NEWTON || hc.it > 0)   // nothing to report of a failed initial step
+        for (int i = 0; i < 6; ++i) mean_sig[i] = hc.mean[i];
     if (hc.status == EVP_ERR_NEWTON) return fail(h, EVP_ERR_NEWTON, "local Newton failed in %d voxels", hc.nfail);
     if (hc.status == EVP_ERR_NONFINITE) return fail(h, EVP_ERR_NONFINITE, "non-finite AL residual");
     return EVP_OK;
@@ -986,7 +985,7 @@ int evp_increment(evp_handle *h, double dE33, double dt, evp_stats *out) {
         }
         const double den = std::fmax(std::sqrt(mn), h->p.tau0);
         err_eq = std::sqrt(hs[6]) / ((double)N3 * den);
-        err_bc = std::sqrt(mu_n) / den;
+        err_bc = std::sqrt(std::fmax(mu_n, 0.0)) / den;
         if (hc.status == EVP_ERR_NEWTON)
             status = fail(h, EVP_ERR_NEWTON, "local Newton failed in %d voxels at iteration %d", hc.nfail, it);
         else if (hc.status == EVP_ERR_NONFINITE)

@@ -988,9 +988,11 @@ __global__ void __launch_bounds__(256) k_al_control(AlCtl *c, const double *__re
         c->nfail = nfail;
         c->status = status;
         c->conv = conv;
-        c->ecmp = ecmp;
-        c->elam = elam;
-        c->ebc = ebc;
+        if (!first && nfail == 0) {   // of the last iteration whose local problems were all solved
+            c->ecmp = ecmp;
+            c->elam = elam;
+            c->ebc = ebc;
+        }
         if (!done && !first && p.eta > 0.0) {
             c->tol_loc = fmax(p.ntol, p.eta * fmax(ecmp, elam));
             c->tol_loc_f = (float)c->tol_loc;
